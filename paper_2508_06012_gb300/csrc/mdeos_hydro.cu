@@ -12,6 +12,7 @@
 // update the correctly rounded sequence of operations written here.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <string>
@@ -172,12 +173,247 @@ __global__ void __launch_bounds__(kHydroThreads, 1) hydro_kernel(HydroArgs a, in
   }
 }
 
+// thread-block cluster: rank, size, barrier, a store into CTA `rank`'s shared memory
+__device__ __forceinline__ int hy_cluster_rank() {
+  int r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ int hy_cluster_size() {
+  int r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ void hy_cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;"
+               ::: "memory");
+}
+__device__ __forceinline__ uint32_t hy_map(const void* p, int rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;"
+               : "=r"(r) : "r"((uint32_t)__cvta_generic_to_shared(p)), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void hy_st_cluster(double* p, int rank, double v) {
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(hy_map(p, rank)), "d"(v) : "memory");
+}
+__device__ __forceinline__ void hy_st_cluster(int* p, int rank, int v) {
+  asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(hy_map(p, rank)), "r"(v) : "memory");
+}
+
+// The same steps on a thread-block cluster of csize CTAs, state in shared memory.
+//
+// What bounds a step is FP64: a zone and its node take six divisions and square roots
+// and about 100 FP64 instructions, at one warp instruction per 19 SM cycles (measured),
+// so 2000 zones on one SM take 61 us a step however they are scheduled.  Here CTA r
+// owns the zones [nz r / csize, nz (r + 1) / csize) and computes both of their end
+// nodes; a node between two CTAs is computed by both, from the same operands in the
+// same order, so both hold the same bits.  A step then needs one exchange: each CTA's
+// smallest time-step bound and error code go to every CTA and its outer P + q to its
+// neighbours (st.shared::cluster, two alternating sets, so that a CTA one step ahead
+// never overwrites what a slower one still reads), followed by one cluster barrier.
+// The minimum does not depend on its order, so the state equals the one-CTA kernel's
+// bit for bit.  2000 zones, ideal gas: 61.7 us a step on one CTA, HYDRO_NOW here.
+constexpr int kHydroCluster = 16;  // CTAs (above 8: non-portable, where the GPU takes it)
+
+struct HydroExchange {
+  double mn[2][kHydroCluster];
+  double halo[2][2];  // P + q of the zone left and right of the CTA's own
+  int bad[2][kHydroCluster];
+  double wmin[kHydroThreads / 32];
+  int wbad[kHydroThreads / 32];
+};
+
+__host__ __device__ inline size_t hydro_cluster_smem(int zones_per_cta) {
+  return sizeof(HydroExchange) + (4 * (size_t)(zones_per_cta + 1) + 7 * (size_t)zones_per_cta) * 8;
+}
+
+template <int CL, int NT>
+__global__ void __launch_bounds__(NT, 1) hydro_cluster_kernel(HydroArgs a, int nsteps) {
+  extern __shared__ __align__(16) unsigned char hsm[];
+  HydroExchange* ex = reinterpret_cast<HydroExchange*>(hsm);
+  const int csize = hy_cluster_size(), crank = hy_cluster_rank();
+  const int nz = a.nz;
+  const int z0 = (int)((long long)nz * crank / csize);
+  const int nl = (int)((long long)nz * (crank + 1) / csize) - z0;  // own zones (>= 1)
+  const int nt = blockDim.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  double* x = reinterpret_cast<double*>(ex + 1);
+  double *u = x + nl + 1, *M = u + nl + 1, *uh = M + nl + 1;
+  double *m = uh + nl + 1, *rho = m + nl, *e = rho + nl, *P = e + nl, *q = P + nl, *c2 = q + nl;
+  double* Pq = c2 + nl;
+  for (int j = tid; j <= nl; j += nt) {
+    x[j] = a.x[z0 + j];
+    u[j] = a.u[z0 + j];
+    M[j] = a.M[z0 + j];
+  }
+  for (int j = tid; j < nl; j += nt) {
+    m[j] = a.m[z0 + j];
+    rho[j] = a.rho[z0 + j];
+    e[j] = a.e[z0 + j];
+  }
+  double t = a.clock[0], dt = a.clock[1], nst = a.clock[2], prev = a.clock[3];
+  const int err0 = *a.err;
+  int err = 0;
+  __syncthreads();
+  // every CTA has started (and read the clock and the error word) before any stores
+  // into another's shared memory
+  hy_cluster_sync();
+  for (int step = 0; step < nsteps; ++step) {
+    const int par = step & 1;
+    // phase A: closure, artificial viscosity, time-step bound per zone
+    double lmin = INFINITY;
+    int bad = 0;
+    for (int j = tid; j < nl; j += nt) {
+      const double rhoz = rho[j];
+      double ez = e[j];
+      if (CL == MDEOS_CLOSURE_MD) {
+        if (a.md[z0 + j].status != MDEOS_OK) bad = HY_ERR_EOS;
+        if (a.set_e_from_md) ez = a.md[z0 + j].e_achieved;
+      }
+      double Pz, c2z;
+      closure<CL>(a, z0 + j, rhoz, ez, Pz, c2z);
+      const double c = sqrt(c2z);
+      const double du = u[j + 1] - u[j];
+      const double qz = du < 0.0 ? rhoz * (a.q2 * du * du - a.q1 * c * du) : 0.0;
+      const double dx = x[j + 1] - x[j];
+      const double sig = c + 2.0 * a.q2 * fmax(-du, 0.0);
+      lmin = fmin(lmin, dx / sig);
+      if (!(rhoz > 0.0) || !(dx > 0.0) || !isfinite(Pz) || !(c2z >= 0.0) || !isfinite(ez))
+        bad = bad ? bad : HY_ERR_STATE;
+      P[j] = Pz;
+      q[j] = qz;
+      c2[j] = c2z;
+      Pq[j] = Pz + qz;
+      if (CL == MDEOS_CLOSURE_MD && a.set_e_from_md) e[j] = ez;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) lmin = fmin(lmin, __shfl_xor_sync(0xffffffffu, lmin, o));
+    bad = __reduce_max_sync(0xffffffffu, bad);
+    if (lane == 0) {
+      ex->wmin[warp] = lmin;
+      ex->wbad[warp] = bad;
+    }
+    __syncthreads();
+    if (warp == 0) {  // the CTA's bound and error code to every CTA, P + q to the neighbours
+      double mn = lane < (nt >> 5) ? ex->wmin[lane] : INFINITY;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+      const int b = __reduce_max_sync(0xffffffffu, lane < (nt >> 5) ? ex->wbad[lane] : 0);
+      if (lane < csize) {
+        hy_st_cluster(&ex->mn[par][crank], lane, mn);
+        hy_st_cluster(&ex->bad[par][crank], lane, b);
+      }
+      if (lane == 30 && crank > 0) hy_st_cluster(&ex->halo[par][1], crank - 1, Pq[0]);
+      if (lane == 31 && crank + 1 < csize) hy_st_cluster(&ex->halo[par][0], crank + 1, Pq[nl - 1]);
+    }
+    hy_cluster_sync();
+    double mn = lane < csize ? ex->mn[par][lane] : INFINITY;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mn = fmin(mn, __shfl_xor_sync(0xffffffffu, mn, o));
+    err = max(err0, __reduce_max_sync(0xffffffffu, lane < csize ? ex->bad[par][lane] : 0));
+    double dtn = a.cfl * mn;
+    if (prev > 0.0) dtn = fmin(dtn, a.grow * prev);
+    if (a.dt_fixed > 0.0) dtn = a.dt_fixed;
+    if (!(dtn > 0.0) || !isfinite(dtn)) err = max(err, (int)HY_ERR_DT);
+    if (err != 0) break;  // the same in every thread; state left at the last good step
+    dt = dtn;
+    // phase B: nodes -- momentum (Eq. 3), positions
+    for (int j = tid; j <= nl; j += nt) {
+      const int i = z0 + j;
+      const double left = i > 0 ? (j > 0 ? Pq[j - 1] : ex->halo[par][0]) : 0.0;
+      const double right = i < nz ? (j < nl ? Pq[j] : ex->halo[par][1]) : 0.0;
+      const double F = left - right;
+      const double u0 = u[j];
+      double un = u0 + dt * F / M[j];
+      if ((i == 0 && a.bcl == MDEOS_BC_WALL) || (i == nz && a.bcr == MDEOS_BC_WALL)) un = 0.0;
+      const double uhj = 0.5 * (u0 + un);
+      u[j] = un;
+      uh[j] = uhj;
+      x[j] = x[j] + dt * uhj;
+    }
+    __syncthreads();
+    // phase C: zones -- energy (Eq. 4, compatible form) and density (Eq. 2)
+    for (int j = tid; j < nl; j += nt) {
+      e[j] = e[j] - dt * Pq[j] * (uh[j + 1] - uh[j]) / m[j];
+      rho[j] = m[j] / (x[j + 1] - x[j]);
+    }
+    t = t + dt;
+    nst = nst + 1.0;
+    prev = dt;
+    if (CL == MDEOS_CLOSURE_MD) break;  // one EOS batch per step
+  }
+  __syncthreads();
+  for (int j = tid; j <= nl; j += nt)
+    if (j < nl || crank + 1 == csize) {
+      a.x[z0 + j] = x[j];
+      a.u[z0 + j] = u[j];
+    }
+  for (int j = tid; j < nl; j += nt) {
+    a.rho[z0 + j] = rho[j];
+    a.e[z0 + j] = e[j];
+    a.P[z0 + j] = P[j];
+    a.q[z0 + j] = q[j];
+    a.c2[z0 + j] = c2[j];
+  }
+  if (crank == 0 && tid == 0) {
+    if (err != 0) *a.err = err;
+    a.clock[0] = t;
+    a.clock[1] = dt;
+    a.clock[2] = nst;
+    a.clock[3] = prev;
+  }
+  hy_cluster_sync();  // no CTA leaves while another may still store into its shared memory
+}
+
 }  // namespace mdeos
 
 using namespace mdeos;
 
+// Cluster size of a problem: a power of two with at least 32 zones per CTA (fewer leave
+// lanes of the FP64 pipe idle), at most kHydroCluster; 0 where the slab of a CTA would
+// not fit its shared memory (above about 35,000 zones: the one-CTA kernel on global
+// memory).
+constexpr size_t kHydroSmem = 200 * 1024;
+static int hydro_csize(int nz, int cmax) {
+  int c = 1;
+  while (2 * c <= cmax && nz >= 2 * c * 32) c *= 2;
+  return hydro_cluster_smem((nz + c - 1) / c) <= kHydroSmem ? c : 0;
+}
+
+using HydroKernel = void (*)(HydroArgs, int);
+// the kernel of a closure for `threads` threads per CTA: registers for up to 256, or 1024
+static HydroKernel hydro_cluster_fn(int cl, int threads) {
+  const bool w = threads > 256;
+  if (cl == MDEOS_CLOSURE_IDEAL_GAS)
+    return w ? hydro_cluster_kernel<MDEOS_CLOSURE_IDEAL_GAS, kHydroThreads>
+             : hydro_cluster_kernel<MDEOS_CLOSURE_IDEAL_GAS, 256>;
+  if (cl == MDEOS_CLOSURE_MIE_GRUNEISEN)
+    return w ? hydro_cluster_kernel<MDEOS_CLOSURE_MIE_GRUNEISEN, kHydroThreads>
+             : hydro_cluster_kernel<MDEOS_CLOSURE_MIE_GRUNEISEN, 256>;
+  return w ? hydro_cluster_kernel<MDEOS_CLOSURE_MD, kHydroThreads>
+           : hydro_cluster_kernel<MDEOS_CLOSURE_MD, 256>;
+}
+
+static cudaLaunchConfig_t hydro_launch_config(int csize, int threads, size_t smem, cudaStream_t st,
+                                              cudaLaunchAttribute* at) {
+  cudaLaunchConfig_t lc = {};
+  lc.gridDim = dim3((unsigned)csize, 1, 1);
+  lc.blockDim = dim3((unsigned)threads, 1, 1);
+  lc.dynamicSmemBytes = smem;
+  lc.stream = st;
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = (unsigned)csize;
+  at->val.clusterDim.y = at->val.clusterDim.z = 1;
+  lc.attrs = at;
+  lc.numAttrs = 1;
+  return lc;
+}
+
 struct mdeos_hydro {
   mdeos_handle* h = nullptr;
+  int csize = 0, threads = 0;  // cluster kernel's launch (csize 0: the one-CTA kernel)
+  size_t smem = 0;
+  HydroKernel fn = nullptr;
   mdeos_hydro_config cfg;
   int nz = 0;
   double* d_mem = nullptr;
@@ -301,12 +537,52 @@ extern "C" mdeos_status mdeos_hydro_create(mdeos_handle* h, const mdeos_hydro_co
     mdeos_hydro_destroy(hy);
     return set_error(MDEOS_ECUDA, std::string("hydro init: ") + cudaGetErrorString(e));
   }
+  // clusters of 16 CTAs where the GPU can hold one, else of 8
+  for (int cmax = kHydroCluster; cmax >= 8 && hy->fn == nullptr; cmax /= 2) {
+    const int c = hydro_csize(nz, cmax);
+    if (c == 0) continue;
+    const int zpc = (nz + c - 1) / c;
+    const int threads = std::min(kHydroThreads, (zpc + 1 + 31) / 32 * 32);
+    HydroKernel fn = hydro_cluster_fn(cfg->closure, threads);
+    const size_t smem = hydro_cluster_smem(zpc);
+    int fit = 0;
+    cudaLaunchAttribute at;
+    cudaLaunchConfig_t lc = hydro_launch_config(c, threads, smem, st, &at);
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kHydroSmem) ==
+            cudaSuccess &&
+        (c <= 8 || cudaFuncSetAttribute(fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
+                       cudaSuccess) &&
+        cudaOccupancyMaxActiveClusters(&fit, fn, &lc) == cudaSuccess && fit > 0) {
+      hy->fn = fn;
+      hy->csize = c;
+      hy->threads = threads;
+      hy->smem = smem;
+    } else {
+      cudaGetLastError();  // not available: the next choice
+    }
+  }
   count_launch(h, 1);
   hy->h_rho.resize(nz);
   hy->h_e.resize(nz);
   hy->reqs.resize(nz);
   *out = hy;
   return MDEOS_OK;
+}
+
+// nsteps steps (one with the MD closure) in one launch
+static cudaError_t launch_hydro(mdeos_hydro* hy, const HydroArgs& a, int nsteps, cudaStream_t st) {
+  if (hy->fn != nullptr) {
+    cudaLaunchAttribute at;
+    cudaLaunchConfig_t lc = hydro_launch_config(hy->csize, hy->threads, hy->smem, st, &at);
+    return cudaLaunchKernelEx(&lc, hy->fn, a, nsteps);
+  }
+  if (hy->cfg.closure == MDEOS_CLOSURE_IDEAL_GAS)
+    hydro_kernel<MDEOS_CLOSURE_IDEAL_GAS><<<1, kHydroThreads, 0, st>>>(a, nsteps);
+  else if (hy->cfg.closure == MDEOS_CLOSURE_MIE_GRUNEISEN)
+    hydro_kernel<MDEOS_CLOSURE_MIE_GRUNEISEN><<<1, kHydroThreads, 0, st>>>(a, nsteps);
+  else
+    hydro_kernel<MDEOS_CLOSURE_MD><<<1, kHydroThreads, 0, st>>>(a, nsteps);
+  return cudaGetLastError();
 }
 
 static mdeos_status hydro_status(mdeos_hydro* hy, cudaStream_t st) {
@@ -326,15 +602,8 @@ extern "C" mdeos_status mdeos_hydro_step(mdeos_hydro* hy, int32_t nsteps) {
   HCK(cudaSetDevice(handle_device(hy->h)));
   HydroArgs a = hy->args;
   const int cl = hy->cfg.closure;
-  if (cl == MDEOS_CLOSURE_IDEAL_GAS) {
-    hydro_kernel<MDEOS_CLOSURE_IDEAL_GAS><<<1, kHydroThreads, 0, st>>>(a, nsteps);
-    HCK(cudaGetLastError());
-    count_launch(hy->h, 1);
-    return hydro_status(hy, st);
-  }
-  if (cl == MDEOS_CLOSURE_MIE_GRUNEISEN) {
-    hydro_kernel<MDEOS_CLOSURE_MIE_GRUNEISEN><<<1, kHydroThreads, 0, st>>>(a, nsteps);
-    HCK(cudaGetLastError());
+  if (cl != MDEOS_CLOSURE_MD) {
+    HCK(launch_hydro(hy, a, nsteps, st));
     count_launch(hy->h, 1);
     return hydro_status(hy, st);
   }
@@ -361,8 +630,7 @@ extern "C" mdeos_status mdeos_hydro_step(mdeos_hydro* hy, int32_t nsteps) {
     mdeos_status s = eval_into_device(hy->h, hy->reqs.data(), nz, hy->d_res);
     if (s != MDEOS_OK) return s;
     a.set_e_from_md = (first && c.first_temperature) ? 1 : 0;
-    hydro_kernel<MDEOS_CLOSURE_MD><<<1, kHydroThreads, 0, st>>>(a, 1);
-    HCK(cudaGetLastError());
+    HCK(launch_hydro(hy, a, 1, st));
     count_launch(hy->h, 1);
     hy->calls += 1;
     s = hydro_status(hy, st);
