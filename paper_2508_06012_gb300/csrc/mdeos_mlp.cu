@@ -46,6 +46,10 @@ struct GemmArgs {
   // (dense), summed in the order s = 0, 1, ... by gemm_splitk_reduce
   int S, kchunk;
   float* ws;
+  // a second batch of products of the same shape, z >= z2 of Z in all (z2 = Z: none)
+  const __nv_bfloat16 *A2, *B2;
+  float* C2;
+  int z2, Z;
 };
 
 // ---------------------------------------------------------------------------
@@ -73,7 +77,8 @@ __device__ __forceinline__ float tanh_act(float x) {
 
 // refresh the bf16 weight copies from the FP32 master parameters
 __global__ void mlp_cast_weights(const float* P, __nv_bfloat16* W1b, __nv_bfloat16* W2b,
-                                 __nv_bfloat16* W3b, __nv_bfloat16* W4b, int E) {
+                                 __nv_bfloat16* W3b, __nv_bfloat16* W4b, __nv_bfloat16* W2t,
+                                 __nv_bfloat16* W3t, int E) {
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
   const long long n = (long long)E * kH * kH;
   if (i >= n) return;
@@ -81,6 +86,9 @@ __global__ void mlp_cast_weights(const float* P, __nv_bfloat16* W1b, __nv_bfloat
   const float* p = P + (long long)e * kNParam;
   W2b[i] = __float2bfloat16_rn(p[kOffW2 + r]);
   W3b[i] = __float2bfloat16_rn(p[kOffW3 + r]);
+  const long long t = (long long)e * kH * kH + (r % kH) * kH + r / kH;  // transposed
+  W2t[t] = W2b[i];
+  W3t[t] = W3b[i];
   if (r < 2 * kH) {
     W1b[(long long)e * 2 * kH + r] = __float2bfloat16_rn(p[kOffW1 + r]);
     W4b[(long long)e * 2 * kH + r] = __float2bfloat16_rn(p[kOffW4 + r]);
@@ -108,119 +116,154 @@ __global__ void mlp_bias_tanh(const float* Z, const float* P, int off_b, __nv_bf
   Hout[i] = __float2bfloat16_rn(tanh_act(Z[i] + P[(long long)e * kNParam + off_b + j]));
 }
 
-// y = W4 h3 + b4 (FP32 accumulation); with targets: dy = 2 (y - t) / (2 B) and the
-// squared-error sum (one atomic per block)
+// y = W4 h3 + b4 (FP32 accumulation)
 __global__ void mlp_output(const __nv_bfloat16* H3, const float* P, const __nv_bfloat16* W4b,
-                           const float* T, float* Y, float* dY, float* loss, int B, int E) {
-  __shared__ float s_l[8];
+                           float* Y, int B, int E) {
   const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  float l = 0.f;
-  if (i < (long long)E * B * 2) {
-    const int o = (int)(i % 2), b = (int)((i / 2) % B), e = (int)(i / (2LL * B));
-    const __nv_bfloat16* h = H3 + ((long long)e * B + b) * kH;
-    const __nv_bfloat16* w = W4b + (long long)e * 2 * kH + o * kH;
-    float y = 0.f;
-    for (int j = 0; j < kH; ++j) y = fmaf(__bfloat162float(w[j]), __bfloat162float(h[j]), y);
-    y += P[(long long)e * kNParam + kOffB4 + o];
-    Y[i] = y;
-    if (T) {
-      const float d = y - T[2 * b + o];
-      dY[i] = d / (float)B;  // 2 (y - t) / (2 B)
-      l = d * d;
+  if (i >= (long long)E * B * 2) return;
+  const int o = (int)(i % 2), b = (int)((i / 2) % B), e = (int)(i / (2LL * B));
+  const __nv_bfloat16* h = H3 + ((long long)e * B + b) * kH;
+  const __nv_bfloat16* w = W4b + (long long)e * 2 * kH + o * kH;
+  float y = 0.f;
+  for (int j = 0; j < kH; ++j) y = fmaf(__bfloat162float(w[j]), __bfloat162float(h[j]), y);
+  Y[i] = y + P[(long long)e * kNParam + kOffB4 + o];
+}
+
+// Gradients that are sums over the batch alone: dW4, db4 (from dy, h3), db3, db2, db1
+// (columns of dz3, dz2, dz1) and dW1 (dz1, x).  Each is one FP32 sum over b = 0, 1, ...
+// in order, a chain of B dependent additions (1 us at B = 512); with the loads in the
+// chain it took 40 us per kernel, five kernels, and 33 us in one kernel with each warp
+// loading its own rows.  Here a CTA (32 columns of one model) copies kColRows rows of all
+// operands into shared memory with cp.async, two stages in turn, and each warp walks its
+// sum through them.
+constexpr int kColRows = 128;
+struct ColStage {
+  __nv_bfloat16 h3[kColRows][32], dz3[kColRows][32], dz2[kColRows][32];
+  float dz1[kColRows][32], dy[kColRows][2], x[kColRows][2];
+};
+constexpr int kColSmem = 2 * (int)sizeof(ColStage);
+
+template <int BYTES>
+__device__ __forceinline__ void cp_async(void* dst, const void* src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], %2;"
+               ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "n"(BYTES) : "memory");
+}
+
+__global__ void __launch_bounds__(256) mlp_column_grads(const float* dY, const __nv_bfloat16* H3,
+                                                        const __nv_bfloat16* dZ3,
+                                                        const __nv_bfloat16* dZ2, const float* dZ1,
+                                                        const float* X, float* G, int B) {
+  extern __shared__ __align__(16) unsigned char csm[];
+  ColStage* st = reinterpret_cast<ColStage*>(csm);
+  const int e = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int j0 = blockIdx.x * 32, j = j0 + lane;
+  float* g = G + (long long)e * kNParam;
+  const long long r0 = (long long)e * B;  // the model's first row
+  auto load = [&](int stage, int b0) {    // rows b0 .. of the batch, at most kColRows
+    ColStage& s = st[stage];
+    const int rows = min(kColRows, B - b0);
+    for (int q = tid; q < rows * 4; q += 256) {  // bf16 rows: four 16-byte pieces
+      const int r = q >> 2, c = (q & 3) * 8;
+      const long long at = (r0 + b0 + r) * kH + j0 + c;
+      cp_async<16>(&s.h3[r][c], H3 + at);
+      cp_async<16>(&s.dz3[r][c], dZ3 + at);
+      cp_async<16>(&s.dz2[r][c], dZ2 + at);
     }
-  }
-  if (T) {
-    for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-    if ((threadIdx.x & 31) == 0) s_l[threadIdx.x >> 5] = l;
+    for (int q = tid; q < rows * 8; q += 256)
+      cp_async<16>(&s.dz1[q >> 3][(q & 7) * 4], dZ1 + (r0 + b0 + (q >> 3)) * kH + j0 + (q & 7) * 4);
+    for (int q = tid; q < rows; q += 256) {
+      cp_async<8>(s.dy[q], dY + (r0 + b0 + q) * 2);
+      cp_async<8>(s.x[q], X + (long long)(b0 + q) * 2);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  };
+  float sum = 0.f;
+  load(0, 0);
+  for (int b0 = 0, k = 0; b0 < B; b0 += kColRows, k ^= 1) {
+    if (b0 + kColRows < B) {
+      load(k ^ 1, b0 + kColRows);
+      asm volatile("cp.async.wait_group 1;" ::: "memory");
+    } else {
+      asm volatile("cp.async.wait_group 0;" ::: "memory");
+    }
     __syncthreads();
-    if (threadIdx.x == 0) {
-      float s = 0.f;
-      for (int w = 0; w < (int)(blockDim.x >> 5); ++w) s += s_l[w];
-      atomicAdd(loss, s);
+    const ColStage& s = st[k];
+    const int rows = min(kColRows, B - b0);
+    if (warp < 2) {  // dW4
+#pragma unroll 16
+      for (int r = 0; r < rows; ++r) sum = fmaf(s.dy[r][warp], __bfloat162float(s.h3[r][lane]), sum);
+    } else if (warp < 4) {  // dW1
+#pragma unroll 16
+      for (int r = 0; r < rows; ++r) sum = fmaf(s.dz1[r][lane], s.x[r][warp - 2], sum);
+    } else if (warp == 4) {
+#pragma unroll 16
+      for (int r = 0; r < rows; ++r) sum += __bfloat162float(s.dz3[r][lane]);
+    } else if (warp == 5) {
+#pragma unroll 16
+      for (int r = 0; r < rows; ++r) sum += __bfloat162float(s.dz2[r][lane]);
+    } else if (warp == 6) {
+#pragma unroll 16
+      for (int r = 0; r < rows; ++r) sum += s.dz1[r][lane];
+    } else {
+#pragma unroll 16
+      for (int r = 0; r < rows; ++r) sum += s.dy[r][lane & 1];
     }
+    __syncthreads();  // the stage is filled again two turns on
   }
-}
-
-// output layer backward: dW4, db4 (reductions over the batch, one thread per weight)
-__global__ void mlp_back_out_w(const float* dY, const __nv_bfloat16* H3, float* G, int B, int E) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= E * (2 * kH + 2)) return;
-  const int e = i / (2 * kH + 2), r = i % (2 * kH + 2);
-  float s = 0.f;
-  if (r < 2 * kH) {
-    const int o = r / kH, j = r % kH;
-    for (int b = 0; b < B; ++b)
-      s = fmaf(dY[((long long)e * B + b) * 2 + o],
-               __bfloat162float(H3[((long long)e * B + b) * kH + j]), s);
-    G[(long long)e * kNParam + kOffW4 + r] = s;
-  } else {
-    const int o = r - 2 * kH;
-    for (int b = 0; b < B; ++b) s += dY[((long long)e * B + b) * 2 + o];
-    G[(long long)e * kNParam + kOffB4 + o] = s;
-  }
-}
-
-// dz3 = bf16((dy W4) * (1 - h3^2))
-__global__ void mlp_back_out_dz(const float* dY, const __nv_bfloat16* H3, const __nv_bfloat16* W4b,
-                                __nv_bfloat16* dZ3, int B, int E) {
-  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i >= (long long)E * B * kH) return;
-  const int j = (int)(i % kH), b = (int)((i / kH) % B), e = (int)(i / ((long long)B * kH));
-  const float* dy = dY + ((long long)e * B + b) * 2;
-  const __nv_bfloat16* w = W4b + (long long)e * 2 * kH;
-  const float dh = dy[0] * __bfloat162float(w[j]) + dy[1] * __bfloat162float(w[kH + j]);
-  const float h = __bfloat162float(H3[i]);
-  dZ3[i] = __float2bfloat16_rn(dh * (1.f - h * h));
-}
-
-// dz = dH (1 - h^2), rounded to bf16 (layer 2) or kept FP32 (layer 1)
-__global__ void mlp_deriv(const float* dH, const __nv_bfloat16* Hh, __nv_bfloat16* dZb, float* dZf,
-                          long long n) {
-  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float h = __bfloat162float(Hh[i]);
-  const float d = dH[i] * (1.f - h * h);
-  if (dZb) dZb[i] = __float2bfloat16_rn(d);
-  if (dZf) dZf[i] = d;
-}
-
-// bias gradient: column sums of dz over the batch
-__global__ void mlp_bias_grad(const __nv_bfloat16* dZb, const float* dZf, float* G, int off_b,
-                              int B, int E) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= E * kH) return;
-  const int e = i / kH, j = i % kH;
-  float s = 0.f;
-  for (int b = 0; b < B; ++b) {
-    const long long k = ((long long)e * B + b) * kH + j;
-    s += dZb ? __bfloat162float(dZb[k]) : dZf[k];
-  }
-  G[(long long)e * kNParam + off_b + j] = s;
-}
-
-// first-layer weight gradient dW1 = dz1^T x (FP32)
-__global__ void mlp_grad_w1(const float* dZ1, const float* X, float* G, int B, int E) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= E * 2 * kH) return;
-  const int e = i / (2 * kH), r = i % (2 * kH), j = r / 2, c = r % 2;
-  float s = 0.f;
-  for (int b = 0; b < B; ++b) s = fmaf(dZ1[((long long)e * B + b) * kH + j], X[2 * b + c], s);
-  G[(long long)e * kNParam + kOffW1 + r] = s;
+  if (warp < 2)
+    g[kOffW4 + warp * kH + j] = sum;
+  else if (warp < 4)
+    g[kOffW1 + 2 * j + warp - 2] = sum;
+  else if (warp < 7)
+    g[(warp == 4 ? kOffB3 : warp == 5 ? kOffB2 : kOffB1) + j] = sum;
+  else if (blockIdx.x == 0 && lane < 2)
+    g[kOffB4 + lane] = sum;
 }
 
 // Adam (Kingma & Ba) on the FP32 master parameters; omb = 1 - beta and c = 1 - beta^t,
-// each evaluated in FP64 on the host and rounded once
-__global__ void mlp_adam(float* P, const float* G, float* Mm, float* Vv, long long n, float lr,
-                         float b1, float b2, float omb1, float omb2, float eps, float c1,
-                         float c2) {
-  const long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const float g = G[i];
-  const float m = b1 * Mm[i] + omb1 * g;
-  const float v = b2 * Vv[i] + omb2 * g * g;
-  Mm[i] = m;
-  Vv[i] = v;
-  P[i] -= lr * (m / c1) / (sqrtf(v / c2) + eps);
+// each evaluated in FP64 on the host and rounded once.  The 128 x 128 weight gradients
+// come as S partial tiles per model (ws[s][which][e][m][n], which 0: W3, 1: W2), added in
+// the order s = 0, 1, ...; the bf16 copies (W2 and W3 also transposed, for the products
+// with dZ) are refreshed with the parameter.
+struct AdamArgs {
+  float *P, *Mm, *Vv;
+  const float *G, *ws;
+  __nv_bfloat16 *W1b, *W2b, *W3b, *W4b, *W2t, *W3t;
+  int E, S;
+  float lr, b1, b2, omb1, omb2, eps, c1, c2;
+};
+
+__global__ void mlp_adam(AdamArgs a) {
+  const int r = blockIdx.x * blockDim.x + threadIdx.x, e = blockIdx.y;
+  if (r >= kNParam) return;
+  const long long i = (long long)e * kNParam + r;
+  const bool w2 = r >= kOffW2 && r < kOffB2, w3 = r >= kOffW3 && r < kOffB3;
+  float g;
+  if ((w2 || w3) && a.S > 1) {
+    const long long part = 2LL * a.E * kH * kH;
+    const float* p = a.ws + ((long long)(w2 ? a.E : 0) + e) * kH * kH + (r - (w2 ? kOffW2 : kOffW3));
+    g = p[0];
+    for (int s = 1; s < a.S; ++s) g += p[s * part];
+  } else {
+    g = a.G[i];
+  }
+  const float m = a.b1 * a.Mm[i] + a.omb1 * g;
+  const float v = a.b2 * a.Vv[i] + a.omb2 * g * g;
+  a.Mm[i] = m;
+  a.Vv[i] = v;
+  const float p = a.P[i] - a.lr * (m / a.c1) / (sqrtf(v / a.c2) + a.eps);
+  a.P[i] = p;
+  const __nv_bfloat16 pb = __float2bfloat16_rn(p);
+  if (w2 || w3) {
+    const int q = r - (w2 ? kOffW2 : kOffW3);
+    const long long at = (long long)e * kH * kH;
+    (w2 ? a.W2b : a.W3b)[at + q] = pb;
+    (w2 ? a.W2t : a.W3t)[at + (q % kH) * kH + q / kH] = pb;
+  } else if (r < kOffB1) {
+    a.W1b[(long long)e * 2 * kH + r] = pb;
+  } else if (r >= kOffW4 && r < kOffB4) {
+    a.W4b[(long long)e * 2 * kH + r - kOffW4] = pb;
+  }
 }
 
 // normalise physical inputs (rho, e) -> x, per sample
@@ -491,6 +534,231 @@ __global__ void __launch_bounds__(kTcThreads) mlp_infer_tc_kernel(const float* X
 }
 
 // ---------------------------------------------------------------------------
+// Forward and backward pass of a training batch in one launch: grid (tiles of 128
+// samples, models), the tiles, descriptors and thread roles of mlp_infer_tc_kernel.
+// The four 128 x 128 weight operands (W2, W3 and their transposes, 32 KB each) are staged
+// once; tile A holds h1, h2, h3, dz3 and dz2 in turn, each the operand of the next
+// product:
+//   Z2 = h1 W2^T, Z3 = h2 W3^T, y and dy from h3, dz3 = (dy W4)(1 - h3^2),
+//   dh2 = dz3 W3, dz2 = dh2 (1 - h2^2), dh1 = dz2 W2, dz1 = dh1 (1 - h1^2).
+// h1..h3, dz3, dz2 (bf16), dz1 and dy (FP32) go to device memory for the sums over the
+// batch.  One launch instead of fourteen, and no FP32 pre-activations in memory: the step
+// was bound by launches and by one-warp sums, not by its products (batch 512, 4 models:
+// a step of an epoch took 328 us, host included, and takes 70 now).  Products accumulate K in the same order of
+// tcgen05.mma steps as bf16_gemm_tc_kernel's chunks, and every element is rounded where
+// the layered form rounds it.
+constexpr int kTrThreads = 512;  // four threads per row (column quarters)
+constexpr int kTrCols = kTrThreads == 512 ? kH / 4 : kH / 2;
+constexpr int kTrSmem = 5 * kTcTile + 1024 + 64 + kTcSmall * 4 + kTcRows * 2 * 4;
+
+struct TrainArgs {
+  const float *X, *T, *P;
+  const __nv_bfloat16 *W1b, *W2b, *W3b, *W4b, *W2t, *W3t;
+  __nv_bfloat16 *H1, *H2, *H3, *dZ3, *dZ2;
+  float *dZ1, *dY, *loss;
+  int B;
+  int* err;
+};
+
+__global__ void __launch_bounds__(kTrThreads) mlp_train_tc_kernel(TrainArgs a) {
+  extern __shared__ __align__(1024) unsigned char tsm[];
+  const uint32_t sbase = ((uint32_t)__cvta_generic_to_shared(tsm) + 1023u) & ~1023u;
+  unsigned char* gbase = tsm + (sbase - (uint32_t)__cvta_generic_to_shared(tsm));
+  const uint32_t sA = sbase, sMbar = sbase + 5 * kTcTile, sTmem = sMbar + 8;
+  unsigned char* gA = gbase;
+  const int e = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int m = tid & (kTcRows - 1), quarter = tid >> 7, c_lo = quarter * kTrCols;
+  const int B = a.B, b = blockIdx.x * kTcRows + m;
+  const bool on = b < B;
+  const long long row = ((long long)e * B + b) * kH;  // this sample's row of the model's arrays
+  const float* p = a.P + (long long)e * kNParam;
+  float* sp = reinterpret_cast<float*>(gbase + 5 * kTcTile + 64);  // small parameters
+  float* sdy = sp + kTcSmall;                                       // dy, then squared errors
+  for (int k = tid; k < 2 * kH; k += kTrThreads) {
+    sp[kTcSW1 + k] = __bfloat162float(a.W1b[(long long)e * 2 * kH + k]);
+    sp[kTcSW4 + k] = __bfloat162float(a.W4b[(long long)e * 2 * kH + k]);
+  }
+  for (int k = tid; k < kH; k += kTrThreads) {
+    sp[kTcSB1 + k] = p[kOffB1 + k];
+    sp[kTcSB2 + k] = p[kOffB2 + k];
+    sp[kTcSB3 + k] = p[kOffB3 + k];
+  }
+  if (tid < 2) sp[kTcSB4 + tid] = p[kOffB4 + tid];
+  {  // the four operands, 16 bytes at a time into the canonical layout
+    const __nv_bfloat16* w[4] = {a.W2b, a.W3b, a.W3t, a.W2t};
+    for (int q = tid; q < kH * kH / 8; q += kTrThreads) {
+      const int n = (q >> 7) * 8 + (q & 7), k = ((q >> 3) & 15) * 8;
+#pragma unroll
+      for (int t = 0; t < 4; ++t)
+        *reinterpret_cast<uint4*>(gbase + (t + 1) * kTcTile + tc_off(n, k)) =
+            *reinterpret_cast<const uint4*>(w[t] + (long long)e * kH * kH + n * kH + k);
+    }
+  }
+  if (tid == 0) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sMbar) : "memory");
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 0) {  // 128 TMEM columns: the 128 x 128 fp32 accumulator
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
+                 ::"r"(sTmem), "r"(kH) : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+  const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(gbase + 5 * kTcTile + 8);
+  const uint32_t tq = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c_lo;
+  // layer 1 on the CUDA cores: this row's units c_lo .. c_lo + 31
+  const float x0 = on ? a.X[2 * b] : 0.f, x1 = on ? a.X[2 * b + 1] : 0.f;
+#pragma unroll 1
+  for (int c = c_lo; c < c_lo + kTrCols; c += 8) {
+    float z[8];
+#pragma unroll
+    for (int j = 0; j < 8; ++j) {
+      const float2 w = *reinterpret_cast<const float2*>(sp + kTcSW1 + 2 * (c + j));
+      z[j] = x0 * w.x + x1 * w.y;
+    }
+    const uint4 pk = tanh_pack8(z, sp + kTcSB1 + c);
+    *reinterpret_cast<uint4*>(gA + tc_off(m, c)) = pk;
+    if (on) *reinterpret_cast<uint4*>(a.H1 + row + c) = pk;
+  }
+  bool ok = true;
+  int layer = 0;
+  // four products, W2, W3, W3 transposed, W2 transposed, each with tile A as it then is
+#pragma unroll 1
+  for (; layer < 4; ++layer) {
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // tile A -> tensor core
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (tid == 0) {
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t sW = sbase + (uint32_t)(layer + 1) * kTcTile;
+#pragma unroll
+      for (int ks = 0; ks < kH / 16; ++ks)  // K step of 16 = two core matrices along K
+        tc_mma(tmem, tc_desc(sA + ks * 2 * kLbo), tc_desc(sW + ks * 2 * kLbo), ks > 0);
+      tc_commit(sMbar);
+    }
+    __syncwarp();
+    const bool done = mbar_wait(sMbar, (uint32_t)layer & 1u);
+    ok = __syncthreads_and(done) != 0;  // the same decision in every thread
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (!ok) break;
+    if (layer < 2) {  // h = bf16(tanh(z + b)) of this row's 32 units
+      const float* bias = sp + (layer == 0 ? kTcSB2 : kTcSB3) + c_lo;
+      __nv_bfloat16* H = (layer == 0 ? a.H2 : a.H3) + row + c_lo;
+#pragma unroll 1
+      for (int c0 = 0; c0 < kTrCols; c0 += 32) {
+        float v[32];
+        tc_ld32(tq + (uint32_t)c0, v);
+#pragma unroll
+        for (int j8 = 0; j8 < 32; j8 += 8) {
+          const uint4 pk = tanh_pack8(v + j8, bias + c0 + j8);
+          *reinterpret_cast<uint4*>(gA + tc_off(m, c_lo + c0 + j8)) = pk;
+          if (on) *reinterpret_cast<uint4*>(H + c0 + j8) = pk;
+        }
+      }
+    } else {  // dz = dh (1 - h^2): bf16 into tile A for the next product, or dz1 in FP32
+      const __nv_bfloat16* H = (layer == 2 ? a.H2 : a.H1) + row + c_lo;
+#pragma unroll 1
+      for (int c0 = 0; c0 < kTrCols; c0 += 32) {
+        float v[32];
+        tc_ld32(tq + (uint32_t)c0, v);
+#pragma unroll
+        for (int j8 = 0; j8 < 32; j8 += 8) {
+          uint4 pk = make_uint4(0u, 0u, 0u, 0u);
+          if (on) pk = *reinterpret_cast<const uint4*>(H + c0 + j8);
+          const __nv_bfloat16* h8 = reinterpret_cast<const __nv_bfloat16*>(&pk);
+          uint4 out;
+          __nv_bfloat16* o8 = reinterpret_cast<__nv_bfloat16*>(&out);
+#pragma unroll
+          for (int j = 0; j < 8; ++j) {
+            const float h = __bfloat162float(h8[j]);
+            v[j8 + j] = v[j8 + j] * (1.f - h * h);
+            o8[j] = __float2bfloat16_rn(v[j8 + j]);
+          }
+          if (layer == 2) {
+            *reinterpret_cast<uint4*>(gA + tc_off(m, c_lo + c0 + j8)) = out;
+            if (on) *reinterpret_cast<uint4*>(a.dZ2 + row + c_lo + c0 + j8) = out;
+          } else if (on) {
+            float4* z1 = reinterpret_cast<float4*>(a.dZ1 + row + c_lo + c0 + j8);
+            z1[0] = make_float4(v[j8], v[j8 + 1], v[j8 + 2], v[j8 + 3]);
+            z1[1] = make_float4(v[j8 + 4], v[j8 + 5], v[j8 + 6], v[j8 + 7]);
+          }
+        }
+      }
+    }
+    if (layer == 1) {  // output layer, its error, dz3
+      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+      __syncthreads();  // h3 of both halves is in tile A
+      float d = 0.f;
+      if (quarter < 2) {  // output unit = quarter
+        const float* w4 = sp + kTcSW4 + quarter * kH;
+        float y = 0.f;
+#pragma unroll 4
+        for (int c = 0; c < kH; c += 8) {
+          const uint4 pk = *reinterpret_cast<const uint4*>(gA + tc_off(m, c));
+          const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&pk);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const float2 hf = __bfloat1622float2(h[j]);
+            y = fmaf(w4[c + 2 * j], hf.x, y);
+            y = fmaf(w4[c + 2 * j + 1], hf.y, y);
+          }
+        }
+        y += sp[kTcSB4 + quarter];
+        d = on ? y - a.T[2 * b + quarter] : 0.f;
+        const float dyv = d / (float)B;  // 2 (y - t) / (2 B)
+        if (on) a.dY[((long long)e * B + b) * 2 + quarter] = dyv;
+        sdy[2 * m + quarter] = dyv;
+      }
+      __syncthreads();  // dy of both outputs; every thread has read its row of h3
+      const float dy0 = sdy[2 * m], dy1 = sdy[2 * m + 1];
+#pragma unroll 1
+      for (int c = c_lo; c < c_lo + kTrCols; c += 8) {
+        const uint4 pk = *reinterpret_cast<const uint4*>(gA + tc_off(m, c));
+        const __nv_bfloat16* h8 = reinterpret_cast<const __nv_bfloat16*>(&pk);
+        uint4 out;
+        __nv_bfloat16* o8 = reinterpret_cast<__nv_bfloat16*>(&out);
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          const float dh = dy0 * sp[kTcSW4 + c + j] + dy1 * sp[kTcSW4 + kH + c + j];
+          const float h = __bfloat162float(h8[j]);
+          o8[j] = __float2bfloat16_rn(dh * (1.f - h * h));
+        }
+        *reinterpret_cast<uint4*>(gA + tc_off(m, c)) = out;
+        if (on) *reinterpret_cast<uint4*>(a.dZ3 + row + c) = out;
+      }
+      // squared errors in sample order: sums of 32 by shuffles, of 256 in warp order,
+      // one atomic per tile
+      __syncthreads();  // dy has been read
+      if (quarter < 2) sdy[2 * m + quarter] = d * d;
+      __syncthreads();
+      float l = tid < 2 * kTcRows ? sdy[tid] : 0.f;
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
+      __syncthreads();
+      if (lane == 0 && tid < 2 * kTcRows) sdy[warp] = l;
+      __syncthreads();
+      if (tid == 0) {
+        float t = 0.f;
+        for (int w = 0; w < 2 * kTcRows / 32; ++w) t += sdy[w];
+        atomicAdd(a.loss, t);
+      }
+    }
+  }
+  if (!ok) {  // the tile's later outputs stay unwritten; let the MMAs in flight finish (bounded)
+    if (tid == 0) atomicExch(a.err, 1);
+    mbar_wait(sMbar, (uint32_t)layer & 1u);
+  }
+  asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+  __syncthreads();
+  __syncwarp();
+  if (warp == 0)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kH)
+                 : "memory");
+}
+
+// ---------------------------------------------------------------------------
 // The training products on the 5th-generation tensor cores: C[z](m, n) =
 // sum_k A[z](m, k) B[z](k, n) with arbitrary strides (GemmArgs), one 128 x 128 tile of
 // C per CTA with the fp32 accumulator in
@@ -515,6 +783,58 @@ __device__ __forceinline__ uint64_t gk_desc(uint32_t saddr) {
          ((uint64_t)((kGSbo >> 4) & 0x3FFF) << 32) | (1ull << 46);
 }
 
+// One K chunk of an operand whose K runs along memory rows and whose row index is
+// contiguous (16-byte aligned, in eights): thread t takes the 8 x 8 block (rows 8 (t % 16),
+// K 8 (t / 16)), eight 16-byte loads along the rows, and transposes it in registers into
+// eight core-matrix rows.  Element loads of the same chunk took 15 us per chunk.
+__device__ __forceinline__ void stage_blocks(unsigned char* tile, const __nv_bfloat16* A, int row0,
+                                             int rows, long long s_k, int k0, int kend, int t) {
+  const int r = (t & 15) * 8, c = (t >> 4) * 8;
+  uint4 v[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    v[u] = make_uint4(0u, 0u, 0u, 0u);
+    if (row0 + r < rows && k0 + c + u < kend)
+      v[u] = *reinterpret_cast<const uint4*>(A + (long long)(k0 + c + u) * s_k + row0 + r);
+  }
+#pragma unroll
+  for (int i = 0; i < 8; ++i) {
+    uint32_t w[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+      const uint4 lo = v[2 * u], hi = v[2 * u + 1];
+      const uint32_t a = i < 2 ? lo.x : i < 4 ? lo.y : i < 6 ? lo.z : lo.w;
+      const uint32_t b = i < 2 ? hi.x : i < 4 ? hi.y : i < 6 ? hi.z : hi.w;
+      w[u] = __byte_perm(a, b, (i & 1) ? 0x7632 : 0x5410);
+    }
+    *reinterpret_cast<uint4*>(tile + gk_off(r + i, c)) = make_uint4(w[0], w[1], w[2], w[3]);
+  }
+}
+
+// one K chunk of an operand whose K runs along memory rows: thread r stages row r (its
+// neighbours' elements are adjacent, so every load is coalesced), all loads of half a
+// chunk in flight before eight elements at a time are stored as one core-matrix row
+__device__ __forceinline__ void stage_strided(unsigned char* tile, const __nv_bfloat16* A, int row,
+                                              int rows, long long s_row, long long s_k, int k0,
+                                              int kend, int r) {
+  const unsigned short* p = reinterpret_cast<const unsigned short*>(A) + (long long)row * s_row;
+#pragma unroll 1
+  for (int h = 0; h < kGK; h += kGK / 2) {
+    uint32_t v[kGK / 4];
+#pragma unroll
+    for (int u = 0; u < kGK / 4; ++u) {
+      const int k = k0 + h + 2 * u;
+      const uint32_t lo = (row < rows && k < kend) ? p[(long long)k * s_k] : 0u;
+      const uint32_t hi = (row < rows && k + 1 < kend) ? p[(long long)(k + 1) * s_k] : 0u;
+      v[u] = lo | (hi << 16);
+    }
+#pragma unroll
+    for (int c = 0; c < kGK / 2; c += 8)
+      *reinterpret_cast<uint4*>(tile + gk_off(r, h + c)) =
+          make_uint4(v[c / 2], v[c / 2 + 1], v[c / 2 + 2], v[c / 2 + 3]);
+  }
+}
+
 __global__ void __launch_bounds__(kTcRows) bf16_gemm_tc_kernel(GemmArgs g, int* err) {
   __shared__ __align__(1024) unsigned char gsm[2 * kGTile];
   __shared__ __align__(8) unsigned long long s_mbar;
@@ -522,8 +842,10 @@ __global__ void __launch_bounds__(kTcRows) bf16_gemm_tc_kernel(GemmArgs g, int* 
   const int z = blockIdx.z / g.S, sk = blockIdx.z - z * g.S;
   const int m0 = blockIdx.y * kTcRows, n0 = blockIdx.x * kH;
   const int kbeg = sk * g.kchunk, kend = min(g.K, kbeg + g.kchunk);  // this CTA's part of K
-  const __nv_bfloat16* A = g.A + (long long)z * g.sa_z;
-  const __nv_bfloat16* B = g.B + (long long)z * g.sb_z;
+  const bool two = z >= g.z2;
+  const int zi = two ? z - g.z2 : z;
+  const __nv_bfloat16* A = (two ? g.A2 : g.A) + (long long)zi * g.sa_z;
+  const __nv_bfloat16* B = (two ? g.B2 : g.B) + (long long)zi * g.sb_z;
   const int tid = threadIdx.x, warp = tid >> 5;
   const uint32_t sA = (uint32_t)__cvta_generic_to_shared(gsm), sB = sA + kGTile;
   const uint32_t mbar = (uint32_t)__cvta_generic_to_shared(&s_mbar);
@@ -540,16 +862,18 @@ __global__ void __launch_bounds__(kTcRows) bf16_gemm_tc_kernel(GemmArgs g, int* 
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&s_tmem);
-  const __nv_bfloat16 zero = __float2bfloat16(0.f);
   uint32_t commits = 0;
   bool ok = true;
   // operands contiguous along K (and 16-byte aligned rows): eight elements per load,
   // one core-matrix row per store; otherwise element by element with the contiguous
   // index (M or N) running fastest across the threads
   const bool a_vec = g.sa_k == 1 && (g.sa_m & 7) == 0 && (g.sa_z & 7) == 0 &&
-                     ((uintptr_t)g.A & 15) == 0 && (g.K & 7) == 0;
+                     ((uintptr_t)A & 15) == 0 && (g.K & 7) == 0;
   const bool b_vec = g.sb_k == 1 && (g.sb_n & 7) == 0 && (g.sb_z & 7) == 0 &&
-                     ((uintptr_t)g.B & 15) == 0 && (g.K & 7) == 0;
+                     ((uintptr_t)B & 15) == 0 && (g.K & 7) == 0;
+  // operands contiguous along M or N, in aligned eights: 8 x 8 blocks
+  const bool a_blk = g.sa_m == 1 && (g.sa_k & 7) == 0 && ((uintptr_t)A & 15) == 0 && (g.M & 7) == 0;
+  const bool b_blk = g.sb_n == 1 && (g.sb_k & 7) == 0 && ((uintptr_t)B & 15) == 0 && (g.N & 7) == 0;
   for (int k0 = kbeg; k0 < kend; k0 += kGK) {
     if (a_vec) {
       for (int q = tid; q < kTcRows * (kGK / 8); q += kTcRows) {
@@ -559,18 +883,10 @@ __global__ void __launch_bounds__(kTcRows) bf16_gemm_tc_kernel(GemmArgs g, int* 
         if (m < g.M && k < kend) v = *reinterpret_cast<const uint4*>(A + (long long)m * g.sa_m + k);
         *reinterpret_cast<uint4*>(gsm + gk_off(r, c)) = v;
       }
-    } else {  // eight loads in flight per thread, then their stores
-      for (int c0 = 0; c0 < kGK; c0 += 8) {
-        const int r = tid, m = m0 + r;  // consecutive threads: rows (M)
-        __nv_bfloat16 v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int k = k0 + c0 + u;
-          v[u] = (m < g.M && k < kend) ? A[(long long)m * g.sa_m + (long long)k * g.sa_k] : zero;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) *reinterpret_cast<__nv_bfloat16*>(gsm + gk_off(r, c0 + u)) = v[u];
-      }
+    } else if (a_blk) {
+      stage_blocks(gsm, A, m0, g.M, g.sa_k, k0, kend, tid);
+    } else {
+      stage_strided(gsm, A, m0 + tid, g.M, g.sa_m, g.sa_k, k0, kend, tid);
     }
     if (b_vec) {
       for (int q = tid; q < kTcRows * (kGK / 8); q += kTcRows) {
@@ -580,19 +896,10 @@ __global__ void __launch_bounds__(kTcRows) bf16_gemm_tc_kernel(GemmArgs g, int* 
         if (n < g.N && k < kend) v = *reinterpret_cast<const uint4*>(B + (long long)n * g.sb_n + k);
         *reinterpret_cast<uint4*>(gsm + kGTile + gk_off(r, c)) = v;
       }
+    } else if (b_blk) {
+      stage_blocks(gsm + kGTile, B, n0, g.N, g.sb_k, k0, kend, tid);
     } else {
-      for (int c0 = 0; c0 < kGK; c0 += 8) {
-        const int r = tid, n = n0 + r;  // consecutive threads: columns (N)
-        __nv_bfloat16 v[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int k = k0 + c0 + u;
-          v[u] = (n < g.N && k < kend) ? B[(long long)k * g.sb_k + (long long)n * g.sb_n] : zero;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u)
-          *reinterpret_cast<__nv_bfloat16*>(gsm + kGTile + gk_off(r, c0 + u)) = v[u];
-      }
+      stage_strided(gsm + kGTile, B, n0 + tid, g.N, g.sb_n, g.sb_k, k0, kend, tid);
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // tiles -> tensor core
     __syncthreads();
@@ -614,8 +921,8 @@ __global__ void __launch_bounds__(kTcRows) bf16_gemm_tc_kernel(GemmArgs g, int* 
   if (ok) {
     const int m = m0 + tid;
     const uint32_t tl = tmem + ((uint32_t)(warp * 32) << 16);
-    const int Z = gridDim.z / g.S;
-    float* C = g.S > 1 ? g.ws + ((long long)sk * Z + z) * g.M * g.N : g.C + (long long)z * g.sc_z;
+    float* C = g.S > 1 ? g.ws + ((long long)sk * g.Z + z) * g.M * g.N
+                       : (two ? g.C2 : g.C) + (long long)zi * g.sc_z;
     const long long cm = g.S > 1 ? g.N : g.sc_m, cn = g.S > 1 ? 1 : g.sc_n;
 #pragma unroll 1
     for (int c0 = 0; c0 < kH; c0 += 32) {
@@ -664,6 +971,50 @@ __global__ void debug_tanh_kernel(const float* x, float* y, int n) {
 
 using namespace mdeos;
 
+// batches of a training segment (see mdeos_surrogate_train), and its size where they are large
+constexpr int kSegBatches = 16;
+constexpr size_t kSegBytes = 16 << 20;
+
+// Buffers of the training calls, kept with the surrogate (allocating pinned memory takes
+// longer than a short call's training) and given back with it: two segments of samples
+// (16 B each) and their batches' losses, grown to the largest segment asked for.
+struct TrainBuffers {
+  size_t floats = 0;  // of one segment
+  float *h[2] = {nullptr, nullptr}, *d[2] = {nullptr, nullptr};
+  float *h_loss = nullptr, *d_loss = nullptr;  // [2][kSegBatches]
+  cudaEvent_t done[2] = {nullptr, nullptr};
+  // no work of an earlier call uses them: training calls end with the stream idle
+  cudaError_t reserve(size_t n) {
+    if (n <= floats) return cudaSuccess;
+    release();
+    cudaError_t e = cudaMallocHost((void**)&h_loss, 2 * kSegBatches * 4);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&d_loss, 2 * kSegBatches * 4);
+    for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
+      e = cudaMallocHost((void**)&h[k], n * 4);
+      if (e == cudaSuccess) e = cudaMalloc((void**)&d[k], n * 4);
+      if (e == cudaSuccess) e = cudaEventCreateWithFlags(&done[k], cudaEventDisableTiming);
+    }
+    if (e == cudaSuccess)
+      floats = n;
+    else
+      release();
+    return e;
+  }
+  void release() {
+    for (int k = 0; k < 2; ++k) {
+      if (h[k]) cudaFreeHost(h[k]);
+      if (d[k]) cudaFree(d[k]);
+      if (done[k]) cudaEventDestroy(done[k]);
+      h[k] = d[k] = nullptr;
+      done[k] = nullptr;
+    }
+    if (h_loss) cudaFreeHost(h_loss);
+    if (d_loss) cudaFree(d_loss);
+    h_loss = d_loss = nullptr;
+    floats = 0;
+  }
+};
+
 struct mdeos_surrogate {
   mdeos_handle* h = nullptr;
   int E = 4, maxB = 0;
@@ -672,6 +1023,7 @@ struct mdeos_surrogate {
   long long step = 0;
   float *P = nullptr, *G = nullptr, *Mm = nullptr, *Vv = nullptr;
   __nv_bfloat16 *W1b = nullptr, *W2b = nullptr, *W3b = nullptr, *W4b = nullptr;
+  __nv_bfloat16 *W2t = nullptr, *W3t = nullptr;  // transposed, for the products with dZ
   __nv_bfloat16 *H1 = nullptr, *H2 = nullptr, *H3 = nullptr, *dZb = nullptr;
   float *Z = nullptr, *dZf = nullptr, *X = nullptr, *T = nullptr, *Y = nullptr, *dY = nullptr;
   float* loss = nullptr;
@@ -680,7 +1032,8 @@ struct mdeos_surrogate {
   float* ws = nullptr;  // partial tiles of the products whose K is split
   long long ws_elems = 0;
   int infer_path = MDEOS_SURROGATE_INFER_TC;
-  bool tc_ready = false;
+  TrainBuffers tb;
+  bool tc_ready = false, train_ready = false;
   int nsm = 1;
   std::vector<void*> allocs;
   // misfit map: RMS relative pressure residual of the ensemble mean per cell of a
@@ -706,25 +1059,34 @@ constexpr int kMaxSplitK = 16;  // most CTAs one tile's K is split over
 // kMaxSplitK CTAs per tile, at least two chunks each, when the workspace ws (ws_elems
 // floats) holds the partial tiles; the partials are summed in a fixed order, so every
 // result is the same from run to run.
+//
+// A second batch (A2, B2 -> C2, same shape and strides) may share the launch; with
+// partials != nullptr the split's partial tiles are left in ws for the caller, who gets
+// the number of splits (1: the products are in C and C2).
 static cudaError_t gemm(cudaStream_t st, int* err, float* ws, long long ws_elems,
                         const __nv_bfloat16* A, const __nv_bfloat16* B, float* C, int M, int N,
                         int K, long long sa_m, long long sa_k, long long sa_z, long long sb_k,
                         long long sb_n, long long sb_z, long long sc_m, long long sc_n,
-                        long long sc_z, int Z) {
+                        long long sc_z, int Z, const __nv_bfloat16* A2 = nullptr,
+                        const __nv_bfloat16* B2 = nullptr, float* C2 = nullptr,
+                        int* partials = nullptr) {
+  // the split depends on one batch's shape, so it is the same with and without a second
   const int tiles = ((N + kH - 1) / kH) * ((M + kTcRows - 1) / kTcRows) * Z;
   const int nch = (K + kGK - 1) / kGK;
+  const int Zall = A2 != nullptr ? 2 * Z : Z;
   int S = 1, per = nch;
   if (ws && tiles < 64 && nch >= 4) {
     const int s0 = std::min(nch / 2, kMaxSplitK);
     per = (nch + s0 - 1) / s0;
     S = (nch + per - 1) / per;  // every split holds at least one chunk
-    if ((long long)S * Z * M * N > ws_elems) S = 1, per = nch;
+    if ((long long)S * Zall * M * N > ws_elems) S = 1, per = nch;
   }
   GemmArgs g{A, B, C, M, N, K, sa_m, sa_k, sa_z, sb_k, sb_n, sb_z, sc_m, sc_n, sc_z,
-             S, per * kGK, S > 1 ? ws : nullptr};
-  dim3 grid((N + kH - 1) / kH, (M + kTcRows - 1) / kTcRows, Z * S);
+             S, per * kGK, S > 1 ? ws : nullptr, A2, B2, C2, Z, Zall};
+  dim3 grid((N + kH - 1) / kH, (M + kTcRows - 1) / kTcRows, Zall * S);
   bf16_gemm_tc_kernel<<<grid, kTcRows, 0, st>>>(g, err);
-  if (S > 1) {
+  if (partials) *partials = S;
+  if (S > 1 && !partials) {
     const long long all = (long long)Z * M * N;
     gemm_splitk_reduce<<<(int)std::min<long long>((all + 255) / 256, 1024), 256, 0, st>>>(
         ws, C, M, N, Z, S, sc_m, sc_n, sc_z);
@@ -734,8 +1096,8 @@ static cudaError_t gemm(cudaStream_t st, int* err, float* ws, long long ws_elems
 
 static int nblk(long long n, int t = 256) { return (int)((n + t - 1) / t); }
 
-// forward of all models on s->X (B samples): H1..H3, Y; with targets also dY and loss
-static cudaError_t forward(mdeos_surrogate* s, int B, const float* T, cudaStream_t st) {
+// layered forward of all models on s->X (B samples): H1..H3, Y
+static cudaError_t forward(mdeos_surrogate* s, int B, cudaStream_t st) {
   const int E = s->E;
   const long long EB = (long long)E * B;
   const long long sz = (long long)B * kH;
@@ -748,40 +1110,47 @@ static cudaError_t forward(mdeos_surrogate* s, int B, const float* T, cudaStream
   e = gemm(st, s->err, s->ws, s->ws_elems, s->H2, s->W3b, s->Z, B, kH, kH, kH, 1, sz, 1, kH, kH * kH, kH, 1, sz, E);
   if (e != cudaSuccess) return e;
   mlp_bias_tanh<<<nblk(EB * kH), 256, 0, st>>>(s->Z, s->P, kOffB3, s->H3, B, E);
-  mlp_output<<<nblk(EB * 2), 256, 0, st>>>(s->H3, s->P, s->W4b, T, s->Y, s->dY, s->loss, B, E);
+  mlp_output<<<nblk(EB * 2), 256, 0, st>>>(s->H3, s->P, s->W4b, s->Y, B, E);
   return cudaGetLastError();
 }
 
-// gradients of the mean-squared error of the batch into s->G
-static cudaError_t backward(mdeos_surrogate* s, int B, cudaStream_t st) {
+// Gradients of the mean-squared error of one batch (X, T: device float[B][2]) in three
+// launches: the fused forward and backward pass per 128 samples, the sums over the batch,
+// the two 128 x 128 weight gradients.  The latter are left as *splits partial tiles in
+// s->ws for mlp_adam, or (splits == nullptr, or one split) added into s->G.
+static cudaError_t gradients(mdeos_surrogate* s, const float* X, const float* T, int B, float* loss,
+                             int* splits, cudaStream_t st) {
   const int E = s->E;
-  const long long EB = (long long)E * B;
   const long long sz = (long long)B * kH;
-  cudaError_t e;
-  mlp_back_out_w<<<nblk(E * (2 * kH + 2)), 256, 0, st>>>(s->dY, s->H3, s->G, B, E);
-  mlp_back_out_dz<<<nblk(EB * kH), 256, 0, st>>>(s->dY, s->H3, s->W4b, s->dZb, B, E);
-  // dW3 = dZ3^T H2: A(m=o, k=b) = dZ3[b][o], B(k=b, n=j) = H2[b][j]
-  e = gemm(st, s->err, s->ws, s->ws_elems, s->dZb, s->H2, s->G + kOffW3, kH, kH, B, 1, kH, sz, kH, 1, sz, kH, 1, kNParam, E);
+  if (!s->train_ready) {
+    cudaError_t e = cudaFuncSetAttribute(mlp_train_tc_kernel,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kTrSmem);
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(mlp_column_grads, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               kColSmem);
+    if (e != cudaSuccess) return e;
+    s->train_ready = true;
+  }
+  __nv_bfloat16* dZ2 = reinterpret_cast<__nv_bfloat16*>(s->Z);  // Z itself is not used here
+  TrainArgs a{X, T, s->P, s->W1b, s->W2b, s->W3b, s->W4b, s->W2t, s->W3t,
+              s->H1, s->H2, s->H3, s->dZb, dZ2, s->dZf, s->dY, loss, B, s->err};
+  dim3 grid((B + kTcRows - 1) / kTcRows, E);
+  mlp_train_tc_kernel<<<grid, kTrThreads, kTrSmem, st>>>(a);
+  mlp_column_grads<<<dim3(kH / 32, E), 256, kColSmem, st>>>(s->dY, s->H3, s->dZb, dZ2, s->dZf, X, s->G, B);
+  // dW3 = dZ3^T H2: A(m=o, k=b) = dZ3[b][o], B(k=b, n=j) = H2[b][j]; dW2 = dZ2^T H1 alike
+  if (splits)
+    return gemm(st, s->err, s->ws, s->ws_elems, s->dZb, s->H2, s->G + kOffW3, kH, kH, B, 1, kH, sz,
+                kH, 1, sz, kH, 1, kNParam, E, dZ2, s->H1, s->G + kOffW2, splits);
+  cudaError_t e = gemm(st, s->err, s->ws, s->ws_elems, s->dZb, s->H2, s->G + kOffW3, kH, kH, B, 1,
+                       kH, sz, kH, 1, sz, kH, 1, kNParam, E);
   if (e != cudaSuccess) return e;
-  mlp_bias_grad<<<nblk(E * kH), 256, 0, st>>>(s->dZb, nullptr, s->G, kOffB3, B, E);
-  // dH2 = dZ3 W3: A(m=b, k=o) = dZ3[b][o], B(k=o, n=j) = W3[o][j]
-  e = gemm(st, s->err, s->ws, s->ws_elems, s->dZb, s->W3b, s->Z, B, kH, kH, kH, 1, sz, kH, 1, kH * kH, kH, 1, sz, E);
-  if (e != cudaSuccess) return e;
-  mlp_deriv<<<nblk(EB * kH), 256, 0, st>>>(s->Z, s->H2, s->dZb, nullptr, EB * kH);
-  e = gemm(st, s->err, s->ws, s->ws_elems, s->dZb, s->H1, s->G + kOffW2, kH, kH, B, 1, kH, sz, kH, 1, sz, kH, 1, kNParam, E);
-  if (e != cudaSuccess) return e;
-  mlp_bias_grad<<<nblk(E * kH), 256, 0, st>>>(s->dZb, nullptr, s->G, kOffB2, B, E);
-  e = gemm(st, s->err, s->ws, s->ws_elems, s->dZb, s->W2b, s->Z, B, kH, kH, kH, 1, sz, kH, 1, kH * kH, kH, 1, sz, E);
-  if (e != cudaSuccess) return e;
-  mlp_deriv<<<nblk(EB * kH), 256, 0, st>>>(s->Z, s->H1, nullptr, s->dZf, EB * kH);
-  mlp_bias_grad<<<nblk(E * kH), 256, 0, st>>>(nullptr, s->dZf, s->G, kOffB1, B, E);
-  mlp_grad_w1<<<nblk(E * 2 * kH), 256, 0, st>>>(s->dZf, s->X, s->G, B, E);
-  return cudaGetLastError();
+  return gemm(st, s->err, s->ws, s->ws_elems, dZ2, s->H1, s->G + kOffW2, kH, kH, B, 1, kH, sz, kH, 1,
+              sz, kH, 1, kNParam, E);
 }
 
 static cudaError_t cast_weights(mdeos_surrogate* s, cudaStream_t st) {
   mlp_cast_weights<<<nblk((long long)s->E * kH * kH), 256, 0, st>>>(s->P, s->W1b, s->W2b, s->W3b,
-                                                                    s->W4b, s->E);
+                                                                    s->W4b, s->W2t, s->W3t, s->E);
   return cudaGetLastError();
 }
 
@@ -813,6 +1182,8 @@ extern "C" mdeos_status mdeos_surrogate_create(mdeos_handle* h, int32_t n_models
   dalloc((void**)&s->W2b, (size_t)E * kH * kH * 2);
   dalloc((void**)&s->W3b, (size_t)E * kH * kH * 2);
   dalloc((void**)&s->W4b, (size_t)E * 2 * kH * 2);
+  dalloc((void**)&s->W2t, (size_t)E * kH * kH * 2);
+  dalloc((void**)&s->W3t, (size_t)E * kH * kH * 2);
   dalloc((void**)&s->H1, EB * kH * 2);
   dalloc((void**)&s->H2, EB * kH * 2);
   dalloc((void**)&s->H3, EB * kH * 2);
@@ -828,7 +1199,7 @@ extern "C" mdeos_status mdeos_surrogate_create(mdeos_handle* h, int32_t n_models
   dalloc((void**)&s->mean, (size_t)max_batch * 2 * 8);
   dalloc((void**)&s->sd, (size_t)max_batch * 2 * 8);
   dalloc((void**)&s->err, 256);
-  s->ws_elems = (long long)kMaxSplitK * E * kH * kH;
+  s->ws_elems = 2LL * kMaxSplitK * E * kH * kH;  // two products' partial tiles
   dalloc((void**)&s->ws, (size_t)s->ws_elems * 4);
   if (e != cudaSuccess) {
     mdeos_surrogate_destroy(s);
@@ -926,9 +1297,8 @@ extern "C" mdeos_status mdeos_surrogate_grads(mdeos_surrogate* s, const double* 
   mdeos_status ms = load_batch(s, x, y, n, st);
   if (ms != MDEOS_OK) return ms;
   SCK(cudaMemsetAsync(s->loss, 0, 4, st));
-  SCK(forward(s, n, s->T, st));
-  SCK(backward(s, n, st));
-  count_launch(s->h, 20);
+  SCK(gradients(s, s->X, s->T, n, s->loss, nullptr, st));
+  count_launch(s->h, 6);
   if (grads)
     SCK(cudaMemcpyAsync(grads, s->G, (size_t)s->E * kNParam * 4, cudaMemcpyDeviceToHost, st));
   float l = 0.f;
@@ -963,41 +1333,68 @@ extern "C" mdeos_status mdeos_surrogate_train(mdeos_surrogate* s, const double* 
   std::mt19937_64 rng(seed);
   std::vector<int> perm(n);
   for (int i = 0; i < n; ++i) perm[i] = i;
-  std::vector<double> bx(2 * (size_t)batch), by(2 * (size_t)batch);
-  const long long np = (long long)s->E * kNParam;
+  // The batches go to the device in segments of up to kSegBatches (two pinned buffers in
+  // turn, so a segment is gathered and normalised while the one before trains), and their
+  // losses come back with them.
+  const int nbat = n / batch;  // full batches only
+  const int seg = std::max(1, (int)std::min<size_t>(std::min(nbat, kSegBatches),
+                                                    kSegBytes / ((size_t)batch * 16)));
+  TrainBuffers& tb = s->tb;
+  SCK(tb.reserve((size_t)seg * batch * 4));
   const float b1 = 0.9f, b2 = 0.999f;
   for (int ep = 0; ep < epochs; ++ep) {
     std::shuffle(perm.begin(), perm.end(), rng);
     double lsum = 0.0;
-    int nb = 0;
-    for (int off = 0; off + batch <= n; off += batch) {  // full batches only
-      for (int k = 0; k < batch; ++k) {
-        const int i = perm[off + k];
-        bx[2 * k] = x[2 * i];
-        bx[2 * k + 1] = x[2 * i + 1];
-        by[2 * k] = y[2 * i];
-        by[2 * k + 1] = y[2 * i + 1];
+    int held[2] = {0, 0};  // batches of the segment in flight in each buffer
+    // the losses of buffer t's segment, once it is done
+    auto collect = [&](int t) -> cudaError_t {
+      if (held[t] == 0) return cudaSuccess;
+      const cudaError_t e = cudaEventSynchronize(tb.done[t]);
+      for (int k = 0; k < held[t]; ++k)
+        lsum += (double)tb.h_loss[t * kSegBatches + k] / (2.0 * batch * s->E);
+      held[t] = 0;
+      return e;
+    };
+    int turn = 0;
+    for (int b0 = 0; b0 < nbat; b0 += seg, turn ^= 1) {
+      const int nb = std::min(seg, nbat - b0);
+      const size_t rows = (size_t)nb * batch;
+      SCK(collect(turn));
+      float* hx = tb.h[turn];
+      float* ht = hx + 2 * rows;
+      for (size_t k = 0; k < rows; ++k) {
+        const size_t i = (size_t)perm[(size_t)b0 * batch + k];
+        for (int c = 0; c < 2; ++c) {
+          const double t = (c == 0 && s->p_asinh) ? std::asinh(y[2 * i]) : y[2 * i + c];
+          hx[2 * k + c] = (float)((x[2 * i + c] - s->norm[c]) / s->norm[2 + c]);
+          ht[2 * k + c] = (float)((t - s->norm[4 + c]) / s->norm[6 + c]);
+        }
       }
-      mdeos_status ms = load_batch(s, bx.data(), by.data(), batch, st);
-      if (ms != MDEOS_OK) return ms;
-      SCK(cudaMemsetAsync(s->loss, 0, 4, st));
-      SCK(forward(s, batch, s->T, st));
-      SCK(backward(s, batch, st));
-      ++s->step;
-      const float c1 = (float)(1.0 - std::pow(0.9, (double)s->step));
-      const float c2 = (float)(1.0 - std::pow(0.999, (double)s->step));
-      mlp_adam<<<nblk(np), 256, 0, st>>>(s->P, s->G, s->Mm, s->Vv, np, (float)lr, b1, b2,
-                                         (float)(1.0 - 0.9), (float)(1.0 - 0.999), 1e-8f, c1, c2);
-      SCK(cudaGetLastError());
-      SCK(cast_weights(s, st));
-      count_launch(s->h, 22);
-      float l = 0.f;
-      SCK(cudaMemcpyAsync(&l, s->loss, 4, cudaMemcpyDeviceToHost, st));
-      SCK(cudaStreamSynchronize(st));
-      lsum += (double)l / (2.0 * batch * s->E);
-      ++nb;
+      float* dx = tb.d[turn];
+      float* dl = tb.d_loss + turn * kSegBatches;
+      SCK(cudaMemcpyAsync(dx, hx, rows * 16, cudaMemcpyHostToDevice, st));
+      SCK(cudaMemsetAsync(dl, 0, (size_t)nb * 4, st));
+      for (int k = 0; k < nb; ++k) {
+        const float* bx = dx + 2 * (size_t)k * batch;
+        int S = 1;
+        SCK(gradients(s, bx, bx + 2 * rows, batch, dl + k, &S, st));
+        ++s->step;
+        AdamArgs a{s->P, s->Mm, s->Vv, s->G, s->ws, s->W1b, s->W2b, s->W3b, s->W4b, s->W2t, s->W3t,
+                   s->E, S, (float)lr, b1, b2, (float)(1.0 - 0.9), (float)(1.0 - 0.999), 1e-8f,
+                   (float)(1.0 - std::pow(0.9, (double)s->step)),
+                   (float)(1.0 - std::pow(0.999, (double)s->step))};
+        mlp_adam<<<dim3(nblk(kNParam), s->E), 256, 0, st>>>(a);
+        SCK(cudaGetLastError());
+        count_launch(s->h, 4);
+      }
+      SCK(cudaMemcpyAsync(tb.h_loss + turn * kSegBatches, dl, (size_t)nb * 4,
+                          cudaMemcpyDeviceToHost, st));
+      SCK(cudaEventRecord(tb.done[turn], st));
+      held[turn] = nb;
     }
-    if (loss_out) loss_out[ep] = nb ? lsum / nb : 0.0;
+    SCK(collect(turn));  // the older segment first: the losses add up in batch order
+    SCK(collect(turn ^ 1));
+    if (loss_out) loss_out[ep] = nbat ? lsum / nbat : 0.0;
   }
   return take_tc_error(s, st);
 }
@@ -1010,7 +1407,7 @@ static cudaError_t infer(mdeos_surrogate* s, const double* dx, int B, double* dm
                                          s->norm[3]);
   cudaError_t e;
   if (path == MDEOS_SURROGATE_INFER_MMA) {
-    e = forward(s, B, nullptr, st);
+    e = forward(s, B, st);
     count_launch(s->h, 9);
   } else {
     if (!s->tc_ready) {
@@ -1221,6 +1618,7 @@ extern "C" mdeos_status mdeos_surrogate_destroy(mdeos_surrogate* s) {
     cudaSetDevice(handle_device(s->h));
     cudaStreamSynchronize(handle_stream(s->h));
   }
+  s->tb.release();
   for (void* p : s->allocs) cudaFree(p);
   delete s;
   return MDEOS_OK;
