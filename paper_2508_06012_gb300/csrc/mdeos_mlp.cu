@@ -276,9 +276,11 @@ __global__ void mlp_normalise(const double* Xp, float* X, int B, double m0, doub
 }
 
 // ensemble mean and (population) standard deviation of the physical outputs; with
-// p_asinh the networks predict asinh(P), mapped back by sinh before averaging
+// p_asinh the networks predict asinh(P), mapped back by sinh before averaging; inv = 1 / E
+// where E is a power of two, else 0
 __global__ void mlp_ensemble(const float* Y, int B, int E, double ym0, double ym1, double ys0,
-                             double ys1, int p_asinh, double* mean, double* sd) {
+                             double ys1, int p_asinh, double inv, double* mean,
+                             double* sd) {
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= B * 2) return;
   const int o = i % 2;
@@ -290,9 +292,17 @@ __global__ void mlp_ensemble(const float* Y, int B, int E, double ym0, double ym
     a += y;
     q += y * y;
   }
-  a /= E;
+  // a power of two divides exactly as a product (a division is ten instructions of the
+  // FP64 pipe, which bounds this kernel)
+  if (inv > 0.0) {
+    a *= inv;
+    q *= inv;
+  } else {
+    a /= E;
+    q /= E;
+  }
   mean[i] = a;
-  sd[i] = sqrt(fmax(q / E - a * a, 0.0));
+  sd[i] = sqrt(fmax(q - a * a, 0.0));
 }
 
 // ---------------------------------------------------------------------------
@@ -317,7 +327,6 @@ constexpr int kTcTile = kH * kH * 2;           // 32 KB per operand tile
 // (w_c0, w_c1) pairs, b1, b2, b3, W4 (output-major), b4
 constexpr int kTcSW1 = 0, kTcSB1 = kTcSW1 + 2 * kH, kTcSB2 = kTcSB1 + kH, kTcSB3 = kTcSB2 + kH;
 constexpr int kTcSW4 = kTcSB3 + kH, kTcSB4 = kTcSW4 + 2 * kH, kTcSmall = kTcSB4 + 4;
-constexpr int kTcSmem = 3 * kTcTile + 1024 + 64 + kTcSmall * 4;
 
 __device__ __forceinline__ uint32_t tc_off(int r, int k) {
   return (uint32_t)((r >> 3) * kSbo + (k >> 3) * kLbo + (r & 7) * 16 + (k & 7) * 2);
@@ -384,76 +393,163 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, float (&v)[32]) {
   for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
 }
 
+// two FP32 values in one register pair; the packed instructions round each half as the
+// scalar ones do
+__device__ __forceinline__ uint64_t f2_pack(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void f2_unpack(uint64_t v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
+// tanh_act of two values: the same operations, the multiply-adds in packed form (they fill
+// half the issue slots; the special-function results bound the rest).  |x| c = |x c| and
+// x poly = copysign(|x| poly, x) exactly, so the absolute value is taken by the exponential
+// and the small branch keeps its sign by itself.
+__device__ __forceinline__ void tanh_act2(uint64_t x, float& t0, float& t1) {
+  const uint64_t one = f2_pack(1.0f, 1.0f);
+  float x0, x1, a0, a1, e0, e1, r0, r1, b0, b1, s0, s1;
+  f2_unpack(x, x0, x1);
+  f2_unpack(f2_mul(x, f2_pack(2.885390081777927f, 2.885390081777927f)), a0, a1);  // 2 log2(e)
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(fabsf(a0)));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(fabsf(a1)));
+  f2_unpack(f2_add(one, f2_pack(e0, e1)), e0, e1);
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(e0));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r1) : "f"(e1));
+  f2_unpack(f2_fma(f2_pack(-2.0f, -2.0f), f2_pack(r0, r1), one), b0, b1);
+  const uint64_t x2 = f2_mul(x, x);
+  uint64_t p = f2_fma(x2, f2_pack(-17.0f / 315.0f, -17.0f / 315.0f), f2_pack(2.0f / 15.0f, 2.0f / 15.0f));
+  p = f2_fma(x2, p, f2_pack(-1.0f / 3.0f, -1.0f / 3.0f));
+  p = f2_fma(x2, p, one);
+  f2_unpack(f2_mul(x, p), s0, s1);
+  t0 = fabsf(x0) < 0.25f ? s0 : copysignf(b0, x0);
+  t1 = fabsf(x1) < 0.25f ? s1 : copysignf(b1, x1);
+}
+
 // bf16(tanh(z + bias)) of 8 consecutive units, packed as one 16-byte core-matrix row
 __device__ __forceinline__ uint4 tanh_pack8(const float* z, const float* bias) {
   uint4 pk;
   __nv_bfloat162* h = reinterpret_cast<__nv_bfloat162*>(&pk);
 #pragma unroll
-  for (int j = 0; j < 8; j += 2)
-    h[j >> 1] = __floats2bfloat162_rn(tanh_act(z[j] + bias[j]), tanh_act(z[j + 1] + bias[j + 1]));
+  for (int j = 0; j < 8; j += 2) {
+    float t0, t1;
+    tanh_act2(f2_add(f2_pack(z[j], z[j + 1]), f2_pack(bias[j], bias[j + 1])), t0, t1);
+    h[j >> 1] = __floats2bfloat162_rn(t0, t1);
+  }
   return pk;
 }
 
-// Persistent: grid (CTAs per model, models).  The CTA stages its model's W2 and W3
-// once, then takes 128-input tiles tile = blockIdx.x, + gridDim.x, ...  Thread t
-// serves row m = t % 128 (TMEM lane m) and column half t / 128: warps w and w + 4
+// Persistent: grid (CTAs per model, models), one CTA per SM.  The CTA stages its model's
+// W2 and W3 once; its groups of 256 threads (up to kTcGroups, each with its own tile A, TMEM
+// columns, mbarrier and named barrier) then take 128-input tiles independently.  Thread t
+// of a group serves row m = t % 128 (TMEM lane m) and column half t / 128: warps w and w + 4
 // read the same 32 lanes, columns 0-63 and 64-127.
-__global__ void __launch_bounds__(kTcThreads) mlp_infer_tc_kernel(const float* X, const float* P,
-                                                                  const __nv_bfloat16* W1b,
-                                                                  const __nv_bfloat16* W2b,
-                                                                  const __nv_bfloat16* W3b,
-                                                                  const __nv_bfloat16* W4b,
-                                                                  float* Y, int B, int* err) {
+//
+// What bounds it is the 384 tanh per row, two special-function results each (16 per clock
+// and SM: 12.3k cycles for two tiles), then the issue slots of the rest.  A tile alternates
+// between its product and its tanh, so other tiles have to fill the gaps: with two CTAs of
+// 256 threads per SM, each with its own copy of the weights (101 KB), two tiles took 21.5k
+// cycles; four groups around one copy (197 KB, all 512 TMEM columns)
+// fill them (2^20 queries, normalising and averaging included: 1348 us before, 1112 now).
+constexpr int kTcGroups = 4;
+constexpr int kTcCtaSmem = (2 + kTcGroups) * kTcTile + 1024 + 128 + kTcSmall * 4;
+
+__device__ __forceinline__ void group_bar(int id) {
+  asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(kTcThreads) : "memory");
+}
+__device__ __forceinline__ bool group_bar_and(int id, bool p) {
+  int r;
+  asm volatile(
+      "{\n\t.reg .pred pi, po;\n\t"
+      "setp.ne.s32 pi, %3, 0;\n\t"
+      "bar.red.and.pred po, %1, %2, pi;\n\t"
+      "selp.s32 %0, 1, 0, po;\n\t}"
+      : "=r"(r) : "r"(id), "n"(kTcThreads), "r"((int)p) : "memory");
+  return r != 0;
+}
+
+__global__ void __launch_bounds__(kTcGroups * kTcThreads, 1)
+    mlp_infer_tc_kernel(const float* X, const float* P, const __nv_bfloat16* W1b,
+                        const __nv_bfloat16* W2b, const __nv_bfloat16* W3b,
+                        const __nv_bfloat16* W4b, float* Y, int B, int* err) {
   extern __shared__ __align__(1024) unsigned char tsm[];
   const uint32_t sbase = ((uint32_t)__cvta_generic_to_shared(tsm) + 1023u) & ~1023u;
   unsigned char* gbase = tsm + (sbase - (uint32_t)__cvta_generic_to_shared(tsm));
-  const uint32_t sA = sbase, sW2 = sbase + kTcTile, sW3 = sbase + 2 * kTcTile;
-  const uint32_t sMbar = sbase + 3 * kTcTile, sTmem = sMbar + 8;
-  unsigned char* gA = gbase;
-  const int e = blockIdx.y, tid = threadIdx.x, warp = tid >> 5;
+  const int groups = blockDim.x / kTcThreads;
+  const int e = blockIdx.y, tid = threadIdx.x % kTcThreads, grp = threadIdx.x / kTcThreads;
+  const int warp = tid >> 5, bar = 1 + grp;
+  const uint32_t sW2 = sbase, sW3 = sbase + kTcTile;
+  const uint32_t sA = sbase + (uint32_t)(2 + grp) * kTcTile;
+  unsigned char* gA = gbase + (2 + grp) * kTcTile;
+  // behind the tiles: an mbarrier per group, the TMEM address, the small parameters
+  const uint32_t sCtl = sbase + (uint32_t)(2 + groups) * kTcTile;
+  unsigned char* gCtl = gbase + (2 + groups) * kTcTile;
+  const uint32_t sMbar = sCtl + 8u * (uint32_t)grp, sTmem = sCtl + 64;
   const int m = tid & (kTcRows - 1), half = tid >> 7, c_lo = half * (kH / 2);
   const int ntiles = (B + kTcRows - 1) / kTcRows;
   const float* p = P + (long long)e * kNParam;
-  float* sp = reinterpret_cast<float*>(gbase + 3 * kTcTile + 64);  // small parameters
-  for (int k = tid; k < 2 * kH; k += kTcThreads) {  // the bf16-rounded weights, as FP32
+  float* sp = reinterpret_cast<float*>(gCtl + 128);  // small parameters
+  for (int k = threadIdx.x; k < 2 * kH; k += blockDim.x) {  // the bf16-rounded weights, as FP32
     sp[kTcSW1 + k] = __bfloat162float(W1b[(long long)e * 2 * kH + k]);
     sp[kTcSW4 + k] = __bfloat162float(W4b[(long long)e * 2 * kH + k]);
   }
-  for (int k = tid; k < kH; k += kTcThreads) {
+  for (int k = threadIdx.x; k < kH; k += blockDim.x) {
     sp[kTcSB1 + k] = p[kOffB1 + k];
     sp[kTcSB2 + k] = p[kOffB2 + k];
     sp[kTcSB3 + k] = p[kOffB3 + k];
   }
-  if (tid < 2) sp[kTcSB4 + tid] = p[kOffB4 + tid];
+  if (threadIdx.x < 2) sp[kTcSB4 + threadIdx.x] = p[kOffB4 + threadIdx.x];
   const float* w4 = sp + kTcSW4 + half * kH;  // output unit = half
   // weights of this model into the canonical layout, 16 bytes at a time; consecutive
   // threads fill consecutive 16-byte rows of the core matrices (no bank conflicts)
-  for (int q = tid; q < kH * kH / 8; q += kTcThreads) {
+  for (int q = threadIdx.x; q < kH * kH / 8; q += blockDim.x) {
     const int n = (q >> 7) * 8 + (q & 7), k = ((q >> 3) & 15) * 8;
     const uint4 a2 = *reinterpret_cast<const uint4*>(W2b + (long long)e * kH * kH + n * kH + k);
     const uint4 a3 = *reinterpret_cast<const uint4*>(W3b + (long long)e * kH * kH + n * kH + k);
-    *reinterpret_cast<uint4*>(gbase + kTcTile + tc_off(n, k)) = a2;
-    *reinterpret_cast<uint4*>(gbase + 2 * kTcTile + tc_off(n, k)) = a3;
+    *reinterpret_cast<uint4*>(gbase + tc_off(n, k)) = a2;
+    *reinterpret_cast<uint4*>(gbase + kTcTile + tc_off(n, k)) = a3;
   }
   if (tid == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sMbar) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
-  if (warp == 0) {  // 128 TMEM columns: the 128 x 128 fp32 accumulator
+  // 128 TMEM columns per group (its 128 x 128 fp32 accumulator), a power of two in all
+  const uint32_t cols = groups == 1 ? kH : (groups == 2 ? 2 * kH : 4 * kH);
+  if (threadIdx.x < 32) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
-                 ::"r"(sTmem), "r"(kH) : "memory");
+                 ::"r"(sTmem), "r"(cols) : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // weights -> tensor core
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(gbase + 3 * kTcTile + 8);
+  const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(gCtl + 64);
+  const uint32_t tacc = tmem + (uint32_t)(grp * kH);  // the group's accumulator
   // this thread's lane quarter (warp % 4) and column half
-  const uint32_t tq = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c_lo;
+  const uint32_t tq = tacc + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c_lo;
   uint32_t commits = 0;  // MMA groups committed so far (mbarrier phase parity)
   bool ok = true;
-  int tile = blockIdx.x;
-  for (; tile < ntiles; tile += gridDim.x) {
+  const int tstep = gridDim.x * groups;
+  int tile = blockIdx.x + grp * gridDim.x;
+  for (; tile < ntiles; tile += tstep) {
     const int b = tile * kTcRows + m;
     // layer 1 on the CUDA cores: this row's units c_lo .. c_lo + 63 -> tile A
     const float x0 = b < B ? X[2 * b] : 0.f, x1 = b < B ? X[2 * b + 1] : 0.f;
@@ -468,19 +564,19 @@ __global__ void __launch_bounds__(kTcThreads) mlp_infer_tc_kernel(const float* X
       *reinterpret_cast<uint4*>(gA + tc_off(m, c)) = tanh_pack8(z, sp + kTcSB1 + c);
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // h1 -> tensor core
-    __syncthreads();
+    group_bar(bar);
     for (int layer = 0; layer < 2; ++layer) {
       if (tid == 0) {
         const uint32_t sW = layer == 0 ? sW2 : sW3;
 #pragma unroll
         for (int ks = 0; ks < kH / 16; ++ks)  // K step of 16 = two core matrices along K
-          tc_mma(tmem, tc_desc(sA + ks * 2 * kLbo), tc_desc(sW + ks * 2 * kLbo), ks > 0);
+          tc_mma(tacc, tc_desc(sA + ks * 2 * kLbo), tc_desc(sW + ks * 2 * kLbo), ks > 0);
         tc_commit(sMbar);
       }
       __syncwarp();
       const bool done = mbar_wait(sMbar, commits & 1u);
       ++commits;
-      ok = __syncthreads_and(done) != 0;  // the same decision in every thread
+      ok = group_bar_and(bar, done);  // the same decision in every thread of the group
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
       if (!ok) break;
       // epilogue: h = bf16(tanh(z + b)) of this row's 64 units -> tile A (the MMA that
@@ -497,7 +593,7 @@ __global__ void __launch_bounds__(kTcThreads) mlp_infer_tc_kernel(const float* X
       }
       if (layer == 0) asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
       asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncthreads();
+      group_bar(bar);
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
     }
     if (!ok) break;
@@ -515,11 +611,11 @@ __global__ void __launch_bounds__(kTcThreads) mlp_infer_tc_kernel(const float* X
       }
     }
     if (b < B) Y[((long long)e * B + b) * 2 + half] = y + sp[kTcSB4 + half];
-    __syncthreads();  // tile A is rewritten by the next tile's layer 1
+    group_bar(bar);  // tile A is rewritten by the next tile's layer 1
   }
-  if (!ok) {  // NaN for this CTA's unfinished tiles; let MMAs in flight finish (bounded)
+  if (!ok) {  // NaN for this group's unfinished tiles; let MMAs in flight finish (bounded)
     if (tid == 0) atomicExch(err, 1);
-    for (; tile < ntiles; tile += gridDim.x) {
+    for (; tile < ntiles; tile += tstep) {
       const int b = tile * kTcRows + m;
       if (b < B) Y[((long long)e * B + b) * 2 + half] = __int_as_float(0x7fc00000);
     }
@@ -528,8 +624,8 @@ __global__ void __launch_bounds__(kTcThreads) mlp_infer_tc_kernel(const float* X
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   __syncwarp();
-  if (warp == 0)
-    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kH)
+  if (threadIdx.x < 32)
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(cols)
                  : "memory");
 }
 
@@ -1412,7 +1508,7 @@ static cudaError_t infer(mdeos_surrogate* s, const double* dx, int B, double* dm
   } else {
     if (!s->tc_ready) {
       e = cudaFuncSetAttribute(mlp_infer_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               kTcSmem);
+                               kTcCtaSmem);
       if (e != cudaSuccess) return e;
       int dev = 0;
       e = cudaGetDevice(&dev);
@@ -1420,18 +1516,23 @@ static cudaError_t infer(mdeos_surrogate* s, const double* dx, int B, double* dm
       if (e != cudaSuccess) return e;
       s->tc_ready = true;
     }
-    // two resident CTAs per SM in all (shared memory bounds it at two)
+    // one CTA per SM and model share; as many groups (tiles at a time) per CTA as keep
+    // every CTA's groups busy: few tiles spread over more SMs first
     const int tiles = (B + kTcRows - 1) / kTcRows;
-    const int per_model = std::max(1, std::min(tiles, (2 * s->nsm + s->E - 1) / s->E));
+    const int per_model = std::max(1, std::min(tiles, s->nsm / s->E));
+    int groups = 1;
+    while (groups < kTcGroups && tiles > per_model * groups) groups *= 2;
     dim3 grid(per_model, s->E);
-    mlp_infer_tc_kernel<<<grid, kTcThreads, kTcSmem, st>>>(s->X, s->P, s->W1b, s->W2b, s->W3b,
-                                                          s->W4b, s->Y, B, s->err);
+    mlp_infer_tc_kernel<<<grid, groups * kTcThreads,
+                          kTcCtaSmem - (kTcGroups - groups) * kTcTile, st>>>(
+        s->X, s->P, s->W1b, s->W2b, s->W3b, s->W4b, s->Y, B, s->err);
     e = cudaGetLastError();
     count_launch(s->h, 3);
   }
   if (e != cudaSuccess) return e;
   mlp_ensemble<<<nblk(2 * B), 256, 0, st>>>(s->Y, B, s->E, s->norm[4], s->norm[5], s->norm[6],
-                                            s->norm[7], s->p_asinh, dmean, dsd);
+                                            s->norm[7], s->p_asinh,
+                                            (s->E & (s->E - 1)) == 0 ? 1.0 / s->E : 0.0, dmean, dsd);
   return cudaGetLastError();
 }
 
