@@ -1111,6 +1111,36 @@ struct TrainBuffers {
   }
 };
 
+// Staging of predict's host arrays, kept with the surrogate: up to kIoRows queries at a
+// time (inputs 16 B; outputs a head with the error word, mean and sd 16 B each, 8 B per
+// model), grown to the largest chunk asked for.
+constexpr int kIoRows = 1 << 18;
+constexpr size_t kIoHead = 256;
+struct PredictBuffers {
+  int rows = 0;
+  char *h_in = nullptr, *h_out = nullptr, *d_out = nullptr;
+  cudaError_t reserve(int n, int E) {
+    if (n <= rows) return cudaSuccess;
+    release();
+    const size_t out = kIoHead + (size_t)n * (32 + 8 * (size_t)E);
+    cudaError_t e = cudaMallocHost((void**)&h_in, (size_t)n * 16);
+    if (e == cudaSuccess) e = cudaMallocHost((void**)&h_out, out);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&d_out, out);
+    if (e == cudaSuccess)
+      rows = n;
+    else
+      release();
+    return e;
+  }
+  void release() {
+    if (h_in) cudaFreeHost(h_in);
+    if (h_out) cudaFreeHost(h_out);
+    if (d_out) cudaFree(d_out);
+    h_in = h_out = d_out = nullptr;
+    rows = 0;
+  }
+};
+
 struct mdeos_surrogate {
   mdeos_handle* h = nullptr;
   int E = 4, maxB = 0;
@@ -1129,6 +1159,7 @@ struct mdeos_surrogate {
   long long ws_elems = 0;
   int infer_path = MDEOS_SURROGATE_INFER_TC;
   TrainBuffers tb;
+  PredictBuffers io;
   bool tc_ready = false, train_ready = false;
   int nsm = 1;
   std::vector<void*> allocs;
@@ -1192,8 +1223,8 @@ static cudaError_t gemm(cudaStream_t st, int* err, float* ws, long long ws_elems
 
 static int nblk(long long n, int t = 256) { return (int)((n + t - 1) / t); }
 
-// layered forward of all models on s->X (B samples): H1..H3, Y
-static cudaError_t forward(mdeos_surrogate* s, int B, cudaStream_t st) {
+// layered forward of all models on s->X (B samples): H1..H3, and the outputs into Y
+static cudaError_t forward(mdeos_surrogate* s, int B, float* Y, cudaStream_t st) {
   const int E = s->E;
   const long long EB = (long long)E * B;
   const long long sz = (long long)B * kH;
@@ -1206,7 +1237,7 @@ static cudaError_t forward(mdeos_surrogate* s, int B, cudaStream_t st) {
   e = gemm(st, s->err, s->ws, s->ws_elems, s->H2, s->W3b, s->Z, B, kH, kH, kH, 1, sz, 1, kH, kH * kH, kH, 1, sz, E);
   if (e != cudaSuccess) return e;
   mlp_bias_tanh<<<nblk(EB * kH), 256, 0, st>>>(s->Z, s->P, kOffB3, s->H3, B, E);
-  mlp_output<<<nblk(EB * 2), 256, 0, st>>>(s->H3, s->P, s->W4b, s->Y, B, E);
+  mlp_output<<<nblk(EB * 2), 256, 0, st>>>(s->H3, s->P, s->W4b, Y, B, E);
   return cudaGetLastError();
 }
 
@@ -1498,12 +1529,12 @@ extern "C" mdeos_status mdeos_surrogate_train(mdeos_surrogate* s, const double* 
 // inference of B <= maxB inputs (device FP64 [B][2]) -> per-model s->Y and the ensemble
 // mean / sd (device FP64 [B][2]) on stream st
 static cudaError_t infer(mdeos_surrogate* s, const double* dx, int B, double* dmean, double* dsd,
-                         int path, cudaStream_t st) {
+                         float* dY, int path, cudaStream_t st) {
   mlp_normalise<<<nblk(B), 256, 0, st>>>(dx, s->X, B, s->norm[0], s->norm[1], s->norm[2],
                                          s->norm[3]);
   cudaError_t e;
   if (path == MDEOS_SURROGATE_INFER_MMA) {
-    e = forward(s, B, st);
+    e = forward(s, B, dY, st);
     count_launch(s->h, 9);
   } else {
     if (!s->tc_ready) {
@@ -1525,12 +1556,12 @@ static cudaError_t infer(mdeos_surrogate* s, const double* dx, int B, double* dm
     dim3 grid(per_model, s->E);
     mlp_infer_tc_kernel<<<grid, groups * kTcThreads,
                           kTcCtaSmem - (kTcGroups - groups) * kTcTile, st>>>(
-        s->X, s->P, s->W1b, s->W2b, s->W3b, s->W4b, s->Y, B, s->err);
+        s->X, s->P, s->W1b, s->W2b, s->W3b, s->W4b, dY, B, s->err);
     e = cudaGetLastError();
     count_launch(s->h, 3);
   }
   if (e != cudaSuccess) return e;
-  mlp_ensemble<<<nblk(2 * B), 256, 0, st>>>(s->Y, B, s->E, s->norm[4], s->norm[5], s->norm[6],
+  mlp_ensemble<<<nblk(2 * B), 256, 0, st>>>(dY, B, s->E, s->norm[4], s->norm[5], s->norm[6],
                                             s->norm[7], s->p_asinh,
                                             (s->E & (s->E - 1)) == 0 ? 1.0 / s->E : 0.0, dmean, dsd);
   return cudaGetLastError();
@@ -1559,7 +1590,7 @@ extern "C" mdeos_status mdeos_surrogate_infer_device(mdeos_surrogate* s, const d
   cudaStream_t st = stream ? (cudaStream_t)stream : handle_stream(s->h);
   for (int off = 0; off < n; off += s->maxB) {
     const int B = std::min(s->maxB, n - off);
-    SCK(infer(s, d_x + 2 * (size_t)off, B, d_mean + 2 * (size_t)off, d_sd + 2 * (size_t)off,
+    SCK(infer(s, d_x + 2 * (size_t)off, B, d_mean + 2 * (size_t)off, d_sd + 2 * (size_t)off, s->Y,
               s->infer_path, st));
   }
   return MDEOS_OK;
@@ -1570,25 +1601,38 @@ extern "C" mdeos_status mdeos_surrogate_predict(mdeos_surrogate* s, const double
   if (!s || !x || n < 0) return set_error(MDEOS_EINVAL, "bad predict arguments");
   SCK(cudaSetDevice(handle_device(s->h)));
   cudaStream_t st = handle_stream(s->h);
-  for (int off = 0; off < n; off += s->maxB) {
-    const int B = std::min(s->maxB, n - off);
-    SCK(cudaMemcpyAsync(s->Xp, x + 2 * (size_t)off, (size_t)B * 16, cudaMemcpyHostToDevice, st));
-    SCK(infer(s, s->Xp, B, s->mean, s->sd, s->infer_path, st));
-    if (mean)
-      SCK(cudaMemcpyAsync(mean + 2 * (size_t)off, s->mean, (size_t)B * 16, cudaMemcpyDeviceToHost, st));
-    if (sd)
-      SCK(cudaMemcpyAsync(sd + 2 * (size_t)off, s->sd, (size_t)B * 16, cudaMemcpyDeviceToHost, st));
+  // One copy in and one out per chunk, through pinned memory: the chunk's mean, sd and
+  // per-model outputs and the error word share a device block.  (Copies to and from pageable
+  // memory are staged and waited for one by one: eight of them took half of a 2000-query
+  // call, 123 us; it takes 67 now.)
+  const int chunk = std::min(s->maxB, kIoRows);
+  SCK(s->io.reserve(std::min(chunk, n), s->E));
+  int err = 0;
+  for (int off = 0; off < n; off += chunk) {
+    const int B = std::min(chunk, n - off);
+    const size_t ob = (size_t)B * 16, yb = per_model ? (size_t)s->E * B * 8 : 0;
+    char* d = s->io.d_out;
+    std::memcpy(s->io.h_in, x + 2 * (size_t)off, ob);
+    SCK(cudaMemcpyAsync(s->Xp, s->io.h_in, ob, cudaMemcpyHostToDevice, st));
+    SCK(infer(s, s->Xp, B, (double*)(d + kIoHead), (double*)(d + kIoHead + ob),
+              (float*)(d + kIoHead + 2 * ob), s->infer_path, st));
+    SCK(cudaMemcpyAsync(d, s->err, 4, cudaMemcpyDeviceToDevice, st));
+    SCK(cudaMemcpyAsync(s->io.h_out, d, kIoHead + 2 * ob + yb, cudaMemcpyDeviceToHost, st));
+    SCK(cudaStreamSynchronize(st));
+    const char* h = s->io.h_out;
+    if (mean) std::memcpy(mean + 2 * (size_t)off, h + kIoHead, ob);
+    if (sd) std::memcpy(sd + 2 * (size_t)off, h + kIoHead + ob, ob);
     if (per_model)
       for (int m = 0; m < s->E; ++m)
-        SCK(cudaMemcpyAsync(per_model + ((size_t)m * n + off) * 2, s->Y + (size_t)m * B * 2,
-                            (size_t)B * 8, cudaMemcpyDeviceToHost, st));
-    SCK(cudaStreamSynchronize(st));
+        std::memcpy(per_model + ((size_t)m * n + off) * 2, h + kIoHead + 2 * ob + (size_t)m * B * 8,
+                    (size_t)B * 8);
+    err |= *reinterpret_cast<const int*>(h);
   }
-  int err = 0;
-  SCK(cudaMemcpyAsync(&err, s->err, 4, cudaMemcpyDeviceToHost, st));
-  SCK(cudaMemsetAsync(s->err, 0, 4, st));
-  SCK(cudaStreamSynchronize(st));
-  if (err) return set_error(MDEOS_ETIMEDOUT, "surrogate: a tensor-core wait ran out");
+  if (err) {
+    SCK(cudaMemsetAsync(s->err, 0, 4, st));
+    SCK(cudaStreamSynchronize(st));
+    return set_error(MDEOS_ETIMEDOUT, "surrogate: a tensor-core wait ran out");
+  }
   return MDEOS_OK;
 }
 
@@ -1720,6 +1764,7 @@ extern "C" mdeos_status mdeos_surrogate_destroy(mdeos_surrogate* s) {
     cudaStreamSynchronize(handle_stream(s->h));
   }
   s->tb.release();
+  s->io.release();
   for (void* p : s->allocs) cudaFree(p);
   delete s;
   return MDEOS_OK;
