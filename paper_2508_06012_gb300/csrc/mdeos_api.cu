@@ -24,7 +24,7 @@ cudaError_t set_batch_attributes(int max_smem);
 cudaError_t launch_eos_batch(const BoxDesc* boxes, const WorkItem* items, int nitems, int* counter,
                              mdeos_result* results, uint16_t* nl, long long nl_elems_per_cta,
                              const RunParams& rp, int grid, int smem, cudaStream_t st,
-                             int* ready, int cluster);
+                             int* ready, int cluster, int threads = kCtaThreads);
 cudaError_t set_debug_attributes(int max_smem);
 cudaError_t launch_debug_lift(const BoxDesc& bd, const RunParams& rp, double T, int apt,
                               int ncell_cap, int smem, float4* x4, float4* v4, double* e_out,
@@ -314,6 +314,7 @@ struct Plan {
   long long nl_per_cta = 0;
   int grid = 0;
   int cluster = 1;  // CTAs per box (thread-block clusters, eos_cluster_kernel); 1: none
+  int threads = kCtaThreads;  // threads per CTA (fewer only for clusters of small boxes)
 };
 
 static mdeos_status make_plan(const mdeos_request* reqs, int n, const mdeos_config& c, int nsm,
@@ -404,7 +405,7 @@ static mdeos_status make_plan(const mdeos_request* reqs, int n, const mdeos_conf
       plan.boxes.push_back(bp[k].bd);
       // room for position windows behind the CTA's BigShared: the whole box when it
       // fits, else all the shared memory there is
-      const int cache = kBigSharedBytes + 16 * big_cap(bp[k].bd.natoms);
+      const int cache = kBigSharedBytes + kBigCluBytes + 16 * big_cap(bp[k].bd.natoms);
       plan.smem = std::max(plan.smem, std::min(cache, smem_max));
       plan.nl_per_cta = std::max(plan.nl_per_cta, (long long)wi.nl_stride);
       items.push_back({wi, bp[k].cost});
@@ -424,7 +425,7 @@ static mdeos_status make_plan(const mdeos_request* reqs, int n, const mdeos_conf
     int nb = 0;
     while (k < bp.size() && bp[k].warps == warps && bp[k].apt == apt && nb < per_cta) {
       const int nc2 = std::max(ncell_cap, bp[k].ncell);
-      const int stride = group_smem_bytes(warps, apt, nc2);
+      const int stride = group_smem_bytes(warps, apt, nc2, plan.cluster > 1);
       if ((nb + 1) * stride > smem_max) break;
       ncell_cap = nc2;
       maxnb = std::max(maxnb, bp[k].bd.maxnb);
@@ -436,7 +437,7 @@ static mdeos_status make_plan(const mdeos_request* reqs, int n, const mdeos_conf
     if (nb == 0) return fail(MDEOS_EINVAL, "a box does not fit in shared memory");
     wi.nbox = nb;
     wi.ncell_cap = ncell_cap;
-    wi.smem_stride = group_smem_bytes(warps, apt, ncell_cap);
+    wi.smem_stride = group_smem_bytes(warps, apt, ncell_cap, plan.cluster > 1);
     wi.nl_stride = ((maxnb + 7) & ~7) * npad;
     plan.smem = std::max(plan.smem, nb * wi.smem_stride);
     plan.nl_per_cta = std::max(plan.nl_per_cta, (long long)nb * wi.nl_stride);
@@ -624,7 +625,8 @@ extern "C" mdeos_status mdeos_create(const mdeos_config* cfg, mdeos_handle** out
   cudaDeviceGetAttribute(&minor, cudaDevAttrComputeCapabilityMinor, h->device);
   cudaDeviceGetAttribute(&h->nsm, cudaDevAttrMultiProcessorCount, h->device);
   cudaDeviceGetAttribute(&h->smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, h->device);
-  h->smem_max -= 2048;  // static shared memory of the kernels (the serving kernel's is ~1.3 KB)
+  // static shared memory of the kernels (the serving kernel's is ~1.3 KB) and kSmemAlign
+  h->smem_max -= 2048 + kSmemAlign;
   e = set_batch_attributes(h->smem_max);
   if (e == cudaSuccess) e = set_debug_attributes(h->smem_max);
   if (e != cudaSuccess) {
@@ -789,7 +791,8 @@ extern "C" mdeos_status mdeos_submit(mdeos_handle* h, const mdeos_request* reqs,
     CK(cudaMemsetAsync(d + off_cnt, 0, sizeof(int), h->stream));
     e = launch_eos_batch((BoxDesc*)d, (WorkItem*)(d + off_items), (int)ni, (int*)(d + off_cnt),
                          (mdeos_result*)(d + off_res), h->d_nl, plan.nl_per_cta, h->rp, plan.grid,
-                         plan.smem, h->stream, nullptr, plan.cluster);
+                         plan.smem, h->stream, nullptr, plan.cluster,
+                         plan.threads);
     if (e != cudaSuccess) return cuda_fail(e, "eos_batch_kernel launch");
     h->launches += 1;
     CK(cudaMemcpyAsync(t.h_out.p, d + off_res, (size_t)n * sizeof(mdeos_result),
@@ -827,7 +830,8 @@ static mdeos_status run_plan_sync(mdeos_handle* h, const Plan& plan, int n, mdeo
   if (e == cudaSuccess)
     e = launch_eos_batch((BoxDesc*)d, (WorkItem*)(d + off_items), (int)ni, (int*)(d + off_cnt),
                          (mdeos_result*)(d + off_res), h->d_nl, plan.nl_per_cta, h->rp, plan.grid,
-                         plan.smem, h->stream, nullptr, plan.cluster);
+                         plan.smem, h->stream, nullptr, plan.cluster,
+                         plan.threads);
   if (e == cudaSuccess)
     e = cudaMemcpyAsync(out, d + off_res, (size_t)n * sizeof(mdeos_result),
                         cudaMemcpyDeviceToHost, h->stream);
@@ -988,7 +992,7 @@ extern "C" mdeos_status mdeos_batch_create(mdeos_handle* h, const mdeos_request*
   cudaMemsetAsync(b->d_counter, 0, sizeof(int), cs);
   if (ni > 0)
     launch_eos_batch(b->d_boxes, b->d_items, (int)ni, b->d_counter, b->d_results, b->d_nl,
-                     p.nl_per_cta, h->rp, p.grid, p.smem, cs, nullptr, p.cluster);
+                     p.nl_per_cta, h->rp, p.grid, p.smem, cs, nullptr, p.cluster, p.threads);
   e = cudaStreamEndCapture(cs, &b->graph);
   cudaStreamDestroy(cs);
   if (e != cudaSuccess) {
@@ -1076,7 +1080,8 @@ static mdeos_status time_plan(mdeos_handle* h, const Plan& plan, int n, float* m
   if (e == cudaSuccess)
     e = launch_eos_batch((BoxDesc*)d, (WorkItem*)(d + off_items), (int)ni, (int*)(d + off_cnt),
                          (mdeos_result*)(d + off_res), h->d_nl, plan.nl_per_cta, h->rp, plan.grid,
-                         plan.smem, h->stream, nullptr, plan.cluster);
+                         plan.smem, h->stream, nullptr, plan.cluster,
+                         plan.threads);
   if (e == cudaSuccess) e = cudaEventRecord(e1, h->stream);
   std::vector<mdeos_result> res(n);
   if (e == cudaSuccess)
@@ -1324,7 +1329,8 @@ mdeos_status eval_into_device(mdeos_handle* h, const mdeos_request* reqs, int n,
   CK(cudaMemsetAsync(d + off_cnt, 0, sizeof(int), h->stream));
   cudaError_t e = launch_eos_batch((BoxDesc*)d, (WorkItem*)(d + off_items), (int)ni,
                                    (int*)(d + off_cnt), d_results, h->d_nl, plan.nl_per_cta, h->rp,
-                                   plan.grid, plan.smem, h->stream, nullptr, plan.cluster);
+                                   plan.grid, plan.smem, h->stream, nullptr, plan.cluster,
+                         plan.threads);
   if (e != cudaSuccess) return cuda_fail(e, "eos_batch_kernel launch");
   h->launches += 1;
   return MDEOS_OK;
@@ -1381,7 +1387,7 @@ static mdeos_status debug_setup(const mdeos_config* cfg, int n, double L, int pa
   cudaGetDevice(&dev);
   int smem_max = 0;
   cudaDeviceGetAttribute(&smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  smem_max -= 1024;
+  smem_max -= 2048;
   if (dev < 64 && !attr_done[dev]) {
     CK(set_debug_attributes(smem_max));
     attr_done[dev] = true;

@@ -52,8 +52,6 @@ struct BigClu {
                    // (shared memory behind BigShared; only with csize > 1)
 };
 
-// shared memory of the cluster partials, behind BigShared (position windows follow)
-constexpr int kBigCluBytes = 2 * kMaxCluster * kRedSlots * 8;
 
 __device__ __forceinline__ BigClu big_clu(int n, int crank, int csize, long long* clu = nullptr) {
   BigClu c;
@@ -134,7 +132,7 @@ struct BigMem {
 __device__ __forceinline__ void big_pos_cache(BigMem& m, const unsigned char* dyn_base, int off) {
   uint32_t dyn;
   asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
-  const int cap = (int)(((long long)dyn - off) / 16);
+  const int cap = (int)(((long long)dyn - kSmemAlign - off) / 16);
   m.sx_a = cap >= 1024 ? (uint32_t)__cvta_generic_to_shared(dyn_base) + (uint32_t)off : 0u;
   m.sx_cap = cap >= 1024 ? cap : 0;
 }

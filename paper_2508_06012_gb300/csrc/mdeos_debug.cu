@@ -195,7 +195,8 @@ __device__ void debug_md_body(const Group& g, const BoxDesc& bd, const RunParams
 __global__ void __launch_bounds__(kCtaThreads, 1)
     debug_lift_kernel(BoxDesc bd, RunParams rp, double T, int apt, int ncell_cap, float4* x4,
                       float4* v4, double* e_out, uint16_t* nl) {
-  extern __shared__ __align__(128) unsigned char smem[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  unsigned char* smem = align_smem(smem_raw);
   const Group g = make_group(smem, threadIdx.x, 32, apt, ncell_cap, 1, nl);
   switch (apt) {
     case 1: debug_lift_body<1>(g, bd, rp, T, x4, v4, e_out); break;
@@ -219,7 +220,8 @@ __device__ void debug_forces_path(const Group& g, const BoxDesc& bd, const RunPa
 __global__ void __launch_bounds__(kCtaThreads, 1)
     debug_forces_kernel(BoxDesc bd, RunParams rp, int apt, int ncell_cap, const float4* x4,
                         float4* f4, double* ew, long long* pairs, uint16_t* nl) {
-  extern __shared__ __align__(128) unsigned char smem[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  unsigned char* smem = align_smem(smem_raw);
   const Group g = make_group(smem, threadIdx.x, 32, apt, ncell_cap, 1, nl);
   switch (apt) {
     case 1: debug_forces_path<1>(g, bd, rp, x4, f4, ew, pairs); break;
@@ -249,7 +251,8 @@ __global__ void __launch_bounds__(kCtaThreads, 1)
     debug_md_kernel(BoxDesc bd, RunParams rp, int apt, int ncell_cap, float4* x4, float4* v4,
                     int steps, double T, int every, double* ep, double* ek, long long* cyc,
                     uint16_t* nl) {
-  extern __shared__ __align__(128) unsigned char smem[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  unsigned char* smem = align_smem(smem_raw);
   const Group g = make_group(smem, threadIdx.x, 32, apt, ncell_cap, 1, nl);
   switch (apt) {
     case 1: debug_md_path<1>(g, bd, rp, x4, v4, steps, T, every, ep, ek, cyc); break;
@@ -312,7 +315,8 @@ __global__ void __launch_bounds__(kCtaThreads, 1)
     debug_force_bench_kernel(BoxDesc bd, RunParams rp, int apt, int ncell_cap, const float4* x4,
                              int passes, int mode, long long* cyc, uint16_t* nl,
                              long long nl_elems) {
-  extern __shared__ __align__(128) unsigned char smem[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  unsigned char* smem = align_smem(smem_raw);
   const Group g = make_group(smem, threadIdx.x, 32, apt, ncell_cap, 1,
                              nl + (long long)blockIdx.x * nl_elems);
   const float4* xb = x4 + (size_t)blockIdx.x * bd.natoms;
@@ -329,9 +333,10 @@ cudaError_t launch_debug_force_bench(const BoxDesc& bd, const RunParams& rp, int
                                      long long* cyc, uint16_t* nl, long long nl_elems,
                                      cudaStream_t st) {
   cudaError_t e = cudaFuncSetAttribute(debug_force_bench_kernel,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                       smem + kSmemAlign);
   if (e != cudaSuccess) return e;
-  debug_force_bench_kernel<<<nbox, kCtaThreads, smem, st>>>(bd, rp, apt, ncell_cap, x4, passes,
+  debug_force_bench_kernel<<<nbox, kCtaThreads, smem + kSmemAlign, st>>>(bd, rp, apt, ncell_cap, x4, passes,
                                                              mode, cyc, nl, nl_elems);
   return cudaGetLastError();
 }
@@ -460,7 +465,9 @@ __global__ void __launch_bounds__(kCtaThreads, 1)
 // dynamic shared memory for the big-box debug kernels: position windows of the
 // whole box when it fits, else all that the device allows
 static int g_debug_big_smem_max = 0;
-static int debug_big_smem(int n) { return std::min(16 * big_cap(n), g_debug_big_smem_max); }
+static int debug_big_smem(int n) {
+  return std::min(16 * big_cap(n) + kSmemAlign, g_debug_big_smem_max);
+}
 
 cudaError_t launch_debug_big_forces(const BoxDesc& bd, const RunParams& rp, unsigned char* scratch,
                                     const float4* x4, float4* f4, double* ew, long long* pairs,
@@ -480,11 +487,14 @@ cudaError_t launch_debug_big_md(const BoxDesc& bd, const RunParams& rp, unsigned
 
 cudaError_t set_debug_attributes(int max_smem) {
   cudaError_t e;
-  e = cudaFuncSetAttribute(debug_lift_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+  e = cudaFuncSetAttribute(debug_lift_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           max_smem + kSmemAlign);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(debug_forces_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+  e = cudaFuncSetAttribute(debug_forces_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           max_smem + kSmemAlign);
   if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(debug_md_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+  e = cudaFuncSetAttribute(debug_md_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           max_smem + kSmemAlign);
   if (e != cudaSuccess) return e;
   // the big-box kernels also hold a static BigShared
   const int big_max = max_smem - (int)sizeof(BigShared);
@@ -500,14 +510,14 @@ cudaError_t set_debug_attributes(int max_smem) {
 cudaError_t launch_debug_lift(const BoxDesc& bd, const RunParams& rp, double T, int apt,
                               int ncell_cap, int smem, float4* x4, float4* v4, double* e_out,
                               uint16_t* nl, cudaStream_t st) {
-  debug_lift_kernel<<<1, kCtaThreads, smem, st>>>(bd, rp, T, apt, ncell_cap, x4, v4, e_out, nl);
+  debug_lift_kernel<<<1, kCtaThreads, smem + kSmemAlign, st>>>(bd, rp, T, apt, ncell_cap, x4, v4, e_out, nl);
   return cudaGetLastError();
 }
 
 cudaError_t launch_debug_forces(const BoxDesc& bd, const RunParams& rp, int apt, int ncell_cap,
                                 int smem, const float4* x4, float4* f4, double* ew,
                                 long long* pairs, uint16_t* nl, cudaStream_t st) {
-  debug_forces_kernel<<<1, kCtaThreads, smem, st>>>(bd, rp, apt, ncell_cap, x4, f4, ew, pairs, nl);
+  debug_forces_kernel<<<1, kCtaThreads, smem + kSmemAlign, st>>>(bd, rp, apt, ncell_cap, x4, f4, ew, pairs, nl);
   return cudaGetLastError();
 }
 
@@ -515,7 +525,7 @@ cudaError_t launch_debug_md(const BoxDesc& bd, const RunParams& rp, int apt, int
                             int smem, float4* x4, float4* v4, int steps, double T, int every,
                             double* ep, double* ek, long long* cyc, uint16_t* nl,
                             cudaStream_t st) {
-  debug_md_kernel<<<1, kCtaThreads, smem, st>>>(bd, rp, apt, ncell_cap, x4, v4, steps, T, every,
+  debug_md_kernel<<<1, kCtaThreads, smem + kSmemAlign, st>>>(bd, rp, apt, ncell_cap, x4, v4, steps, T, every,
                                                 ep, ek, cyc, nl);
   return cudaGetLastError();
 }

@@ -27,7 +27,9 @@ constexpr int kMaxCluster = 8;        // CTAs of a thread-block cluster that sha
 // boxes above kMaxAtoms run one per CTA with their state in global memory
 constexpr int kMaxAtomsBig = 32768;   // uint16 neighbour indices
 constexpr int kMaxCellsBig = 32768;   // cells of the list build (<= 32 per axis)
-constexpr int kBigSharedBytes = 4096; // shared memory of a big-box CTA (reductions only)
+constexpr int kBigSharedBytes = 4096; // shared memory of a big-box CTA: reductions, then
+constexpr int kBigCluBytes = 2 * kMaxCluster * kRedSlots * 8;  // the cluster partials and
+                                                               // the position windows
 
 // Cells per axis of a shared-memory box's Verlet-list build: side at least
 // R / 2 (R = rc + skin), at most 12 per axis; 0 = no cell grid (a scan of all
@@ -152,7 +154,16 @@ constexpr int kAccDoubles = 2 * kMaxSeBlocks + 24;  // block sums of P and T, ru
 //   FP64 accumulators              double[kAccDoubles]
 //   block counts                   int[kMaxSeBlocks]
 //   control words                  int[16]
-//   cluster partials               int64[kMaxCluster][kRedSlots]  (16-B aligned)
+//   cluster partials              int64[kMaxCluster][kRedSlots]  (16-B aligned; only in
+//                                 a thread-block cluster)
+//   list-build rings              2 KB per warp, 1-KB aligned: the force array itself with
+//                                 four atoms per thread (exactly 2 KB of it per warp), else
+//                                 an area of their own behind the rest
+// The group's base is 1-KB aligned: group_smem_bytes is a multiple of it, and kernels align
+// the start of their dynamic shared memory (align_smem), for which every launch adds
+// kSmemAlign bytes.
+constexpr int kSmemAlign = 1024;
+
 __host__ __device__ inline int group_red_offset(int warps, int apt, int ncell_cap) {
   int npad = warps * 32 * apt;
   int b = npad * 48 + (2 * ncell_cap + 2) * 4;
@@ -166,9 +177,20 @@ __host__ __device__ inline int group_cluster_offset(int warps, int apt, int ncel
   return (b + 15) & ~15;
 }
 
-__host__ __device__ inline int group_smem_bytes(int warps, int apt, int ncell_cap) {
+__host__ __device__ inline int group_ring_offset(int warps, int apt, int ncell_cap) {
+  if (apt >= 4) return warps * 32 * apt * 16;  // the force array
   const int b = group_cluster_offset(warps, apt, ncell_cap) + kMaxCluster * kRedSlots * 8;
-  return (b + 127) & ~127;
+  return (b + kSmemAlign - 1) & ~(kSmemAlign - 1);
+}
+
+// `cluster`: with the cluster partials (the rings of fewer than four atoms per thread lie
+// behind them in any case)
+__host__ __device__ inline int group_smem_bytes(int warps, int apt, int ncell_cap,
+                                                bool cluster = false) {
+  const int b = apt < 4 ? group_ring_offset(warps, apt, ncell_cap) + warps * 2048
+                        : group_cluster_offset(warps, apt, ncell_cap) +
+                              (cluster ? kMaxCluster * kRedSlots * 8 : 0);
+  return (b + kSmemAlign - 1) & ~(kSmemAlign - 1);
 }
 
 }  // namespace mdeos

@@ -30,7 +30,8 @@ __global__ void __launch_bounds__(kCtaThreads, 1)
     eos_batch_static_kernel(unsigned char* scratch, long long off_items, long long off_counter,
                             long long off_nl, int nitems, mdeos_result* results,
                             long long nl_elems_per_cta, RunParams rp) {
-  extern __shared__ __align__(128) unsigned char smem[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  unsigned char* smem = align_smem(smem_raw);
   __shared__ int s_item;
   const BoxDesc* boxes = reinterpret_cast<const BoxDesc*>(scratch);
   const WorkItem* items = reinterpret_cast<const WorkItem*>(scratch + off_items);
@@ -105,9 +106,10 @@ extern "C" mdeos_status mdeos_submit_noalloc(const mdeos_config* cfg, const mdeo
                                                 cudaGetErrorString(e));
       cudaDeviceGetAttribute(&d.nsm, cudaDevAttrMultiProcessorCount, dev);
       cudaDeviceGetAttribute(&d.smem_max, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-      d.smem_max -= 1024;
+      d.smem_max -= 2048;  // static shared memory and alignment
       e = cudaFuncSetAttribute(eos_batch_static_kernel,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, d.smem_max);
+                               cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               d.smem_max + kSmemAlign);
       if (e != cudaSuccess)
         return set_error(MDEOS_ECUDA, std::string("kernel attribute: ") +
                                                 cudaGetErrorString(e));
@@ -157,7 +159,7 @@ extern "C" mdeos_status mdeos_submit_noalloc(const mdeos_config* cfg, const mdeo
     // the queue counter keeps the previous call's value: clear it
     if (e == cudaSuccess) e = cudaMemsetAsync(d.ptr + off_counter, 0, sizeof(int), s);
     if (e == cudaSuccess) {
-      eos_batch_static_kernel<<<grid, kCtaThreads, smem, s>>>(
+      eos_batch_static_kernel<<<grid, kCtaThreads, smem + kSmemAlign, s>>>(
           d.ptr, (long long)off_items, (long long)off_counter, (long long)off_nl,
           (int)items.size(), d_results, nl_per_cta, rp);
       e = cudaGetLastError();

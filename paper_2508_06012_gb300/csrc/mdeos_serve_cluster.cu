@@ -52,7 +52,8 @@ constexpr unsigned long long kRoundNs = 100000000ull;  // longest claiming time 
 __global__ void __launch_bounds__(kCtaThreads, 1)
     eos_serve_cluster_kernel(ServeQueue q, RunParams rp, uint16_t* nl_scratch,
                              long long nl_elems_per_cta) {
-  extern __shared__ __align__(128) unsigned char smem[];
+  extern __shared__ __align__(128) unsigned char smem_raw[];
+  unsigned char* smem = align_smem(smem_raw);
   __shared__ int s_slot, s_lslot, s_cmd;
   __shared__ int s_ok[kMaxCluster];
   __shared__ long long s_got[1];
@@ -239,7 +240,7 @@ __global__ void __launch_bounds__(kCtaThreads, 1)
 
 cudaError_t set_serve_cluster_attributes(int max_smem) {
   return cudaFuncSetAttribute(eos_serve_cluster_kernel,
-                              cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem);
+                              cudaFuncAttributeMaxDynamicSharedMemorySize, max_smem + kSmemAlign);
 }
 
 // grid: a multiple of cluster
@@ -249,7 +250,7 @@ cudaError_t launch_eos_serve_cluster(const ServeQueue& q, const RunParams& rp, u
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3((unsigned)grid, 1, 1);
   lc.blockDim = dim3(kCtaThreads, 1, 1);
-  lc.dynamicSmemBytes = (size_t)smem;
+  lc.dynamicSmemBytes = (size_t)smem + kSmemAlign;
   lc.stream = st;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeClusterDimension;
