@@ -127,8 +127,9 @@ struct BigMem {
   bool l2;                   // other CTAs write the box too: read their slots from L2
 };
 
-// Position windows in the dynamic shared memory from offset `off` on: address and
-// capacity (in float4) of what the launch provides, at least 1024 atoms, else none.
+// Position windows in the dynamic shared memory from offset `off` behind its aligned
+// start on: address and capacity (in float4) of what the launch provides (less the
+// alignment), at least 1024 atoms, else none.
 __device__ __forceinline__ void big_pos_cache(BigMem& m, const unsigned char* dyn_base, int off) {
   uint32_t dyn;
   asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
@@ -212,6 +213,159 @@ __device__ inline void big_wrap(const BigMem& m, float L, float invL) {
   }
 }
 
+// List word of a slot (f.w): its entries (bits 0..29), and whether the atom lies within
+// R of a face of the box, so that some of its neighbours are images.
+constexpr int kBigFace = 1 << 30;
+constexpr int kBigCount = kBigFace - 1;
+
+// A home atom's list under construction: the word being assembled (each new entry enters
+// at the top, after eight the first sits in the low half of w0), the entries so far
+struct BigRow {
+  uint32_t w0, w1, w2, w3;
+  int k, maxw, cap;
+  uint4* row;  // the slot's words, cap apart
+};
+
+__device__ __forceinline__ void big_push(BigRow& r, uint32_t e) {
+  r.w0 = __funnelshift_r(r.w0, r.w1, 16);
+  r.w1 = __funnelshift_r(r.w1, r.w2, 16);
+  r.w2 = __funnelshift_r(r.w2, r.w3, 16);
+  r.w3 = __funnelshift_r(r.w3, e, 16);
+  ++r.k;
+  if ((r.k & 7) == 0 && (r.k >> 3) <= r.maxw)
+    r.row[(size_t)((r.k >> 3) - 1) * r.cap] = make_uint4(r.w0, r.w1, r.w2, r.w3);
+}
+
+// One bit per candidate e .. e + cnt - 1 (at most 32), the first at the top: the sign of r^2 -
+// R^2.  Reads up to three positions past the last one (the windows and the state arrays
+// leave room for them).
+template <bool WIN, bool SHIFT>
+__device__ __forceinline__ uint32_t big_tests(const float4* x, uint32_t sx_a, bool l2, int e, int cnt,
+                                              const float4& xi, float sx, float sy, float sz,
+                                              float rs2) {
+  uint32_t m = 0u;
+  int done = 0;
+#pragma unroll 1
+  for (; done < cnt; done += 4) {
+    float4 xj[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      xj[q] = WIN ? ld_shared4(sx_a + 16u * (uint32_t)(e + done + q)) : big_ld4(x + e + done + q, l2);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const float dx = xi.x - (SHIFT ? xj[q].x + sx : xj[q].x);
+      const float dy = xi.y - (SHIFT ? xj[q].y + sy : xj[q].y);
+      const float dz = xi.z - (SHIFT ? xj[q].z + sz : xj[q].z);
+      const float r2 = fmaf(dx, dx, fmaf(dy, dy, dz * dz));
+      m = __funnelshift_l(__float_as_uint(r2 - rs2), m, 1);
+    }
+  }
+  return cnt > 0 ? (m << (32 - done)) & (0xffffffffu << (32 - cnt)) : 0u;
+}
+
+// Candidates e0 .. e1 - 1 (window indices, or slots without a window), their positions
+// shifted by (sx, sy, sz): 64 tests at a time, then the set bits are pushed in order.  The
+// lanes of a warp are atoms of one to three cells and walk nearly the same candidates; one
+// in eight is pushed.
+template <bool WIN, bool SHIFT>
+__device__ __forceinline__ void big_scan(const float4* x, uint32_t sx_a, bool l2, BigRow& r, int e0,
+                                         int e1, const float4& xi, float sx, float sy, float sz,
+                                         float rs2) {
+#pragma unroll 1
+  for (int e = e0; e < e1; e += 64) {
+    uint32_t m = big_tests<WIN, SHIFT>(x, sx_a, l2, e, min(32, e1 - e), xi, sx, sy, sz, rs2);
+    uint32_t m2 = big_tests<WIN, SHIFT>(x, sx_a, l2, e + 32, min(32, e1 - e - 32), xi, sx, sy, sz, rs2);
+    int at = e;
+    if (m == 0u) {
+      m = m2;
+      m2 = 0u;
+      at = e + 32;
+    }
+    while (m != 0u) {
+      const int t = __clz(m);
+      m &= ~(0x80000000u >> t);
+      big_push(r, (uint32_t)(at + t));
+      if (m == 0u) {
+        m = m2;
+        m2 = 0u;
+        at = e + 32;
+      }
+    }
+  }
+}
+
+// Lists of slots sb .. se - 1 (the caller's own, one round): a home atom's 27 cells are
+// nine rows of three x-adjacent cells, whose slots are contiguous (also in the window: its
+// cyclic seam falls on a layer boundary); at an x face the cell across it is a part of its
+// own.  A row or slot outside its window (impossible by construction) fails the box without
+// any read.  Returns whether a list overflowed or a row lay outside.  Out of line and fed
+// scalars; the last word of a list is completed with the atom itself.
+template <bool WIN>
+static __device__ __noinline__ bool big_search(const float4* x, uint32_t sx_a, const int* start,
+                                               float4* f, uint4* nl, int cap, int n, int nc, int wl,
+                                               int ws, int sb, int se, float L, float cinv,
+                                               float rs2, int maxnb, bool l2) {
+  const float margin = 1.0001f * sqrtf(rs2);
+  bool fail = false;
+#pragma unroll 1
+  for (int s = sb + (int)threadIdx.x; s < se; s += (int)blockDim.x) {
+    int si = s - wl;
+    if (si < 0) si += n;
+    if (si >= ws) {
+      fail = true;
+      f[s].w = __int_as_float(0);
+      continue;
+    }
+    const float4 xi = WIN ? ld_shared4(sx_a + 16u * (uint32_t)si) : x[s];
+    const int cx = min((int)(xi.x * cinv), nc - 1);
+    const int cy = min((int)(xi.y * cinv), nc - 1);
+    const int cz = min((int)(xi.z * cinv), nc - 1);
+    BigRow r = {0u, 0u, 0u, 0u, 0, maxnb >> 3, cap, nl + s};
+#pragma unroll 1
+    for (int d = 0; d < 9; ++d) {
+      const int dz = d / 3 - 1, dy = d % 3 - 1;
+      int zz = cz + dz, yy = cy + dy;
+      float sy = 0.f, sz = 0.f;
+      if (zz < 0) { zz += nc; sz = -L; } else if (zz >= nc) { zz -= nc; sz = L; }
+      if (yy < 0) { yy += nc; sy = -L; } else if (yy >= nc) { yy -= nc; sy = L; }
+      const int* row = start + (zz * nc + yy) * nc;
+      // parts in x order: the cell across the lower face, the row (up to the atom itself,
+      // then past it, in its own), the cell across the upper face
+      const int lo = max(cx - 1, 0), hi = min(cx + 2, nc);
+#pragma unroll 1
+      for (int part = 0; part < 4; ++part) {
+        if ((part == 0 && cx > 0) || (part == 3 && cx < nc - 1)) continue;
+        if (part == 2 && d != 4) continue;
+        const int c0 = part == 0 ? nc - 1 : (part == 3 ? 0 : lo);
+        const int c1 = part == 0 ? nc : (part == 3 ? 1 : hi);
+        const int j0 = big_ldi(row + c0, l2), j1 = big_ldi(row + c1, l2);
+        int e0 = j0 - wl;  // window index of the part's first slot
+        if (e0 < 0) e0 += n;
+        int e1 = e0 + (j1 - j0);
+        if (e1 > ws) {
+          fail = true;
+          continue;
+        }
+        if (d == 4 && part == 1) e1 = si;
+        if (part == 2) e0 = si + 1;
+        const float sx = part == 0 ? -L : (part == 3 ? L : 0.f);
+        if (__any_sync(__activemask(), sx != 0.f || sy != 0.f || sz != 0.f))
+          big_scan<WIN, true>(x, sx_a, l2, r, e0, e1, xi, sx, sy, sz, rs2);
+        else
+          big_scan<WIN, false>(x, sx_a, l2, r, e0, e1, xi, 0.f, 0.f, 0.f, rs2);
+      }
+    }
+    const int k = r.k;
+    while (r.k & 7) big_push(r, (uint32_t)si);
+    fail = fail || k > maxnb;
+    // atoms within R of a face have neighbours across it
+    const bool face = fminf(fminf(xi.x, xi.y), xi.z) < margin ||
+                      fmaxf(fmaxf(xi.x, xi.y), xi.z) > L - margin;
+    f[s].w = __int_as_float(min(k, maxnb) | (face ? kBigFace : 0));
+  }
+  return fail;
+}
+
 // Verlet list from wrapped positions: counting sort into cell order (inside a
 // cell by previous slot: deterministic), permutation of x and v into the second
 // buffers (then swapped), 27-cell search with one image shift per cell.  In a
@@ -272,23 +426,19 @@ static __device__ bool big_build(BigMem& m, BigShared* sh, BigClu& cl, int n, in
     reinterpret_cast<float*>(m.x2 + s)[3] = __int_as_float(i);
   }
   big_bar(cl);
-  for (int c = gt; c < ncell; c += gn) {  // insertion sort of the previous slots
+  // order inside a cell: an atom's place is the number of the cell's atoms with a smaller
+  // previous slot (independent loads, where an insertion sort per cell is a chain of them)
+  for (int i = m.lo + tid; i < m.hi; i += nt) {
+    const int c = __float_as_int(m.f[i].x);
     const int lo = big_ldi(m.start + c, l2), hi = big_ldi(m.start + c + 1, l2);
-    for (int a = lo + 1; a < hi; ++a) {
-      const float key = big_ldw(m.x2 + a, l2);
-      const int kk = __float_as_int(key);
-      int b = a - 1;
-      float wb;
-      while (b >= lo && __float_as_int(wb = big_ldw(m.x2 + b, l2)) > kk) {
-        reinterpret_cast<float*>(m.x2 + b + 1)[3] = wb;
-        --b;
-      }
-      reinterpret_cast<float*>(m.x2 + b + 1)[3] = key;
-    }
+    int r = lo;
+#pragma unroll 4
+    for (int t = lo; t < hi; ++t) r += __float_as_int(big_ldw(m.x2 + t, l2)) < i ? 1 : 0;
+    reinterpret_cast<float*>(m.v2 + r)[3] = __int_as_float(i);
   }
   big_bar(cl);
   for (int s = m.lo + tid; s < m.hi; s += nt) {
-    const int i = __float_as_int(big_ldw(m.x2 + s, l2));
+    const int i = __float_as_int(big_ldw(m.v2 + s, l2));
     m.x2[s] = big_ld4(m.x + i, l2);
     const float4 vi = big_ld4(m.v + i, l2);
     m.v2[s] = make_float4(vi.x, vi.y, vi.z, 0.f);
@@ -329,7 +479,7 @@ static __device__ bool big_build(BigMem& m, BigShared* sh, BigClu& cl, int n, in
             const int hi = big_ldi(m.start + (hz + 1) * nc2, l2);
             sz = lz <= hz ? hi - lo : (n - lo) + hi;
           }
-          fits = sz <= m.sx_cap;
+          fits = sz + 4 <= m.sx_cap;  // the search reads past a row's end
           sh->wlo[q] = lo;
           sh->wsz[q] = sz;
         }
@@ -346,12 +496,7 @@ static __device__ bool big_build(BigMem& m, BigShared* sh, BigClu& cl, int n, in
   m.rsz = sh->rsz;
   m.wlo = sh->wlo;
   m.wsz = sh->wsz;
-  uint16_t* row = reinterpret_cast<uint16_t*>(m.nl);
-  const size_t wstride = (size_t)m.cap * 8;  // uint16 entries between words of one slot
-  // The search runs in the same rounds, candidates read from the round's window: a
-  // cell's slots are contiguous in the window (the window's cyclic seam falls on a
-  // cell boundary), so one offset per cell maps them.  A cell or slot outside its
-  // window (impossible by construction) fails the box without any read.
+  // the search runs in the same rounds, candidates read from the round's window
   const bool win = m.nround > 0;
   for (int q = 0; q < (win ? m.nround : 1); ++q) {
     const int wl = win ? m.wlo[q] : 0, ws = win ? m.wsz[q] : n;
@@ -365,55 +510,11 @@ static __device__ bool big_build(BigMem& m, BigShared* sh, BigClu& cl, int n, in
       }
       __syncthreads();
     }
-    for (int s = sb + tid; s < se; s += nt) {
-      int si = s - wl;
-      if (si < 0) si += n;
-      if (si >= ws) {
-        atomicOr(&sh->ctrl[CTRL_OVERFLOW], 1);
-        m.f[s].w = __int_as_float(0);
-        continue;
-      }
-      const float4 xi = win ? ld_shared4(m.sx_a + 16u * (uint32_t)si) : m.x[s];
-      const int cx = min((int)(xi.x * cinv), nc - 1);
-      const int cy = min((int)(xi.y * cinv), nc - 1);
-      const int cz = min((int)(xi.z * cinv), nc - 1);
-      int k = 0;
-      for (int dz = -1; dz <= 1; ++dz) {
-        int zz = cz + dz;
-        float sz = 0.f;
-        if (zz < 0) { zz += nc; sz = -L; } else if (zz >= nc) { zz -= nc; sz = L; }
-        for (int dy = -1; dy <= 1; ++dy) {
-          int yy = cy + dy;
-          float sy = 0.f;
-          if (yy < 0) { yy += nc; sy = -L; } else if (yy >= nc) { yy -= nc; sy = L; }
-          for (int dx = -1; dx <= 1; ++dx) {
-            int xx = cx + dx;
-            float sx_ = 0.f;
-            if (xx < 0) { xx += nc; sx_ = -L; } else if (xx >= nc) { xx -= nc; sx_ = L; }
-            const int c = (zz * nc + yy) * nc + xx;
-            const int j0 = big_ldi(m.start + c, l2), j1 = big_ldi(m.start + c + 1, l2);
-            int jb = j0 - wl;  // window index of the cell's first slot
-            if (jb < 0) jb += n;
-            if (jb + (j1 - j0) > ws) {
-              atomicOr(&sh->ctrl[CTRL_OVERFLOW], 1);
-              continue;
-            }
-            for (int j = j0; j < j1; ++j) {
-              const int e = jb + (j - j0);  // window-relative slot (= j without windows)
-              const float4 xj = win ? ld_shared4(m.sx_a + 16u * (uint32_t)e) : big_ld4(m.x + j, l2);
-              const float ddx = xi.x - (xj.x + sx_), ddy = xi.y - (xj.y + sy), ddz = xi.z - (xj.z + sz);
-              const float r2 = fmaf(ddx, ddx, fmaf(ddy, ddy, ddz * ddz));
-              if (j != s && r2 < rs2) {
-                if (k < maxnb) row[(size_t)(k >> 3) * wstride + (size_t)s * 8 + (k & 7)] = (uint16_t)e;
-                ++k;
-              }
-            }
-          }
-        }
-      }
-      if (k > maxnb) atomicOr(&sh->ctrl[CTRL_OVERFLOW], 1);
-      m.f[s].w = __int_as_float(min(k, maxnb));
-    }
+    const bool fail = win ? big_search<true>(m.x, m.sx_a, m.start, m.f, m.nl, m.cap, n, nc, wl, ws,
+                                             sb, se, L, cinv, rs2, maxnb, l2)
+                          : big_search<false>(m.x, 0u, m.start, m.f, m.nl, m.cap, n, nc, wl, ws,
+                                              sb, se, L, cinv, rs2, maxnb, l2);
+    if (fail) atomicOr(&sh->ctrl[CTRL_OVERFLOW], 1);
     if (win) __syncthreads();  // before the next window overwrites this one
   }
   __syncthreads();
@@ -433,10 +534,16 @@ static __device__ bool big_build(BigMem& m, BigShared* sh, BigClu& cl, int n, in
 // SM: slots [s0, s1) of one round, positions from the round's window in shared
 // memory (slot wl at index 0, cyclic over the n slots; list entries are window
 // indices).  Otherwise all slots, positions and list entries as global slots.
+//
+// Atoms away from the faces have no images among their neighbours (list word); a warp
+// without any takes plain differences, which is what the minimum image gives for them, in
+// nine instructions fewer per pair.  List words are padded with the atom itself, masked by
+// index.
 template <bool EN, bool VIR, bool CNT, bool SM>
 __device__ __noinline__ FSums big_force_pass(const float4* x, uint32_t sx_a, int s0, int s1,
                                              int wl, float4* f, const uint4* nl, int cap, int n,
                                              float L, float invL, bool l2, LJ c) {
+  constexpr int kPairGroup = EN ? 4 : 8;  // as in force_pass
   unsigned long long es = 0, ws[6] = {0, 0, 0, 0, 0, 0};
   int np = 0, bad = 0;
 #pragma unroll 1
@@ -450,27 +557,40 @@ __device__ __noinline__ FSums big_force_pass(const float4* x, uint32_t sx_a, int
     }
     const float4 xi = SM ? ld_shared4(sx_a + 16u * (uint32_t)si) : x[s];
     const float cw = f[s].w;
-    const int cn = __float_as_int(cw);
-    const int nw = (cn + 7) >> 3;
+    const int nw = ((__float_as_int(cw) & kBigCount) + 7) >> 3;
     float fx = 0.f, fy = 0.f, fz = 0.f;
     const uint4* p = nl + s;
     uint4 q = nw > 0 ? __ldcg(p) : make_uint4(0u, 0u, 0u, 0u);
+    const bool face = __any_sync(__activemask(), (__float_as_int(cw) & kBigFace) != 0);
+    if (face) {
 #pragma unroll 1
-    for (int kb = 0; kb < nw; ++kb) {
-      const uint4 cur = q;
-      if (kb + 1 < nw) q = __ldcg(p + (size_t)(kb + 1) * cap);
-      const int left = cn - (kb << 3);
+      for (int kb = 0; kb < nw; ++kb) {
+        const uint4 cur = q;
+        if (kb + 1 < nw) q = __ldcg(p + (size_t)(kb + 1) * cap);
 #pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const unsigned wd = u < 2 ? cur.x : (u < 4 ? cur.y : (u < 6 ? cur.z : cur.w));
-        const int jj = (int)((wd >> (16 * (u & 1))) & 0xffffu);
-        const bool ok = u < left;
-        const int jr = ok ? jj : si;
-        const float4 xj = SM ? ld_shared4(sx_a + 16u * (uint32_t)jr) : big_ld4(x + jr, l2);
-        const float dx = min_img(xi.x - xj.x, L, invL);
-        const float dy = min_img(xi.y - xj.y, L, invL);
-        const float dz = min_img(xi.z - xj.z, L, invL);
-        lj_pair<EN, VIR>(dx, dy, dz, ok, c, fx, fy, fz, e, w, np);
+        for (int g = 0; g < 8; g += kPairGroup)
+          pair_group<kPairGroup, EN, VIR, true>(
+              [&](int q) {
+                const int j = word_entry(cur, g + q);
+                return SM ? ld_shared4(sx_a + 16u * (uint32_t)j) : big_ld4(x + j, l2);
+              },
+              [&](int q) { return word_entry(cur, g + q) != si; }, xi.x, xi.y, xi.z, L, invL, c, fx,
+              fy, fz, e, w, np);
+      }
+    } else {
+#pragma unroll 1
+      for (int kb = 0; kb < nw; ++kb) {
+        const uint4 cur = q;
+        if (kb + 1 < nw) q = __ldcg(p + (size_t)(kb + 1) * cap);
+#pragma unroll
+        for (int g = 0; g < 8; g += kPairGroup)
+          pair_group<kPairGroup, EN, VIR, false>(
+              [&](int q) {
+                const int j = word_entry(cur, g + q);
+                return SM ? ld_shared4(sx_a + 16u * (uint32_t)j) : big_ld4(x + j, l2);
+              },
+              [&](int q) { return word_entry(cur, g + q) != si; }, xi.x, xi.y, xi.z, L, invL, c, fx,
+              fy, fz, e, w, np);
       }
     }
     f[s] = make_float4(fx, fy, fz, cw);
@@ -729,7 +849,7 @@ static __device__ __noinline__ void run_big(unsigned char* scratch, BigShared* s
         kt[3] += (unsigned long long)fxp(rp.mass_f * vi.x * vi.y);
         kt[4] += (unsigned long long)fxp(rp.mass_f * vi.x * vi.z);
         kt[5] += (unsigned long long)fxp(rp.mass_f * vi.y * vi.z);
-        cand += __float_as_int(fi.w);
+        cand += __float_as_int(fi.w) & kBigCount;
       }
     }
     {
@@ -751,7 +871,7 @@ static __device__ __noinline__ void run_big(unsigned char* scratch, BigShared* s
           const long long sk = warp_sum_ll((long long)(kt[k] + wv[k]));
           if (lane == 0) red[k] = sk;
         }
-        const long long sp = warp_sum_ll(r.np), sc = warp_sum_ll(cand);
+        const long long sp = warp_sum_i(r.np), sc = warp_sum_i(cand);
         if (lane == 0) {
           red[8] = sp;
           red[9] = sc;
