@@ -88,8 +88,9 @@ typedef struct {
                                   rho = 0.9 if higher, + 32).  A box whose list overflows is
                                   re-run by mdeos_poll with twice the capacity. */
   int32_t max_cluster;         /* CTAs per box for batches of few boxes (thread-block
-                                  clusters, see mdeos_submit): 0 = up to 4, at most 8,
-                                  1 = none */
+                                  clusters, see mdeos_submit): at most 8, 1 = none; 0 = up
+                                  to 8, but 4 if a box has at most 768 atoms, or above
+                                  4096 atoms fewer than 16000 */
 } mdeos_config;
 
 /* One EOS query.  Layout is part of the ABI. */
@@ -146,10 +147,10 @@ mdeos_status mdeos_create(const mdeos_config* cfg, mdeos_handle** out);
  * persistent kernel launch; per-box problems are reported in the results.
  * Launch shape: a batch that fills the GPU packs boxes into work items of one
  * CTA; one with no more boxes than SMs gives each box its own CTA; one with fewer
- * boxes than half the SMs, all of at most 768 atoms, runs each box on a
- * thread-block cluster of up to cfg.max_cluster CTAs (each holds the box and computes
- * the forces of its share of the atoms); one with fewer boxes than half the SMs, all
- * above 4096 atoms, does the same with one state per box in global memory (each CTA
+ * boxes than half the SMs, all of at most 4096 atoms, runs each box on a thread-block
+ * cluster of up to cfg.max_cluster CTAs (each holds the box and builds the lists and
+ * computes the forces of its share of the atoms); one with fewer boxes than half the SMs,
+ * all above 4096 atoms, does the same with one state per box in global memory (each CTA
  * owns a slab of the cell-ordered atoms).  Results do not depend on the launch shape.
  * Errors: MDEOS_EINVAL (n < 1, NULL, or a request field out of range),
  * MDEOS_ENOMEM, MDEOS_ECUDA. */

@@ -25,6 +25,7 @@ cudaError_t launch_eos_batch(const BoxDesc* boxes, const WorkItem* items, int ni
                              mdeos_result* results, uint16_t* nl, long long nl_elems_per_cta,
                              const RunParams& rp, int grid, int smem, cudaStream_t st,
                              int* ready, int cluster, int threads = kCtaThreads);
+cudaError_t max_resident_clusters(int cluster, int smem, int* n);
 cudaError_t set_debug_attributes(int max_smem);
 cudaError_t launch_debug_lift(const BoxDesc& bd, const RunParams& rp, double T, int apt,
                               int ncell_cap, int smem, float4* x4, float4* v4, double* e_out,
@@ -320,7 +321,7 @@ struct Plan {
 static mdeos_status make_plan(const mdeos_request* reqs, int n, const mdeos_config& c, int nsm,
                               int smem_max, Plan& plan, bool allow_big = true,
                               const ShapeTable* tuned = nullptr, const int* cap_min = nullptr,
-                              bool allow_cluster = false) {
+                              bool allow_cluster = false, const int* fit = nullptr) {
   plan.boxes.clear();
   plan.items.clear();
   plan.status.assign(n, MDEOS_OK);
@@ -345,33 +346,55 @@ static mdeos_status make_plan(const mdeos_request* reqs, int n, const mdeos_conf
       p.apt = q.apt;
     }
   }
-  // Fewer boxes than half the SMs, all searched without cells: a thread-block
-  // cluster of up to kMaxCluster CTAs per box (the whole CTA as its group), the
-  // largest power of two that keeps every box's cluster on the GPU at once
+  // Few shared-memory boxes (spread): a thread-block cluster of C CTAs per box, C the
+  // largest power of two whose clusters are all on the GPU at once.  A cluster's CTAs
+  // share a GPC, so that number is the GPU's own answer for one CTA per SM (fit[C]), not
+  // an SM count: 16 boxes on clusters of 8 ran in two waves (338 EOS/s against 611 on 4).
+  // One box of 4000 atoms: 226k SM cycles a step on one CTA, 137k on 2, 75k on 8.  Boxes
+  // searched without cells stay at 4 by default: an 8th of one is 32-96 atoms, less than
+  // the exchange costs (500 atoms: 40k cycles a step on 4 and on 8).  Boxes that scan all
+  // pairs have no list to share.  The CTA has two atoms per thread, or a thread per list
+  // unit of its share if that is more: a warp without atoms still runs every step's sums
+  // (16 x 256 atoms: 13.2 us a step with 32 warps, 11.4 with the 8 that hold atoms, 8.1
+  // with their lists fetched further ahead as well).
   plan.cluster = 1;
-  // default up to 4: clusters of 8 CTAs did not all fit on the GPU at once (16 boxes:
-  // 338 EOS/s against 611 with 4 and 583 with none)
-  const int cmax = c.max_cluster > 0 ? std::min(c.max_cluster, kMaxCluster) : 4;
+  const int cmax = c.max_cluster > 0 ? std::min(c.max_cluster, kMaxCluster) : 0;
+  const auto fits = [&](int C, int boxes) { return fit != nullptr && boxes <= fit[C]; };
   if (allow_cluster && spread && (int)bp.size() == nsmall) {
-    bool all = true;
-    for (const BoxPlan& p : bp) all = all && p.bd.path == PATH_NLIST && p.bd.nc_cell == 0;
+    bool brute = false, list = false;
+    for (const BoxPlan& p : bp) {
+      brute = brute || p.bd.natoms <= kBruteMaxAtoms;
+      list = list || p.bd.path == PATH_NLIST;
+    }
+    const int top = cmax > 0 ? cmax : (brute ? 4 : kMaxCluster);
     int C = 1;
-    while (2 * C <= cmax && 2LL * C * nsmall <= nsm) C *= 2;
-    if (all && C > 1) {
+    while (list && 2 * C <= top && 2LL * C * nsmall <= nsm && fits(2 * C, nsmall)) C *= 2;
+    if (C > 1) {
       plan.cluster = C;
+      int warps = 4;
+      for (const BoxPlan& p : bp) {
+        const int n = p.bd.natoms, share = (n + C - 1) / C;
+        const int tpa = (p.bd.path == PATH_NLIST && p.bd.nc_cell == 0) ? brute_tpa(n) : 1;
+        warps = std::max(warps, pow2_ceil(std::min(32, std::max((n + 63) / 64,
+                                                                (share * tpa + 31) / 32))));
+      }
+      plan.threads = warps * 32;
       for (BoxPlan& p : bp) {
-        p.warps = kCtaThreads / 32;
-        p.apt = round_apt((p.bd.natoms + kCtaThreads - 1) / kCtaThreads);
+        p.warps = warps;
+        p.apt = round_apt((p.bd.natoms + plan.threads - 1) / plan.threads);
       }
     }
   }
-  // Only boxes above the shared-memory limit, fewer than half the SMs: each on a
-  // cluster of CTAs sharing its global-memory state (a slab of slots per CTA), the
-  // same cluster size rule
+  // Only boxes above the shared-memory limit, fewer than half the SMs: each on a cluster
+  // of CTAs sharing its global-memory state (a slab of slots per CTA); by default up to
+  // 4, and 8 where a slab keeps 2000 atoms (32000 atoms: 0.62 s on 4, 0.34 s on 8)
   const int nbig = (int)bp.size() - nsmall;
   if (allow_cluster && nsmall == 0 && nbig > 0) {
+    int nmin = kMaxAtomsBig;
+    for (const BoxPlan& p : bp) nmin = std::min(nmin, p.bd.natoms);
+    const int top = cmax > 0 ? cmax : (nmin >= 2000 * kMaxCluster ? kMaxCluster : 4);
     int C = 1;
-    while (2 * C <= cmax && 2LL * (2 * C) * nbig <= nsm) C *= 2;
+    while (2 * C <= top && 2LL * (2 * C) * nbig <= nsm && fits(2 * C, nbig)) C *= 2;
     if (C > 1) plan.cluster = C;
   }
   // size classes by (warps, apt); inside a class, sort by cost so an item's
@@ -534,6 +557,7 @@ struct mdeos_handle {
   PinnedBlockPtr eval_pinned;
   RunParams rp;
   int device = 0, nsm = 0, smem_max = 0;
+  int fit[kMaxCluster + 1] = {0};  // clusters of 2, 4, 8 full-size CTAs resident at once
   cudaStream_t stream = nullptr;
   bool own_stream = false;
   uint16_t* d_nl = nullptr;
@@ -602,6 +626,26 @@ static mdeos_status ensure_scratch(mdeos_handle* h, size_t bytes) {
   return MDEOS_OK;
 }
 
+// Plan a batch of handle h for a launch that takes `extra` more device bytes (own_scratch:
+// and its list scratch from them rather than from the handle).  A cluster plan keeps a list
+// scratch per CTA, several per box: where the HBM budget has no room for that, one CTA per
+// box.
+static mdeos_status plan_for_handle(mdeos_handle* h, const mdeos_request* reqs, int n, Plan& plan,
+                                    size_t extra, bool own_scratch, const int* cap_min = nullptr) {
+  mdeos_status st = make_plan(reqs, n, h->cfg, h->nsm, h->smem_max, plan, true, &h->tuned_skin,
+                              cap_min, true, h->fit);
+  if (st != MDEOS_OK || plan.cluster == 1 || h->cfg.hbm_budget_bytes == 0) return st;
+  const size_t need = (size_t)plan.grid * plan.nl_per_cta * sizeof(uint16_t);
+  const size_t held = own_scratch ? 0 : h->nl_bytes;
+  if (h->used_bytes + extra + (need > held ? need - held : 0) <= h->cfg.hbm_budget_bytes) return st;
+  return make_plan(reqs, n, h->cfg, h->nsm, h->smem_max, plan, true, &h->tuned_skin, cap_min);
+}
+
+// upper bound of a batch's boxes, items, results and counter
+static size_t table_bytes(int n) {
+  return (size_t)n * (sizeof(BoxDesc) + sizeof(WorkItem) + sizeof(mdeos_result)) + 2048;
+}
+
 extern "C" mdeos_status mdeos_create(const mdeos_config* cfg, mdeos_handle** out) {
   if (!out) return fail(MDEOS_EINVAL, "out is NULL");
   *out = nullptr;
@@ -629,6 +673,8 @@ extern "C" mdeos_status mdeos_create(const mdeos_config* cfg, mdeos_handle** out
   h->smem_max -= 2048 + kSmemAlign;
   e = set_batch_attributes(h->smem_max);
   if (e == cudaSuccess) e = set_debug_attributes(h->smem_max);
+  for (int C = 2; e == cudaSuccess && C <= kMaxCluster; C *= 2)
+    e = max_resident_clusters(C, h->smem_max, &h->fit[C]);
   if (e != cudaSuccess) {
     delete h;
     return cuda_fail(e, "kernel attributes (is this an sm_103 GPU?)");
@@ -737,8 +783,7 @@ extern "C" mdeos_status mdeos_submit(mdeos_handle* h, const mdeos_request* reqs,
   std::lock_guard<std::mutex> lock(h->mu);
   CK(cudaSetDevice(h->device));
   Plan plan;
-  mdeos_status st =
-      make_plan(reqs, n, h->cfg, h->nsm, h->smem_max, plan, true, &h->tuned_skin, nullptr, true);
+  mdeos_status st = plan_for_handle(h, reqs, n, plan, table_bytes(n), false);
   if (st != MDEOS_OK) return st;
   assign_warm(h, plan, reqs);
   TicketState t;
@@ -864,8 +909,7 @@ static void rerun_overflowed(mdeos_handle* h, TicketState& t, mdeos_result* res)
       cmin[k] = 2 * cap[idx[k]];
     }
     Plan plan;
-    if (make_plan(sub.data(), m, h->cfg, h->nsm, h->smem_max, plan, true, &h->tuned_skin,
-                  cmin.data(), true) != MDEOS_OK)
+    if (plan_for_handle(h, sub.data(), m, plan, table_bytes(m), false, cmin.data()) != MDEOS_OK)
       return;
     for (BoxDesc& bd : plan.boxes) {  // same warm slot and stored box side as the first plan
       const BoxDesc& first = t.planned[idx[bd.out_index]];
@@ -948,8 +992,7 @@ extern "C" mdeos_status mdeos_batch_create(mdeos_handle* h, const mdeos_request*
   mdeos_batch* b = new mdeos_batch();
   b->h = h;
   b->n = n;
-  mdeos_status st = make_plan(reqs, n, h->cfg, h->nsm, h->smem_max, b->plan, true,
-                              &h->tuned_skin, nullptr, true);
+  mdeos_status st = plan_for_handle(h, reqs, n, b->plan, table_bytes(n), true);
   if (st != MDEOS_OK) {
     delete b;
     return st;
@@ -1282,8 +1325,7 @@ mdeos_status eval_into_device(mdeos_handle* h, const mdeos_request* reqs, int n,
   CK(cudaSetDevice(h->device));
   CK(cudaStreamSynchronize(h->stream));
   Plan plan;
-  mdeos_status st =
-      make_plan(reqs, n, h->cfg, h->nsm, h->smem_max, plan, true, &h->tuned_skin, nullptr, true);
+  mdeos_status st = plan_for_handle(h, reqs, n, plan, table_bytes(n), false);
   if (st != MDEOS_OK) return st;
   assign_warm(h, plan, reqs);
   const size_t nb = plan.boxes.size(), ni = plan.items.size();

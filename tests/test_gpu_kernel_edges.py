@@ -90,6 +90,34 @@ def test_list_holds_every_neighbour_once(m, n, rho):
     assert bool((err <= 16 * 2.0 ** -24 * mag + 1e-5 * fr.norm(dim=1)).all())
 
 
+@pytest.mark.parametrize("n", [769, 1000, 1372, 2500, 4096])
+def test_cell_boxes_on_clusters_equal_one_cta(m, n):
+    reqs = [dict(rho=0.35 + 0.4 * k, e=m.e_from_temperature(1.2 + 0.3 * k, n), natoms=n - k,
+                 steps_equil=40, steps_avg=40, seed=n + k) for k in range(2)]
+    with m.Engine(max_cluster=1) as e:
+        ref = e.evaluate(reqs)
+    assert (ref["status"] == 0).all() and (ref["nlist_builds"] > 2).all()
+    for c in (0, 2, 4, 8):
+        with m.Engine(max_cluster=c) as e:
+            assert e.evaluate(reqs).tobytes() == ref.tobytes(), c
+    # a list overflow on a cluster, against the same on one CTA
+    with m.Engine(nlist_capacity=16) as a, m.Engine(nlist_capacity=16, max_cluster=1) as b:
+        ra, rb = a.evaluate(reqs), b.evaluate(reqs)
+    assert (ra["nlist_retries"] > 0).all() and ra.tobytes() == rb.tobytes()
+
+
+def test_mixed_small_batch_on_clusters(m):
+    sizes = [108, 256, 500, 864, 4000]
+    reqs = [dict(rho=0.7, e=m.e_from_temperature(1.5, n), natoms=n, steps_equil=30, steps_avg=30,
+                 seed=9 + n, element_id=n) for n in sizes]
+    cfg = dict(warm_slots=8, warm_atoms=4096)
+    with m.Engine(**cfg) as a, m.Engine(max_cluster=1, **cfg) as b:
+        for _ in range(2):   # cold, then warm
+            ra, rb = a.evaluate(reqs), b.evaluate(reqs)
+            assert (ra["status"] == 0).all() and ra.tobytes() == rb.tobytes()
+        assert (ra["warm"] == 1).all()
+
+
 # slabs of one CTA, cluster sizes 1 to 16 and their edges, more zones per CTA than threads,
 # and a mesh whose slabs do not fit (the one-CTA kernel)
 @pytest.mark.parametrize("nz", [1, 3, 63, 64, 65, 127, 1023, 1025, 20011, 40000])
@@ -168,3 +196,17 @@ def test_inference_groups_give_the_same_outputs(m, h, n):
     assert np.array_equal(pm[:, k], pm1) and np.array_equal(mean[k], mean1)
     assert np.array_equal(sd[k], sd1)
 
+
+def test_cluster_scratch_stays_within_the_budget(m):
+    """A budget with room for one CTA's list scratch but not for a cluster's still takes the
+    box (on one CTA), with the same answer."""
+    q = [dict(rho=0.8, e=m.e_from_temperature(1.5, 4000), natoms=4000, steps_equil=20, steps_avg=20,
+              seed=5)]
+    budget = 4 << 20
+    with m.Engine() as a, m.Engine(hbm_budget_bytes=budget) as b:
+        ra, rb = a.evaluate(q), b.evaluate(q)
+        assert m.mdeos_stats(a.h)["device_bytes"] > budget >= m.mdeos_stats(b.h)["device_bytes"]
+        batch = m.mdeos_batch_create(b.h, q)
+        assert m.mdeos_batch_info(batch)["ctas"] == 1
+        m.mdeos_batch_destroy(batch)
+    assert ra["status"][0] == 0 and ra.tobytes() == rb.tobytes()
