@@ -1020,11 +1020,19 @@ __global__ void __launch_bounds__(kTcRows) bf16_gemm_tc_kernel(GemmArgs g, int* 
     float* C = g.S > 1 ? g.ws + ((long long)sk * g.Z + z) * g.M * g.N
                        : (two ? g.C2 : g.C) + (long long)zi * g.sc_z;
     const long long cm = g.S > 1 ? g.N : g.sc_m, cn = g.S > 1 ? 1 : g.sc_n;
+    // rows of C in aligned fours: 16-byte stores (a lane owns a row, so each store of a warp
+    // touches 32 sectors either way)
+    const bool vec = cn == 1 && (cm & 3) == 0 && ((uintptr_t)C & 15) == 0;
 #pragma unroll 1
     for (int c0 = 0; c0 < kH; c0 += 32) {
       float v[32];
       tc_ld32(tl + (uint32_t)c0, v);  // every lane of the warp, in or out of the matrix
-      if (m < g.M)
+      if (m < g.M && vec && n0 + c0 + 32 <= g.N) {
+        float4* row = reinterpret_cast<float4*>(C + (long long)m * cm + n0 + c0);
+#pragma unroll
+        for (int j = 0; j < 8; ++j)
+          row[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+      } else if (m < g.M)
 #pragma unroll
         for (int j = 0; j < 32; ++j) {
           const int n = n0 + c0 + j;
