@@ -471,7 +471,10 @@ struct ListReader {
 // selects of the branch-free form only add to it (energy + virial, 4000 atoms: 164k SM cycles
 // in groups, 146k one by one); a pass with the minimum image and the virial of every pair
 // is bound by issue slots, and a branch per entry costs more than the selects (500 atoms,
-// eight boxes per CTA: 149k one by one, 136k in groups).
+// eight boxes per CTA: 149k one by one, 136k in groups), but not with several threads per
+// atom: their sub-lists are two or three words, a third of them padding, which a branch
+// skips (1216 boxes of 256 atoms, 420 steps: rho 1.0 37.4 ms in groups, 36.2 one by one; 0.5
+// 28.8 and 29.7; 152 boxes, rho 0.75: 6.4 and 6.1).
 template <bool EN, bool VIR, bool MI>
 constexpr bool kPairInGroups = MDEOS_LIST_AHEAD > 1 || (VIR && MI);
 
@@ -651,7 +654,7 @@ __device__ __noinline__ FSums force_pass(uint32_t xs_a, float4* fs, const uint16
 #pragma unroll 1
           for (int kb = 0; kb < nw; ++kb) {
             const uint4 cur = rd.next();
-            if constexpr (kPairInGroups<EN, VIR, true>) {
+            if (kPairInGroups<EN, VIR, true> && (MDEOS_LIST_AHEAD > 1 || tpa == 1)) {
 #pragma unroll
               for (int g = 0; g < 8; g += kPairGroup)
                 pair_group<kPairGroup, EN, VIR, true>(
@@ -694,8 +697,14 @@ __device__ __noinline__ FSums force_pass(uint32_t xs_a, float4* fs, const uint16
           }
         }
       }
+      // The warp's lanes of this turn (those up to u1) meet again here.  Their lists differ in
+      // length, and a shuffle among the four lanes of an atom does not bring the others
+      // back: without this the parts of a warp ran the remaining turns one after another
+      // (1216 boxes of 300 atoms, rho 0.5, 420 steps: 61.7 ms without, 41.8 with).
+      const int left = u1 - (u - (tid & 31));
+      const unsigned m = left >= 32 ? 0xffffffffu : (1u << left) - 1u;
+      __syncwarp(m);
       if (tpa > 1) {  // the partial forces of the atom's units, in a fixed order
-        const unsigned m = tpa_mask(tpa);
         fx += __shfl_xor_sync(m, fx, 1);
         fy += __shfl_xor_sync(m, fy, 1);
         fz += __shfl_xor_sync(m, fz, 1);
