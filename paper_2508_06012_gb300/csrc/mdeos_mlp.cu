@@ -9,9 +9,9 @@
 // and the Adam state are FP32 (FP32 master weights).
 //
 // The 128x128 layers (forward Z = H W^T, backward dW = dZ^T H and dH = dZ W) run on the
-// tensor cores through one GEMM kernel (mma.m16n8k16, bf16 x bf16 -> fp32), batched
-// over the ensemble members on grid z; the 2-wide layers and the elementwise steps
-// run on the CUDA cores.
+// 5th-generation tensor cores (tcgen05.mma, bf16 x bf16 -> fp32 in tensor memory): fused
+// kernels for inference and for the forward and backward pass of a training batch, one
+// GEMM for the rest; the 2-wide layers and the elementwise steps run on the CUDA cores.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -129,94 +129,115 @@ __global__ void mlp_output(const __nv_bfloat16* H3, const float* P, const __nv_b
   Y[i] = y + P[(long long)e * kNParam + kOffB4 + o];
 }
 
-// Gradients that are sums over the batch alone: dW4, db4 (from dy, h3), db3, db2, db1
-// (columns of dz3, dz2, dz1) and dW1 (dz1, x).  Each is one FP32 sum over b = 0, 1, ...
-// in order, a chain of B dependent additions (1 us at B = 512); with the loads in the
-// chain it took 40 us per kernel, five kernels, and 33 us in one kernel with each warp
-// loading its own rows.  Here a CTA (32 columns of one model) copies kColRows rows of all
-// operands into shared memory with cp.async, two stages in turn, and each warp walks its
-// sum through them.
-constexpr int kColRows = 128;
-struct ColStage {
-  __nv_bfloat16 h3[kColRows][32], dz3[kColRows][32], dz2[kColRows][32];
-  float dz1[kColRows][32], dy[kColRows][2], x[kColRows][2];
-};
-constexpr int kColSmem = 2 * (int)sizeof(ColStage);
-
 template <int BYTES>
 __device__ __forceinline__ void cp_async(void* dst, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], %2;"
                ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src), "n"(BYTES) : "memory");
 }
 
-__global__ void __launch_bounds__(256) mlp_column_grads(const float* dY, const __nv_bfloat16* H3,
-                                                        const __nv_bfloat16* dZ3,
-                                                        const __nv_bfloat16* dZ2, const float* dZ1,
-                                                        const float* X, float* G, int B) {
-  extern __shared__ __align__(16) unsigned char csm[];
-  ColStage* st = reinterpret_cast<ColStage*>(csm);
-  const int e = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int j0 = blockIdx.x * 32, j = j0 + lane;
-  float* g = G + (long long)e * kNParam;
+// Gradients that are sums over the batch alone: dW4, db4 (from dy, h3), db3, db2, db1
+// (columns of dz3, dz2, dz1) and dW1 (dz1, x).  Each is one FP32 sum over b = 0, 1, ...
+// in order, a chain of B dependent additions (1 us at B = 512); with the loads in the
+// chain it took 40 us per kernel, five kernels.  Here a CTA (32 columns of one model)
+// copies kColRows rows of its operands at a time into a ring of kColStages in shared memory
+// with cp.async, and four warps walk a sum each through them.  Part 0 has dW4, db3 and
+// db4, part 1 has dW1, db2 and db1: the walk is bound by shared-memory loads (one or two per
+// row and sum), so the eight sums of 32 columns go to two SMs.
+constexpr int kColRows = 128, kColStages = 4;
+struct ColStage {                     // part 0 / part 1
+  float f[kColRows][32];              // - / dz1
+  __nv_bfloat16 a[kColRows][32];      // dz3 / dz2
+  __nv_bfloat16 h[kColRows][32];      // h3 / -
+  float p[kColRows][2];               // dy / x
+};
+constexpr int kColSmem = kColStages * (int)sizeof(ColStage);
+
+struct ColArgs {
+  const float *dY, *dZ1, *X;
+  const __nv_bfloat16 *H3, *dZ3, *dZ2;
+  float* G;
+  int B;
+  const float* part;  // sums of squared errors of npart tiles
+  int npart;
+  float* loss;
+};
+
+__device__ __forceinline__ void column_grads(const ColArgs& a, int e, int block, int part,
+                                             unsigned char* sm) {
+  ColStage* st = reinterpret_cast<ColStage*>(sm);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int j0 = block * 32, j = j0 + lane, B = a.B;
   const long long r0 = (long long)e * B;  // the model's first row
-  auto load = [&](int stage, int b0) {    // rows b0 .. of the batch, at most kColRows
-    ColStage& s = st[stage];
-    const int rows = min(kColRows, B - b0);
+  auto load = [&](int k) {                // chunk k of the batch, at most kColRows rows
+    const int b0 = k * kColRows, rows = min(kColRows, B - b0);
+    ColStage& s = st[k & (kColStages - 1)];
+    const __nv_bfloat16* dz = part == 0 ? a.dZ3 : a.dZ2;
     for (int q = tid; q < rows * 4; q += 256) {  // bf16 rows: four 16-byte pieces
       const int r = q >> 2, c = (q & 3) * 8;
       const long long at = (r0 + b0 + r) * kH + j0 + c;
-      cp_async<16>(&s.h3[r][c], H3 + at);
-      cp_async<16>(&s.dz3[r][c], dZ3 + at);
-      cp_async<16>(&s.dz2[r][c], dZ2 + at);
+      cp_async<16>(&s.a[r][c], dz + at);
+      if (part == 0) cp_async<16>(&s.h[r][c], a.H3 + at);
     }
-    for (int q = tid; q < rows * 8; q += 256)
-      cp_async<16>(&s.dz1[q >> 3][(q & 7) * 4], dZ1 + (r0 + b0 + (q >> 3)) * kH + j0 + (q & 7) * 4);
-    for (int q = tid; q < rows; q += 256) {
-      cp_async<8>(s.dy[q], dY + (r0 + b0 + q) * 2);
-      cp_async<8>(s.x[q], X + (long long)(b0 + q) * 2);
-    }
-    asm volatile("cp.async.commit_group;" ::: "memory");
+    if (part != 0)
+      for (int q = tid; q < rows * 8; q += 256)
+        cp_async<16>(&s.f[q >> 3][(q & 7) * 4], a.dZ1 + (r0 + b0 + (q >> 3)) * kH + j0 + (q & 7) * 4);
+    for (int q = tid; q < rows; q += 256)
+      cp_async<8>(s.p[q], part == 0 ? a.dY + (r0 + b0 + q) * 2 : a.X + (long long)(b0 + q) * 2);
   };
-  float sum = 0.f;
-  load(0, 0);
-  for (int b0 = 0, k = 0; b0 < B; b0 += kColRows, k ^= 1) {
-    if (b0 + kColRows < B) {
-      load(k ^ 1, b0 + kColRows);
-      asm volatile("cp.async.wait_group 1;" ::: "memory");
-    } else {
-      asm volatile("cp.async.wait_group 0;" ::: "memory");
+  if (e == 0 && block == 0 && part == 0 && warp == 7 && lane == 0) {
+    // in order (reproducible), the rounding errors of the sum added at its end
+    float l = 0.f, c = 0.f;
+#pragma unroll 8
+    for (int k = 0; k < a.npart; ++k) {
+      const float t = a.part[k], n = l + t, d = n - l;
+      c += (l - (n - d)) + (t - d);
+      l = n;
     }
-    __syncthreads();
-    const ColStage& s = st[k];
-    const int rows = min(kColRows, B - b0);
-    if (warp < 2) {  // dW4
-#pragma unroll 16
-      for (int r = 0; r < rows; ++r) sum = fmaf(s.dy[r][warp], __bfloat162float(s.h3[r][lane]), sum);
-    } else if (warp < 4) {  // dW1
-#pragma unroll 16
-      for (int r = 0; r < rows; ++r) sum = fmaf(s.dz1[r][lane], s.x[r][warp - 2], sum);
-    } else if (warp == 4) {
-#pragma unroll 16
-      for (int r = 0; r < rows; ++r) sum += __bfloat162float(s.dz3[r][lane]);
-    } else if (warp == 5) {
-#pragma unroll 16
-      for (int r = 0; r < rows; ++r) sum += __bfloat162float(s.dz2[r][lane]);
-    } else if (warp == 6) {
-#pragma unroll 16
-      for (int r = 0; r < rows; ++r) sum += s.dz1[r][lane];
-    } else {
-#pragma unroll 16
-      for (int r = 0; r < rows; ++r) sum += s.dy[r][lane & 1];
-    }
-    __syncthreads();  // the stage is filled again two turns on
+    *a.loss = l + c;
   }
+  const int nk = (B + kColRows - 1) / kColRows;
+  for (int k = 0; k < kColStages - 1; ++k) {
+    if (k < nk) load(k);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
+  float sum = 0.f;
+  for (int k = 0; k < nk; ++k) {
+    if (k + kColStages - 1 < nk) load(k + kColStages - 1);
+    asm volatile("cp.async.commit_group;" ::: "memory");
+    asm volatile("cp.async.wait_group %0;" ::"n"(kColStages - 1) : "memory");
+    __syncthreads();
+    const ColStage& s = st[k & (kColStages - 1)];
+    const int rows = min(kColRows, B - k * kColRows);
+    if (warp < 2) {  // dW4 / dW1
+      if (part == 0) {
+#pragma unroll 16
+        for (int r = 0; r < rows; ++r) sum = fmaf(s.p[r][warp], __bfloat162float(s.h[r][lane]), sum);
+      } else {
+#pragma unroll 16
+        for (int r = 0; r < rows; ++r) sum = fmaf(s.f[r][lane], s.p[r][warp], sum);
+      }
+    } else if (warp == 2) {  // db3 / db2
+#pragma unroll 16
+      for (int r = 0; r < rows; ++r) sum += __bfloat162float(s.a[r][lane]);
+    } else if (warp == 3) {  // db4 / db1
+      if (part == 0) {
+#pragma unroll 16
+        for (int r = 0; r < rows; ++r) sum += s.p[r][lane & 1];
+      } else {
+#pragma unroll 16
+        for (int r = 0; r < rows; ++r) sum += s.f[r][lane];
+      }
+    }
+    __syncthreads();  // the stage is filled again in the next turn
+  }
+  float* g = a.G + (long long)e * kNParam;
   if (warp < 2)
-    g[kOffW4 + warp * kH + j] = sum;
-  else if (warp < 4)
-    g[kOffW1 + 2 * j + warp - 2] = sum;
-  else if (warp < 7)
-    g[(warp == 4 ? kOffB3 : warp == 5 ? kOffB2 : kOffB1) + j] = sum;
-  else if (blockIdx.x == 0 && lane < 2)
+    g[part == 0 ? kOffW4 + warp * kH + j : kOffW1 + 2 * j + warp] = sum;
+  else if (warp == 2)
+    g[(part == 0 ? kOffB3 : kOffB2) + j] = sum;
+  else if (warp == 3 && part != 0)
+    g[kOffB1 + j] = sum;
+  else if (warp == 3 && block == 0 && lane < 2)
     g[kOffB4 + lane] = sum;
 }
 
@@ -243,6 +264,7 @@ __global__ void mlp_adam(AdamArgs a) {
     const long long part = 2LL * a.E * kH * kH;
     const float* p = a.ws + ((long long)(w2 ? a.E : 0) + e) * kH * kH + (r - (w2 ? kOffW2 : kOffW3));
     g = p[0];
+#pragma unroll 4
     for (int s = 1; s < a.S; ++s) g += p[s * part];
   } else {
     g = a.G[i];
@@ -362,7 +384,7 @@ __device__ __forceinline__ unsigned long long tc_clock_ns() {
 
 // wait on an mbarrier phase for at most ~1 s; false if it did not complete
 __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity) {
-  const unsigned long long t0 = tc_clock_ns();
+  unsigned long long t0 = 0;
   for (int it = 0; it < (1 << 24); ++it) {
     uint32_t done;
     asm volatile(
@@ -370,7 +392,11 @@ __device__ __forceinline__ bool mbar_wait(uint32_t mbar, uint32_t parity) {
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(done) : "r"(mbar), "r"(parity) : "memory");
     if (done) return true;
-    if ((it & 255) == 255 && tc_clock_ns() - t0 > 1000000000ull) break;
+    if ((it & 255) == 255) {
+      const unsigned long long t = tc_clock_ns();
+      if (t0 == 0) t0 = t;
+      if (t - t0 > 1000000000ull) break;
+    }
   }
   return false;
 }
@@ -632,44 +658,99 @@ __global__ void __launch_bounds__(kTcGroups * kTcThreads, 1)
 // ---------------------------------------------------------------------------
 // Forward and backward pass of a training batch in one launch: grid (tiles of 128
 // samples, models), the tiles, descriptors and thread roles of mlp_infer_tc_kernel.
-// The four 128 x 128 weight operands (W2, W3 and their transposes, 32 KB each) are staged
-// once; tile A holds h1, h2, h3, dz3 and dz2 in turn, each the operand of the next
-// product:
 //   Z2 = h1 W2^T, Z3 = h2 W3^T, y and dy from h3, dz3 = (dy W4)(1 - h3^2),
 //   dh2 = dz3 W3, dz2 = dh2 (1 - h2^2), dh1 = dz2 W2, dz1 = dh1 (1 - h1^2).
 // h1..h3, dz3, dz2 (bf16), dz1 and dy (FP32) go to device memory for the sums over the
-// batch.  One launch instead of fourteen, and no FP32 pre-activations in memory: the step
-// was bound by launches and by one-warp sums, not by its products (batch 512, 4 models:
-// a step of an epoch took 328 us, host included, and takes 70 now).  Products accumulate K in the same order of
-// tcgen05.mma steps as bf16_gemm_tc_kernel's chunks, and every element is rounded where
-// the layered form rounds it.
-constexpr int kTrThreads = 512;  // four threads per row (column quarters)
-constexpr int kTrCols = kTrThreads == 512 ? kH / 4 : kH / 2;
-constexpr int kTrSmem = 5 * kTcTile + 1024 + 64 + kTcSmall * 4 + kTcRows * 2 * 4;
+// batch.  Products accumulate K in the same order of tcgen05.mma steps as
+// bf16_gemm_tc_kernel's chunks, and every element is rounded where the layered form rounds it.
+//
+// A few CTAs walk one serial chain, so what bounds it is the latency of that chain.  All of
+// it stays in shared memory, in five tiles of 32 KB: h1, W2, W3 and the transposes of W3 and
+// W2.  h2 takes W2's place once its product is done, h3 W3's; dz3 and dz2 overwrite h3 and
+// h2, and dz1 (FP32) the transposes.  The weights arrive by cp.async, W2 first.  A finished
+// tile goes to device memory while the next product runs, 64 bytes of a row per lane group
+// (a thread storing its own row touches 32 lines per store, and reading it back for the
+// backward pass again).  Batch 512, 4 models: 27.5 us with the tiles stored and
+// read back by rows, 21.4 now; with the sums and Adam a step of an epoch takes 46 us, host
+// included (328 us with a launch per layer and product).
+constexpr int kTrThreads = 512;    // four threads per row (column quarters)
+constexpr int kTrCols = kH / 4;
+constexpr int kTrSmem = 5 * kTcTile + 1024 + 64 + (kTcSmall + 4 * kTcRows + 8) * 4;
 
 struct TrainArgs {
   const float *X, *T, *P;
   const __nv_bfloat16 *W1b, *W2b, *W3b, *W4b, *W2t, *W3t;
   __nv_bfloat16 *H1, *H2, *H3, *dZ3, *dZ2;
-  float *dZ1, *dY, *loss;
+  float *dZ1, *dY, *part;
   int B;
   int* err;
 };
+
+// 16-byte unit u (0..2047) of a tile: eight lanes take eight rows of one core matrix (no bank
+// conflicts), a warp 64 bytes of each of those rows
+__device__ __forceinline__ void tile_unit(int u, int& r, int& c) {
+  r = (u >> 7) * 8 + (u & 7);
+  c = (((u >> 5) & 3) * 4 + ((u >> 3) & 3)) * 8;
+}
+
+// a tile's first `rows` rows to dst (rows of kH elements), by threads t of nt
+__device__ __forceinline__ void store_tile(const unsigned char* tile, __nv_bfloat16* dst, int rows,
+                                           int t, int nt) {
+#pragma unroll 4
+  for (int u = t; u < kTcRows * kH / 8; u += nt) {
+    int r, c;
+    tile_unit(u, r, c);
+    if (r < rows)
+      *reinterpret_cast<uint4*>(dst + (long long)r * kH + c) =
+          *reinterpret_cast<const uint4*>(tile + tc_off(r, c));
+  }
+}
+
+// dz = dh (1 - h^2) of eight units, h as packed bf16; returns bf16(dz) packed
+__device__ __forceinline__ uint4 dtanh8(float* v, uint4 h) {
+  const __nv_bfloat16* h8 = reinterpret_cast<const __nv_bfloat16*>(&h);
+  uint4 out;
+  __nv_bfloat16* o8 = reinterpret_cast<__nv_bfloat16*>(&out);
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const float x = __bfloat162float(h8[j]);
+    v[j] = v[j] * (1.f - x * x);
+    o8[j] = __float2bfloat16_rn(v[j]);
+  }
+  return out;
+}
 
 __global__ void __launch_bounds__(kTrThreads) mlp_train_tc_kernel(TrainArgs a) {
   extern __shared__ __align__(1024) unsigned char tsm[];
   const uint32_t sbase = ((uint32_t)__cvta_generic_to_shared(tsm) + 1023u) & ~1023u;
   unsigned char* gbase = tsm + (sbase - (uint32_t)__cvta_generic_to_shared(tsm));
-  const uint32_t sA = sbase, sMbar = sbase + 5 * kTcTile, sTmem = sMbar + 8;
-  unsigned char* gA = gbase;
+  const uint32_t sMbar = sbase + 5 * kTcTile, sTmem = sMbar + 8;
+  unsigned char *const g1 = gbase, *const g2 = gbase + kTcTile, *const g3 = gbase + 2 * kTcTile;
   const int e = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int m = tid & (kTcRows - 1), quarter = tid >> 7, c_lo = quarter * kTrCols;
-  const int B = a.B, b = blockIdx.x * kTcRows + m;
+  const int B = a.B, b0 = blockIdx.x * kTcRows, b = b0 + m, rows = min(kTcRows, B - b0);
   const bool on = b < B;
-  const long long row = ((long long)e * B + b) * kH;  // this sample's row of the model's arrays
+  const long long row0 = ((long long)e * B + b0) * kH;  // the tile's first row in the model's arrays
   const float* p = a.P + (long long)e * kNParam;
   float* sp = reinterpret_cast<float*>(gbase + 5 * kTcTile + 64);  // small parameters
-  float* sdy = sp + kTcSmall;                                       // dy, then squared errors
+  float* sdy = sp + kTcSmall;                                       // dy
+  float* ssq = sdy + 2 * kTcRows;                                   // squared errors
+  float* spart = ssq + 2 * kTcRows;                                 // their sums by warp
+  {  // the four operands, 16 bytes at a time into the canonical layout
+    const __nv_bfloat16* w[4] = {a.W2b, a.W3b, a.W3t, a.W2t};
+#pragma unroll
+    for (int t = 0; t < 4; ++t) {
+#pragma unroll
+      for (int u = tid; u < kH * kH / 8; u += kTrThreads) {
+        int n, k;
+        tile_unit(u, n, k);
+        cp_async<16>(gbase + (t + 1) * kTcTile + tc_off(n, k),
+                     w[t] + (long long)e * kH * kH + n * kH + k);
+      }
+      if (t == 0) asm volatile("cp.async.commit_group;" ::: "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+  }
   for (int k = tid; k < 2 * kH; k += kTrThreads) {
     sp[kTcSW1 + k] = __bfloat162float(a.W1b[(long long)e * 2 * kH + k]);
     sp[kTcSW4 + k] = __bfloat162float(a.W4b[(long long)e * 2 * kH + k]);
@@ -680,16 +761,8 @@ __global__ void __launch_bounds__(kTrThreads) mlp_train_tc_kernel(TrainArgs a) {
     sp[kTcSB3 + k] = p[kOffB3 + k];
   }
   if (tid < 2) sp[kTcSB4 + tid] = p[kOffB4 + tid];
-  {  // the four operands, 16 bytes at a time into the canonical layout
-    const __nv_bfloat16* w[4] = {a.W2b, a.W3b, a.W3t, a.W2t};
-    for (int q = tid; q < kH * kH / 8; q += kTrThreads) {
-      const int n = (q >> 7) * 8 + (q & 7), k = ((q >> 3) & 15) * 8;
-#pragma unroll
-      for (int t = 0; t < 4; ++t)
-        *reinterpret_cast<uint4*>(gbase + (t + 1) * kTcTile + tc_off(n, k)) =
-            *reinterpret_cast<const uint4*>(w[t] + (long long)e * kH * kH + n * kH + k);
-    }
-  }
+  const float x0 = on ? a.X[2 * b] : 0.f, x1 = on ? a.X[2 * b + 1] : 0.f;
+  const float target = on && quarter < 2 ? a.T[2 * b + quarter] : 0.f;
   if (tid == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(sMbar) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
@@ -704,8 +777,40 @@ __global__ void __launch_bounds__(kTrThreads) mlp_train_tc_kernel(TrainArgs a) {
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(gbase + 5 * kTcTile + 8);
   const uint32_t tq = tmem + ((uint32_t)((warp & 3) * 32) << 16) + (uint32_t)c_lo;
-  // layer 1 on the CUDA cores: this row's units c_lo .. c_lo + 31
-  const float x0 = on ? a.X[2 * b] : 0.f, x1 = on ? a.X[2 * b + 1] : 0.f;
+  // accumulator = tile A times tile W (by number), once every thread has written its part
+  // of tile A and its share of the weights has arrived
+  const auto product = [&](int tA, int tW) {
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // shared memory -> tensor core
+    asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
+    __syncthreads();
+    if (tid == 0) {
+      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t sA = sbase + (uint32_t)tA * kTcTile, sW = sbase + (uint32_t)tW * kTcTile;
+#pragma unroll
+      for (int ks = 0; ks < kH / 16; ++ks)  // K step of 16 = two core matrices along K
+        tc_mma(tmem, tc_desc(sA + ks * 2 * kLbo), tc_desc(sW + ks * 2 * kLbo), ks > 0);
+      tc_commit(sMbar);
+    }
+    __syncwarp();
+  };
+  // the product's end, the same answer in every thread; false: the wait ran out
+  int layer = 0;
+  const auto finished = [&]() {
+    const bool done = mbar_wait(sMbar, (uint32_t)layer & 1u);
+    const bool ok = __syncthreads_and(done) != 0;
+    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+    if (ok) ++layer;
+    return ok;
+  };
+  // h = bf16(tanh(z + b)) of this row's 32 units
+  const auto hidden = [&](unsigned char* tile, const float* bias) {
+    float v[32];
+    tc_ld32(tq, v);
+#pragma unroll
+    for (int j = 0; j < 32; j += 8)
+      *reinterpret_cast<uint4*>(tile + tc_off(m, c_lo + j)) = tanh_pack8(v + j, bias + c_lo + j);
+  };
+  // layer 1 on the CUDA cores
 #pragma unroll 1
   for (int c = c_lo; c < c_lo + kTrCols; c += 8) {
     float z[8];
@@ -714,136 +819,111 @@ __global__ void __launch_bounds__(kTrThreads) mlp_train_tc_kernel(TrainArgs a) {
       const float2 w = *reinterpret_cast<const float2*>(sp + kTcSW1 + 2 * (c + j));
       z[j] = x0 * w.x + x1 * w.y;
     }
-    const uint4 pk = tanh_pack8(z, sp + kTcSB1 + c);
-    *reinterpret_cast<uint4*>(gA + tc_off(m, c)) = pk;
-    if (on) *reinterpret_cast<uint4*>(a.H1 + row + c) = pk;
+    *reinterpret_cast<uint4*>(g1 + tc_off(m, c)) = tanh_pack8(z, sp + kTcSB1 + c);
   }
-  bool ok = true;
-  int layer = 0;
-  // four products, W2, W3, W3 transposed, W2 transposed, each with tile A as it then is
-#pragma unroll 1
-  for (; layer < 4; ++layer) {
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // tile A -> tensor core
+  asm volatile("cp.async.wait_group 1;" ::: "memory");  // W2
+  product(0, 1);
+  store_tile(g1, a.H1 + row0, rows, tid, kTrThreads);
+  bool ok = finished();
+  if (ok) {
+    hidden(g2, sp + kTcSB2);
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+    product(1, 2);
+    store_tile(g2, a.H2 + row0, rows, tid, kTrThreads);
+    ok = finished();
+  }
+  if (ok) {
+    hidden(g3, sp + kTcSB3);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-    __syncthreads();
-    if (tid == 0) {
-      asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-      const uint32_t sW = sbase + (uint32_t)(layer + 1) * kTcTile;
-#pragma unroll
-      for (int ks = 0; ks < kH / 16; ++ks)  // K step of 16 = two core matrices along K
-        tc_mma(tmem, tc_desc(sA + ks * 2 * kLbo), tc_desc(sW + ks * 2 * kLbo), ks > 0);
-      tc_commit(sMbar);
-    }
-    __syncwarp();
-    const bool done = mbar_wait(sMbar, (uint32_t)layer & 1u);
-    ok = __syncthreads_and(done) != 0;  // the same decision in every thread
-    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (!ok) break;
-    if (layer < 2) {  // h = bf16(tanh(z + b)) of this row's 32 units
-      const float* bias = sp + (layer == 0 ? kTcSB2 : kTcSB3) + c_lo;
-      __nv_bfloat16* H = (layer == 0 ? a.H2 : a.H3) + row + c_lo;
-#pragma unroll 1
-      for (int c0 = 0; c0 < kTrCols; c0 += 32) {
-        float v[32];
-        tc_ld32(tq + (uint32_t)c0, v);
-#pragma unroll
-        for (int j8 = 0; j8 < 32; j8 += 8) {
-          const uint4 pk = tanh_pack8(v + j8, bias + c0 + j8);
-          *reinterpret_cast<uint4*>(gA + tc_off(m, c_lo + c0 + j8)) = pk;
-          if (on) *reinterpret_cast<uint4*>(H + c0 + j8) = pk;
-        }
-      }
-    } else {  // dz = dh (1 - h^2): bf16 into tile A for the next product, or dz1 in FP32
-      const __nv_bfloat16* H = (layer == 2 ? a.H2 : a.H1) + row + c_lo;
-#pragma unroll 1
-      for (int c0 = 0; c0 < kTrCols; c0 += 32) {
-        float v[32];
-        tc_ld32(tq + (uint32_t)c0, v);
-#pragma unroll
-        for (int j8 = 0; j8 < 32; j8 += 8) {
-          uint4 pk = make_uint4(0u, 0u, 0u, 0u);
-          if (on) pk = *reinterpret_cast<const uint4*>(H + c0 + j8);
-          const __nv_bfloat16* h8 = reinterpret_cast<const __nv_bfloat16*>(&pk);
-          uint4 out;
-          __nv_bfloat16* o8 = reinterpret_cast<__nv_bfloat16*>(&out);
-#pragma unroll
-          for (int j = 0; j < 8; ++j) {
-            const float h = __bfloat162float(h8[j]);
-            v[j8 + j] = v[j8 + j] * (1.f - h * h);
-            o8[j] = __float2bfloat16_rn(v[j8 + j]);
-          }
-          if (layer == 2) {
-            *reinterpret_cast<uint4*>(gA + tc_off(m, c_lo + c0 + j8)) = out;
-            if (on) *reinterpret_cast<uint4*>(a.dZ2 + row + c_lo + c0 + j8) = out;
-          } else if (on) {
-            float4* z1 = reinterpret_cast<float4*>(a.dZ1 + row + c_lo + c0 + j8);
-            z1[0] = make_float4(v[j8], v[j8 + 1], v[j8 + 2], v[j8 + 3]);
-            z1[1] = make_float4(v[j8 + 4], v[j8 + 5], v[j8 + 6], v[j8 + 7]);
-          }
-        }
-      }
-    }
-    if (layer == 1) {  // output layer, its error, dz3
-      asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
-      __syncthreads();  // h3 of both halves is in tile A
-      float d = 0.f;
-      if (quarter < 2) {  // output unit = quarter
-        const float* w4 = sp + kTcSW4 + quarter * kH;
-        float y = 0.f;
+    __syncthreads();  // h3 is complete
+    if (quarter < 2) {  // output unit = quarter
+      const float* w4 = sp + kTcSW4 + quarter * kH;
+      float y = 0.f;
 #pragma unroll 4
-        for (int c = 0; c < kH; c += 8) {
-          const uint4 pk = *reinterpret_cast<const uint4*>(gA + tc_off(m, c));
-          const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&pk);
+      for (int c = 0; c < kH; c += 8) {
+        const uint4 pk = *reinterpret_cast<const uint4*>(g3 + tc_off(m, c));
+        const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&pk);
+        const float4 wa = *reinterpret_cast<const float4*>(w4 + c);
+        const float4 wb = *reinterpret_cast<const float4*>(w4 + c + 4);
+        const float w[8] = {wa.x, wa.y, wa.z, wa.w, wb.x, wb.y, wb.z, wb.w};
 #pragma unroll
-          for (int j = 0; j < 4; ++j) {
-            const float2 hf = __bfloat1622float2(h[j]);
-            y = fmaf(w4[c + 2 * j], hf.x, y);
-            y = fmaf(w4[c + 2 * j + 1], hf.y, y);
-          }
+        for (int j = 0; j < 4; ++j) {
+          const float2 hf = __bfloat1622float2(h[j]);
+          y = fmaf(w[2 * j], hf.x, y);
+          y = fmaf(w[2 * j + 1], hf.y, y);
         }
-        y += sp[kTcSB4 + quarter];
-        d = on ? y - a.T[2 * b + quarter] : 0.f;
-        const float dyv = d / (float)B;  // 2 (y - t) / (2 B)
-        if (on) a.dY[((long long)e * B + b) * 2 + quarter] = dyv;
-        sdy[2 * m + quarter] = dyv;
       }
-      __syncthreads();  // dy of both outputs; every thread has read its row of h3
-      const float dy0 = sdy[2 * m], dy1 = sdy[2 * m + 1];
+      y += sp[kTcSB4 + quarter];
+      const float d = on ? y - target : 0.f;
+      const float dyv = d / (float)B;  // 2 (y - t) / (2 B)
+      if (on) a.dY[((long long)e * B + b) * 2 + quarter] = dyv;
+      sdy[2 * m + quarter] = dyv;
+      ssq[2 * m + quarter] = d * d;
+    } else {
+      store_tile(g3, a.H3 + row0, rows, tid - kTrThreads / 2, kTrThreads / 2);
+    }
+    __syncthreads();  // dy of both outputs; h3 has been read
+    const float dy0 = sdy[2 * m], dy1 = sdy[2 * m + 1];
 #pragma unroll 1
-      for (int c = c_lo; c < c_lo + kTrCols; c += 8) {
-        const uint4 pk = *reinterpret_cast<const uint4*>(gA + tc_off(m, c));
-        const __nv_bfloat16* h8 = reinterpret_cast<const __nv_bfloat16*>(&pk);
-        uint4 out;
-        __nv_bfloat16* o8 = reinterpret_cast<__nv_bfloat16*>(&out);
+    for (int c = c_lo; c < c_lo + kTrCols; c += 8) {
+      float v[8];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
-          const float dh = dy0 * sp[kTcSW4 + c + j] + dy1 * sp[kTcSW4 + kH + c + j];
-          const float h = __bfloat162float(h8[j]);
-          o8[j] = __float2bfloat16_rn(dh * (1.f - h * h));
-        }
-        *reinterpret_cast<uint4*>(gA + tc_off(m, c)) = out;
-        if (on) *reinterpret_cast<uint4*>(a.dZ3 + row + c) = out;
-      }
-      // squared errors in sample order: sums of 32 by shuffles, of 256 in warp order,
-      // one atomic per tile
-      __syncthreads();  // dy has been read
-      if (quarter < 2) sdy[2 * m + quarter] = d * d;
-      __syncthreads();
-      float l = tid < 2 * kTcRows ? sdy[tid] : 0.f;
+      for (int j = 0; j < 8; ++j) v[j] = dy0 * sp[kTcSW4 + c + j] + dy1 * sp[kTcSW4 + kH + c + j];
+      uint4* h = reinterpret_cast<uint4*>(g3 + tc_off(m, c));
+      *h = dtanh8(v, *h);
+    }
+    product(2, 3);
+    // squared errors in sample order: sums of 32 by shuffles, of 256 in warp order; the
+    // tiles' sums are added in order by mlp_batch_sums
+    if (warp < 2 * kTcRows / 32) {
+      float l = ssq[tid];
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) l += __shfl_xor_sync(0xffffffffu, l, o);
-      __syncthreads();
-      if (lane == 0 && tid < 2 * kTcRows) sdy[warp] = l;
-      __syncthreads();
-      if (tid == 0) {
-        float t = 0.f;
-        for (int w = 0; w < 2 * kTcRows / 32; ++w) t += sdy[w];
-        atomicAdd(a.loss, t);
-      }
+      if (lane == 0) spart[warp] = l;
+    }
+    store_tile(g3, a.dZ3 + row0, rows, tid, kTrThreads);
+    ok = finished();
+    if (tid == 0) {
+      float t = 0.f;
+      for (int w = 0; w < 2 * kTcRows / 32; ++w) t += spart[w];
+      a.part[(long long)e * gridDim.x + blockIdx.x] = t;
     }
   }
-  if (!ok) {  // the tile's later outputs stay unwritten; let the MMAs in flight finish (bounded)
+  if (ok) {
+    float v[32];
+    tc_ld32(tq, v);
+#pragma unroll
+    for (int j = 0; j < 32; j += 8) {
+      uint4* h = reinterpret_cast<uint4*>(g2 + tc_off(m, c_lo + j));
+      *h = dtanh8(v + j, *h);
+    }
+    product(1, 4);
+    store_tile(g2, a.dZ2 + row0, rows, tid, kTrThreads);
+    ok = finished();
+  }
+  if (ok) {
+    // dz1 by rows of 512 B, their 16-byte units swapped by row (no bank conflicts), where
+    // the transposes were
+    float4* z1 = reinterpret_cast<float4*>(gbase + 3 * kTcTile);
+    float v[32];
+    tc_ld32(tq, v);
+#pragma unroll
+    for (int j = 0; j < 32; j += 8) {
+      dtanh8(v + j, *reinterpret_cast<const uint4*>(g1 + tc_off(m, c_lo + j)));
+      const int c = (c_lo + j) >> 2;
+      z1[m * 32 + (c ^ (m & 7))] = make_float4(v[j], v[j + 1], v[j + 2], v[j + 3]);
+      z1[m * 32 + ((c + 1) ^ (m & 7))] = make_float4(v[j + 4], v[j + 5], v[j + 6], v[j + 7]);
+    }
+    __syncthreads();
+    float4* out = reinterpret_cast<float4*>(a.dZ1 + row0);
+#pragma unroll 4
+    for (int u = tid; u < kTcRows * 32; u += kTrThreads) {
+      const int r = u >> 5, c = u & 31;
+      if (r < rows) out[(long long)r * 32 + c] = z1[r * 32 + (c ^ (r & 7))];
+    }
+  } else {  // the tile's later outputs stay unwritten; let the MMAs in flight finish (bounded)
     if (tid == 0) atomicExch(a.err, 1);
+    asm volatile("cp.async.wait_all;" ::: "memory");
     mbar_wait(sMbar, (uint32_t)layer & 1u);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -858,13 +938,14 @@ __global__ void __launch_bounds__(kTrThreads) mlp_train_tc_kernel(TrainArgs a) {
 // The training products on the 5th-generation tensor cores: C[z](m, n) =
 // sum_k A[z](m, k) B[z](k, n) with arbitrary strides (GemmArgs), one 128 x 128 tile of
 // C per CTA with the fp32 accumulator in
-// tensor memory.  K runs in chunks of 64: the 128 threads stage A's 128 x 64 and B's
-// (128 columns of C) x 64 elements into the canonical no-swizzle K-major layout (8 x 8
-// core matrices of 128 B: element (r, k) at (r / 8) * 1024 + (k / 8) * 128 + (r % 8) * 16
-// + (k % 8) * 2; zero outside the matrices), one thread issues four tcgen05.mma of
-// K = 16 and commits to an mbarrier, and every thread waits (at most ~1 s, then the
-// error flag is set and the tile is left unwritten) before the next chunk overwrites the
-// tiles.  Epilogue: thread t reads TMEM lane t (row m0 + t), 32 columns at a time.
+// tensor memory.  K runs in chunks of 64, in two pairs of tiles in turn: 128 threads stage A's
+// 128 x 64, the other 128 B's (128 columns of C) x 64 elements into the canonical no-swizzle
+// K-major layout (8 x 8 core matrices of 128 B: element (r, k) at (r / 8) * 1024 + (k / 8) *
+// 128 + (r % 8) * 16 + (k % 8) * 2; zero outside the matrices), one thread issues four
+// tcgen05.mma of K = 16 and commits to the pair's mbarrier.  Every thread waits for a pair's
+// last product (at most ~1 s, then the error flag is set and the tile is left unwritten)
+// before it is filled again.  Epilogue: the accumulator goes through shared memory, so that a
+// warp stores rows of C (a thread storing its own row touches 32 lines per store).
 
 constexpr int kGK = 64;                   // K per staged chunk
 constexpr uint32_t kGSbo = 1024;          // bytes between 8-row groups of a chunk
@@ -931,22 +1012,25 @@ __device__ __forceinline__ void stage_strided(unsigned char* tile, const __nv_bf
   }
 }
 
-__global__ void __launch_bounds__(kTcRows) bf16_gemm_tc_kernel(GemmArgs g, int* err) {
-  __shared__ __align__(1024) unsigned char gsm[2 * kGTile];
-  __shared__ __align__(8) unsigned long long s_mbar;
+constexpr int kGThreads = 256;
+constexpr int kGSmem = 4 * kGTile + 1024;
+
+__device__ __forceinline__ void gemm_tile(const GemmArgs& g, int bx, int by, int bz,
+                                          unsigned char* raw, int* err) {
+  __shared__ __align__(8) unsigned long long s_mbar[2];
   __shared__ uint32_t s_tmem;
-  const int z = blockIdx.z / g.S, sk = blockIdx.z - z * g.S;
-  const int m0 = blockIdx.y * kTcRows, n0 = blockIdx.x * kH;
+  const uint32_t sbase = ((uint32_t)__cvta_generic_to_shared(raw) + 1023u) & ~1023u;
+  unsigned char* gsm = raw + (sbase - (uint32_t)__cvta_generic_to_shared(raw));
+  const int z = bz / g.S, sk = bz - z * g.S;
+  const int m0 = by * kTcRows, n0 = bx * kH;
   const int kbeg = sk * g.kchunk, kend = min(g.K, kbeg + g.kchunk);  // this CTA's part of K
   const bool two = z >= g.z2;
   const int zi = two ? z - g.z2 : z;
-  const __nv_bfloat16* A = (two ? g.A2 : g.A) + (long long)zi * g.sa_z;
-  const __nv_bfloat16* B = (two ? g.B2 : g.B) + (long long)zi * g.sb_z;
-  const int tid = threadIdx.x, warp = tid >> 5;
-  const uint32_t sA = (uint32_t)__cvta_generic_to_shared(gsm), sB = sA + kGTile;
-  const uint32_t mbar = (uint32_t)__cvta_generic_to_shared(&s_mbar);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const uint32_t mbar = (uint32_t)__cvta_generic_to_shared(&s_mbar[0]);
   if (tid == 0) {
     asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar) : "memory");
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar + 8) : "memory");
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 0) {  // 128 TMEM columns: the 128 x 128 fp32 accumulator
@@ -958,90 +1042,98 @@ __global__ void __launch_bounds__(kTcRows) bf16_gemm_tc_kernel(GemmArgs g, int* 
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(&s_tmem);
-  uint32_t commits = 0;
+  // the operand this thread stages: rows o0 .. of `rows`, element (r, k) at O[r so_r + k so_k]
+  const bool isB = tid >= kTcRows;
+  const int t = tid & (kTcRows - 1);
+  const __nv_bfloat16* O = isB ? (two ? g.B2 : g.B) + (long long)zi * g.sb_z
+                               : (two ? g.A2 : g.A) + (long long)zi * g.sa_z;
+  const int o0 = isB ? n0 : m0, orows = isB ? g.N : g.M;
+  const long long so_r = isB ? g.sb_n : g.sa_m, so_k = isB ? g.sb_k : g.sa_k;
+  // contiguous along K (and 16-byte aligned rows): eight elements per load, one core-matrix
+  // row per store; contiguous along the rows, in aligned eights: 8 x 8 blocks; otherwise
+  // element by element with the row index running fastest across the threads
+  const bool al = ((uintptr_t)O & 15) == 0;
+  const bool vec_k = so_k == 1 && (so_r & 7) == 0 && al && (g.K & 7) == 0;
+  const bool blk = so_r == 1 && (so_k & 7) == 0 && al && (orows & 7) == 0;
+  int nk = 0;  // chunks issued
   bool ok = true;
-  // operands contiguous along K (and 16-byte aligned rows): eight elements per load,
-  // one core-matrix row per store; otherwise element by element with the contiguous
-  // index (M or N) running fastest across the threads
-  const bool a_vec = g.sa_k == 1 && (g.sa_m & 7) == 0 && (g.sa_z & 7) == 0 &&
-                     ((uintptr_t)A & 15) == 0 && (g.K & 7) == 0;
-  const bool b_vec = g.sb_k == 1 && (g.sb_n & 7) == 0 && (g.sb_z & 7) == 0 &&
-                     ((uintptr_t)B & 15) == 0 && (g.K & 7) == 0;
-  // operands contiguous along M or N, in aligned eights: 8 x 8 blocks
-  const bool a_blk = g.sa_m == 1 && (g.sa_k & 7) == 0 && ((uintptr_t)A & 15) == 0 && (g.M & 7) == 0;
-  const bool b_blk = g.sb_n == 1 && (g.sb_k & 7) == 0 && ((uintptr_t)B & 15) == 0 && (g.N & 7) == 0;
-  for (int k0 = kbeg; k0 < kend; k0 += kGK) {
-    if (a_vec) {
-      for (int q = tid; q < kTcRows * (kGK / 8); q += kTcRows) {
-        const int r = q & (kTcRows - 1), c = (q >> 7) * 8;  // consecutive threads: rows
-        const int m = m0 + r, k = k0 + c;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (m < g.M && k < kend) v = *reinterpret_cast<const uint4*>(A + (long long)m * g.sa_m + k);
-        *reinterpret_cast<uint4*>(gsm + gk_off(r, c)) = v;
-      }
-    } else if (a_blk) {
-      stage_blocks(gsm, A, m0, g.M, g.sa_k, k0, kend, tid);
-    } else {
-      stage_strided(gsm, A, m0 + tid, g.M, g.sa_m, g.sa_k, k0, kend, tid);
+  for (int k0 = kbeg; k0 < kend; k0 += kGK, ++nk) {
+    const int buf = nk & 1;
+    if (nk >= 2) {  // the pair's last product
+      const bool done = mbar_wait(mbar + 8 * buf, (uint32_t)((nk >> 1) - 1) & 1u);
+      ok = __syncthreads_and(done) != 0;  // the same decision in every thread
+      if (!ok) break;
     }
-    if (b_vec) {
-      for (int q = tid; q < kTcRows * (kGK / 8); q += kTcRows) {
-        const int r = q & (kTcRows - 1), c = (q >> 7) * 8;
-        const int n = n0 + r, k = k0 + c;
+    unsigned char* tile = gsm + (2 * buf + (isB ? 1 : 0)) * kGTile;
+    if (vec_k) {
+#pragma unroll
+      for (int c = 0; c < kGK; c += 8) {
+        const int k = k0 + c;
         uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (n < g.N && k < kend) v = *reinterpret_cast<const uint4*>(B + (long long)n * g.sb_n + k);
-        *reinterpret_cast<uint4*>(gsm + kGTile + gk_off(r, c)) = v;
+        if (o0 + t < orows && k < kend)
+          v = *reinterpret_cast<const uint4*>(O + (long long)(o0 + t) * so_r + k);
+        *reinterpret_cast<uint4*>(tile + gk_off(t, c)) = v;
       }
-    } else if (b_blk) {
-      stage_blocks(gsm + kGTile, B, n0, g.N, g.sb_k, k0, kend, tid);
+    } else if (blk) {
+      stage_blocks(tile, O, o0, orows, so_k, k0, kend, t);
     } else {
-      stage_strided(gsm + kGTile, B, n0 + tid, g.N, g.sb_n, g.sb_k, k0, kend, tid);
+      stage_strided(tile, O, o0 + t, orows, so_r, so_k, k0, kend, t);
     }
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // tiles -> tensor core
     __syncthreads();
     if (tid == 0) {
       asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+      const uint32_t sA = sbase + (uint32_t)(2 * buf) * kGTile, sB = sA + kGTile;
 #pragma unroll
       for (int ks = 0; ks < kGK / 16; ++ks)  // K step of 16 = two core matrices along K
         tc_mma(tmem, gk_desc(sA + ks * 2 * kLbo), gk_desc(sB + ks * 2 * kLbo),
                (k0 > kbeg || ks > 0) ? 1u : 0u);
-      tc_commit(mbar);
+      tc_commit(mbar + 8 * buf);
     }
     __syncwarp();
-    const bool done = mbar_wait(mbar, commits & 1u);
-    ++commits;
-    ok = __syncthreads_and(done) != 0;  // the same decision in every thread
+  }
+  if (nk > 0) {  // the last commit covers every product before it
+    const bool done = mbar_wait(mbar + 8 * ((nk - 1) & 1), (uint32_t)((nk - 1) >> 1) & 1u);
+    ok = (__syncthreads_and(done) != 0) && ok;
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    if (!ok) break;
   }
   if (ok) {
-    const int m = m0 + tid;
-    const uint32_t tl = tmem + ((uint32_t)(warp * 32) << 16);
+    // rows of 512 B in shared memory (no product reads it any more), their 16-byte units
+    // swapped by row: warps w and w + 4 take TMEM lanes 32 (w % 4) .., 64 columns each
+    float4* cs = reinterpret_cast<float4*>(gsm);
+    const int r = (warp & 3) * 32 + lane;
+    const uint32_t tl = tmem + ((uint32_t)((warp & 3) * 32) << 16);
+#pragma unroll 1
+    for (int c0 = (warp >> 2) * 64; c0 < (warp >> 2) * 64 + 64; c0 += 32) {
+      float v[32];
+      tc_ld32(tl + (uint32_t)c0, v);
+#pragma unroll
+      for (int j = 0; j < 8; ++j)
+        cs[r * 32 + (((c0 >> 2) + j) ^ (r & 7))] =
+            make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+    }
+    __syncthreads();
     float* C = g.S > 1 ? g.ws + ((long long)sk * g.Z + z) * g.M * g.N
                        : (two ? g.C2 : g.C) + (long long)zi * g.sc_z;
     const long long cm = g.S > 1 ? g.N : g.sc_m, cn = g.S > 1 ? 1 : g.sc_n;
-    // rows of C in aligned fours: 16-byte stores (a lane owns a row, so each store of a warp
-    // touches 32 sectors either way)
-    const bool vec = cn == 1 && (cm & 3) == 0 && ((uintptr_t)C & 15) == 0;
-#pragma unroll 1
-    for (int c0 = 0; c0 < kH; c0 += 32) {
-      float v[32];
-      tc_ld32(tl + (uint32_t)c0, v);  // every lane of the warp, in or out of the matrix
-      if (m < g.M && vec && n0 + c0 + 32 <= g.N) {
-        float4* row = reinterpret_cast<float4*>(C + (long long)m * cm + n0 + c0);
-#pragma unroll
-        for (int j = 0; j < 8; ++j)
-          row[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
-      } else if (m < g.M)
-#pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          const int n = n0 + c0 + j;
-          if (n < g.N) C[(long long)m * cm + (long long)n * cn] = v[j];
-        }
+    const bool vec = cn == 1 && (cm & 3) == 0 && ((uintptr_t)C & 15) == 0;  // 16-byte stores
+#pragma unroll 4
+    for (int u = tid; u < kTcRows * 32; u += kGThreads) {
+      const int i = u >> 5, q = u & 31, m = m0 + i, n = n0 + 4 * q;
+      if (m >= g.M || n >= g.N) continue;
+      const float4 x = cs[i * 32 + (q ^ (i & 7))];
+      float* c = C + (long long)m * cm + (long long)n * cn;
+      if (vec && n + 4 <= g.N) {
+        *reinterpret_cast<float4*>(c) = x;
+      } else {
+        c[0] = x.x;
+        if (n + 1 < g.N) c[cn] = x.y;
+        if (n + 2 < g.N) c[2 * cn] = x.z;
+        if (n + 3 < g.N) c[3 * cn] = x.w;
+      }
     }
-  } else {  // leave the tile unwritten; let the MMAs in flight finish (bounded)
-    if (tid == 0) atomicExch(err, 1);
-    mbar_wait(mbar, (commits - 1u) & 1u);
+  } else if (tid == 0) {  // leave the tile unwritten (the wait above was the MMAs' last chance)
+    atomicExch(err, 1);
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -1051,9 +1143,29 @@ __global__ void __launch_bounds__(kTcRows) bf16_gemm_tc_kernel(GemmArgs g, int* 
                  : "memory");
 }
 
-// C[z](m, n) = sum over s = 0, 1, ..., S - 1 of the partial tiles ws[s][z][m][n]
-__global__ void gemm_splitk_reduce(const float* ws, float* C, int M, int N, int Z, int S,
-                                   long long sc_m, long long sc_n, long long sc_z) {
+__global__ void __launch_bounds__(kGThreads) bf16_gemm_tc_kernel(GemmArgs g, int* err) {
+  extern __shared__ __align__(1024) unsigned char tsm[];
+  gemm_tile(g, blockIdx.x, blockIdx.y, blockIdx.z, tsm, err);
+}
+
+// Everything of a training batch that is a sum over its samples, in one launch: CTAs
+// 0 .. 2 (kH / 32) E - 1 the column sums (the longer ones), the others the 128 x 128 weight
+// gradients of both products.  Independent of one another and too few to fill the GPU, one
+// after the other they took 9.4 + 18.1 us; together they take 9.7 (batch 512, 4 models).
+constexpr int kSumSmem = kColSmem > kGSmem ? kColSmem : kGSmem;
+__global__ void __launch_bounds__(kGThreads) mlp_batch_sums(ColArgs c, GemmArgs g, int ncol,
+                                                            int* err) {
+  extern __shared__ __align__(1024) unsigned char tsm[];
+  const int i = blockIdx.x;
+  if (i < ncol)
+    column_grads(c, i / (2 * (kH / 32)), (i >> 1) & (kH / 32 - 1), i & 1, tsm);
+  else
+    gemm_tile(g, 0, 0, i - ncol, tsm, err);
+}
+
+// C[z](m, n) = sum over s = 0, 1, ..., S - 1 of the partial tiles ws[s][z][m][n]; C2 for z >= z2
+__global__ void gemm_splitk_reduce(const float* ws, float* C, float* C2, int z2, int M, int N,
+                                   int Z, int S, long long sc_m, long long sc_n, long long sc_z) {
   const long long per = (long long)M * N, all = per * Z;
   for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < all;
        i += (long long)gridDim.x * blockDim.x) {
@@ -1062,7 +1174,7 @@ __global__ void gemm_splitk_reduce(const float* ws, float* C, int M, int N, int 
     const int m = (int)(r / N), n = (int)(r - (long long)m * N);
     float acc = ws[i];
     for (int s = 1; s < S; ++s) acc += ws[s * all + i];
-    C[z * sc_z + m * sc_m + n * sc_n] = acc;
+    (z < z2 ? C + z * sc_z : C2 + (z - z2) * sc_z)[m * sc_m + n * sc_n] = acc;
   }
 }
 
@@ -1161,7 +1273,7 @@ struct mdeos_surrogate {
   __nv_bfloat16 *H1 = nullptr, *H2 = nullptr, *H3 = nullptr, *dZb = nullptr;
   float *Z = nullptr, *dZf = nullptr, *X = nullptr, *T = nullptr, *Y = nullptr, *dY = nullptr;
   float* loss = nullptr;
-  double *Xp = nullptr, *mean = nullptr, *sd = nullptr;
+  double* Xp = nullptr;
   int* err = nullptr;  // set by the fused kernel when an MMA wait ran out
   float* ws = nullptr;  // partial tiles of the products whose K is split
   long long ws_elems = 0;
@@ -1195,17 +1307,14 @@ constexpr int kMaxSplitK = 16;  // most CTAs one tile's K is split over
 // floats) holds the partial tiles; the partials are summed in a fixed order, so every
 // result is the same from run to run.
 //
-// A second batch (A2, B2 -> C2, same shape and strides) may share the launch; with
-// partials != nullptr the split's partial tiles are left in ws for the caller, who gets
-// the number of splits (1: the products are in C and C2).
-static cudaError_t gemm(cudaStream_t st, int* err, float* ws, long long ws_elems,
-                        const __nv_bfloat16* A, const __nv_bfloat16* B, float* C, int M, int N,
-                        int K, long long sa_m, long long sa_k, long long sa_z, long long sb_k,
-                        long long sb_n, long long sb_z, long long sc_m, long long sc_n,
-                        long long sc_z, int Z, const __nv_bfloat16* A2 = nullptr,
-                        const __nv_bfloat16* B2 = nullptr, float* C2 = nullptr,
-                        int* partials = nullptr) {
-  // the split depends on one batch's shape, so it is the same with and without a second
+// gemm_plan fixes the split; a second batch (A2, B2 -> C2, same shape and strides) may share
+// the launch and does not change it.
+static GemmArgs gemm_plan(float* ws, long long ws_elems, const __nv_bfloat16* A,
+                          const __nv_bfloat16* B, float* C, int M, int N, int K, long long sa_m,
+                          long long sa_k, long long sa_z, long long sb_k, long long sb_n,
+                          long long sb_z, long long sc_m, long long sc_n, long long sc_z, int Z,
+                          const __nv_bfloat16* A2 = nullptr, const __nv_bfloat16* B2 = nullptr,
+                          float* C2 = nullptr) {
   const int tiles = ((N + kH - 1) / kH) * ((M + kTcRows - 1) / kTcRows) * Z;
   const int nch = (K + kGK - 1) / kGK;
   const int Zall = A2 != nullptr ? 2 * Z : Z;
@@ -1216,17 +1325,33 @@ static cudaError_t gemm(cudaStream_t st, int* err, float* ws, long long ws_elems
     S = (nch + per - 1) / per;  // every split holds at least one chunk
     if ((long long)S * Zall * M * N > ws_elems) S = 1, per = nch;
   }
-  GemmArgs g{A, B, C, M, N, K, sa_m, sa_k, sa_z, sb_k, sb_n, sb_z, sc_m, sc_n, sc_z,
-             S, per * kGK, S > 1 ? ws : nullptr, A2, B2, C2, Z, Zall};
-  dim3 grid((N + kH - 1) / kH, (M + kTcRows - 1) / kTcRows, Zall * S);
-  bf16_gemm_tc_kernel<<<grid, kTcRows, 0, st>>>(g, err);
-  if (partials) *partials = S;
-  if (S > 1 && !partials) {
-    const long long all = (long long)Z * M * N;
+  return GemmArgs{A, B, C, M, N, K, sa_m, sa_k, sa_z, sb_k, sb_n, sb_z, sc_m, sc_n, sc_z,
+                  S, per * kGK, S > 1 ? ws : nullptr, A2, B2, C2, Z, Zall};
+}
+
+// the partial tiles of a split summed into C (and C2)
+static cudaError_t gemm_reduce(const GemmArgs& g, cudaStream_t st) {
+  if (g.S > 1) {
+    const long long all = (long long)g.Z * g.M * g.N;
     gemm_splitk_reduce<<<(int)std::min<long long>((all + 255) / 256, 1024), 256, 0, st>>>(
-        ws, C, M, N, Z, S, sc_m, sc_n, sc_z);
+        g.ws, g.C, g.C2, g.z2, g.M, g.N, g.Z, g.S, g.sc_m, g.sc_n, g.sc_z);
   }
   return cudaGetLastError();
+}
+
+static cudaError_t gemm(cudaStream_t st, int* err, float* ws, long long ws_elems,
+                        const __nv_bfloat16* A, const __nv_bfloat16* B, float* C, int M, int N,
+                        int K, long long sa_m, long long sa_k, long long sa_z, long long sb_k,
+                        long long sb_n, long long sb_z, long long sc_m, long long sc_n,
+                        long long sc_z, int Z) {
+  const GemmArgs g = gemm_plan(ws, ws_elems, A, B, C, M, N, K, sa_m, sa_k, sa_z, sb_k, sb_n, sb_z,
+                               sc_m, sc_n, sc_z, Z);
+  cudaError_t e = cudaFuncSetAttribute(bf16_gemm_tc_kernel,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, kGSmem);
+  if (e != cudaSuccess) return e;
+  dim3 grid((N + kH - 1) / kH, (M + kTcRows - 1) / kTcRows, Z * g.S);
+  bf16_gemm_tc_kernel<<<grid, kGThreads, kGSmem, st>>>(g, err);
+  return gemm_reduce(g, st);
 }
 
 static int nblk(long long n, int t = 256) { return (int)((n + t - 1) / t); }
@@ -1249,10 +1374,10 @@ static cudaError_t forward(mdeos_surrogate* s, int B, float* Y, cudaStream_t st)
   return cudaGetLastError();
 }
 
-// Gradients of the mean-squared error of one batch (X, T: device float[B][2]) in three
-// launches: the fused forward and backward pass per 128 samples, the sums over the batch,
-// the two 128 x 128 weight gradients.  The latter are left as *splits partial tiles in
-// s->ws for mlp_adam, or (splits == nullptr, or one split) added into s->G.
+// Gradients of the mean-squared error of one batch (X, T: device float[B][2]) in two
+// launches: the fused forward and backward pass per 128 samples, the sums over the batch.
+// With `splits` the two 128 x 128 weight gradients are left as *splits partial tiles in
+// s->ws for mlp_adam (one split: in s->G), else they are added into s->G.
 static cudaError_t gradients(mdeos_surrogate* s, const float* X, const float* T, int B, float* loss,
                              int* splits, cudaStream_t st) {
   const int E = s->E;
@@ -1261,26 +1386,28 @@ static cudaError_t gradients(mdeos_surrogate* s, const float* X, const float* T,
     cudaError_t e = cudaFuncSetAttribute(mlp_train_tc_kernel,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize, kTrSmem);
     if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(mlp_column_grads, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               kColSmem);
+      e = cudaFuncSetAttribute(mlp_batch_sums, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               kSumSmem);
     if (e != cudaSuccess) return e;
     s->train_ready = true;
   }
   __nv_bfloat16* dZ2 = reinterpret_cast<__nv_bfloat16*>(s->Z);  // Z itself is not used here
   TrainArgs a{X, T, s->P, s->W1b, s->W2b, s->W3b, s->W4b, s->W2t, s->W3t,
-              s->H1, s->H2, s->H3, s->dZb, dZ2, s->dZf, s->dY, loss, B, s->err};
+              s->H1, s->H2, s->H3, s->dZb, dZ2, s->dZf, s->dY, s->Y, B, s->err};
   dim3 grid((B + kTcRows - 1) / kTcRows, E);
   mlp_train_tc_kernel<<<grid, kTrThreads, kTrSmem, st>>>(a);
-  mlp_column_grads<<<dim3(kH / 32, E), 256, kColSmem, st>>>(s->dY, s->H3, s->dZb, dZ2, s->dZf, X, s->G, B);
   // dW3 = dZ3^T H2: A(m=o, k=b) = dZ3[b][o], B(k=b, n=j) = H2[b][j]; dW2 = dZ2^T H1 alike
-  if (splits)
-    return gemm(st, s->err, s->ws, s->ws_elems, s->dZb, s->H2, s->G + kOffW3, kH, kH, B, 1, kH, sz,
-                kH, 1, sz, kH, 1, kNParam, E, dZ2, s->H1, s->G + kOffW2, splits);
-  cudaError_t e = gemm(st, s->err, s->ws, s->ws_elems, s->dZb, s->H2, s->G + kOffW3, kH, kH, B, 1,
-                       kH, sz, kH, 1, sz, kH, 1, kNParam, E);
-  if (e != cudaSuccess) return e;
-  return gemm(st, s->err, s->ws, s->ws_elems, dZ2, s->H1, s->G + kOffW2, kH, kH, B, 1, kH, sz, kH, 1,
-              sz, kH, 1, kNParam, E);
+  const GemmArgs g = gemm_plan(s->ws, s->ws_elems, s->dZb, s->H2, s->G + kOffW3, kH, kH, B, 1, kH,
+                               sz, kH, 1, sz, kH, 1, kNParam, E, dZ2, s->H1, s->G + kOffW2);
+  // the tiles' squared errors go through Y, which only inference uses
+  const ColArgs c{s->dY, s->dZf, X, s->H3, s->dZb, dZ2, s->G, B, s->Y, (int)(grid.x * grid.y), loss};
+  const int ncol = 2 * (kH / 32) * E;
+  mlp_batch_sums<<<ncol + g.Z * g.S, kGThreads, kSumSmem, st>>>(c, g, ncol, s->err);
+  if (splits) {
+    *splits = g.S;
+    return cudaGetLastError();
+  }
+  return gemm_reduce(g, st);
 }
 
 static cudaError_t cast_weights(mdeos_surrogate* s, cudaStream_t st) {
@@ -1331,8 +1458,6 @@ extern "C" mdeos_status mdeos_surrogate_create(mdeos_handle* h, int32_t n_models
   dalloc((void**)&s->dY, EB * 2 * 4);
   dalloc((void**)&s->loss, 256);
   dalloc((void**)&s->Xp, (size_t)max_batch * 2 * 8);
-  dalloc((void**)&s->mean, (size_t)max_batch * 2 * 8);
-  dalloc((void**)&s->sd, (size_t)max_batch * 2 * 8);
   dalloc((void**)&s->err, 256);
   s->ws_elems = 2LL * kMaxSplitK * E * kH * kH;  // two products' partial tiles
   dalloc((void**)&s->ws, (size_t)s->ws_elems * 4);
@@ -1431,9 +1556,8 @@ extern "C" mdeos_status mdeos_surrogate_grads(mdeos_surrogate* s, const double* 
   cudaStream_t st = handle_stream(s->h);
   mdeos_status ms = load_batch(s, x, y, n, st);
   if (ms != MDEOS_OK) return ms;
-  SCK(cudaMemsetAsync(s->loss, 0, 4, st));
   SCK(gradients(s, s->X, s->T, n, s->loss, nullptr, st));
-  count_launch(s->h, 6);
+  count_launch(s->h, 3);
   if (grads)
     SCK(cudaMemcpyAsync(grads, s->G, (size_t)s->E * kNParam * 4, cudaMemcpyDeviceToHost, st));
   float l = 0.f;
@@ -1508,7 +1632,6 @@ extern "C" mdeos_status mdeos_surrogate_train(mdeos_surrogate* s, const double* 
       float* dx = tb.d[turn];
       float* dl = tb.d_loss + turn * kSegBatches;
       SCK(cudaMemcpyAsync(dx, hx, rows * 16, cudaMemcpyHostToDevice, st));
-      SCK(cudaMemsetAsync(dl, 0, (size_t)nb * 4, st));
       for (int k = 0; k < nb; ++k) {
         const float* bx = dx + 2 * (size_t)k * batch;
         int S = 1;
@@ -1520,7 +1643,7 @@ extern "C" mdeos_status mdeos_surrogate_train(mdeos_surrogate* s, const double* 
                    (float)(1.0 - std::pow(0.999, (double)s->step))};
         mlp_adam<<<dim3(nblk(kNParam), s->E), 256, 0, st>>>(a);
         SCK(cudaGetLastError());
-        count_launch(s->h, 4);
+        count_launch(s->h, 3);
       }
       SCK(cudaMemcpyAsync(tb.h_loss + turn * kSegBatches, dl, (size_t)nb * 4,
                           cudaMemcpyDeviceToHost, st));

@@ -135,16 +135,16 @@ def test_hydro_slabs_equal_the_oracle_bitwise(m, h, nz):
             assert s["t"] == o.t
 
 
-@pytest.mark.parametrize("n", [1, 2, 63, 127, 128, 129, 257, 640])
+@pytest.mark.parametrize("n", [1, 2, 63, 127, 128, 129, 257, 640, 4203])
 def test_gradients_of_ragged_batches_match_oracle(m, h, n):
     """The bound of the 300-sample gradient test (bf16 roundings one ulp apart), for batches
-    around the 128-sample tiles, the K chunks of 64 and the split of K."""
+    around the 128-sample tiles, the K chunks of 64, the split of K and its rings."""
     rng = np.random.default_rng(n)
     p = S.init_params(5, 2).astype(np.float32).astype(np.float64)
     norm = np.array([0.75, -1.0, 0.25, 2.0, 1.5, 1.2, 2.0, 0.6])
     x = np.stack([rng.uniform(0.3, 1.2, n), rng.uniform(-5.0, 3.0, n)], axis=1)
     y = np.stack([x[:, 0] * (x[:, 1] + 3.0), 0.5 * x[:, 1] + 2.0], axis=1)
-    with m.Surrogate(h, 2, 640, seed=1) as sg:
+    with m.Surrogate(h, 2, 4203, seed=1) as sg:
         sg.set_params(p, norm)
         g, loss = sg.grads(x, y)
         g2, _ = sg.grads(x, y)
