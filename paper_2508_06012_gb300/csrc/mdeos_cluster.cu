@@ -2,6 +2,10 @@
 // unit of its own: its CTAs have few warps with work, so its force passes fetch their lists
 // further ahead (MDEOS_LIST_AHEAD, mdeos_device.cuh).
 #define MDEOS_LIST_AHEAD 3
+#include <array>
+#include <map>
+#include <mutex>
+
 #include "mdeos_big.cuh"
 
 namespace mdeos {
@@ -57,8 +61,22 @@ cudaError_t set_cluster_attributes(int dyn) {
   return cudaFuncSetAttribute(eos_cluster_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, dyn);
 }
 
-// clusters of `cluster` full-size CTAs (one per SM) that the GPU holds at once
+// Clusters of `cluster` full-size CTAs (one per SM) that the current device holds at once: a
+// property of the device and the launch, so it is asked once per process (50 us a question,
+// a fifth of creating a handle for three of them).
 cudaError_t max_resident_clusters(int cluster, int smem, int* n) {
+  static std::mutex mu;
+  static std::map<std::array<int, 3>, int> known;
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  std::lock_guard<std::mutex> lock(mu);
+  const std::array<int, 3> key{dev, cluster, smem};
+  const auto it = known.find(key);
+  if (it != known.end()) {
+    *n = it->second;
+    return cudaSuccess;
+  }
   cudaLaunchConfig_t lc = {};
   lc.gridDim = dim3((unsigned)cluster, 1, 1);
   lc.blockDim = dim3(kCtaThreads, 1, 1);
@@ -70,7 +88,9 @@ cudaError_t max_resident_clusters(int cluster, int smem, int* n) {
   at[0].val.clusterDim.z = 1;
   lc.attrs = at;
   lc.numAttrs = 1;
-  return cudaOccupancyMaxActiveClusters(n, eos_cluster_kernel, &lc);
+  e = cudaOccupancyMaxActiveClusters(n, eos_cluster_kernel, &lc);
+  if (e == cudaSuccess) known[key] = *n;
+  return e;
 }
 
 cudaError_t launch_eos_cluster(const BoxDesc* boxes, const WorkItem* items, int nitems,
