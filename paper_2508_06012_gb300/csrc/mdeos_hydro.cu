@@ -2,10 +2,11 @@
 // grid, closed by an ideal gas, the Mie-Grueneisen form of Eq. 1, or the batched
 // atomistic EOS of this library (one request per zone and step, Sec. III).
 //
-// The hydro state is a few thousand zones: one CTA of 1024 threads runs a whole
-// step (phases separated by __syncthreads), and the analytic closures run many
-// steps per launch.  With the MD closure a step is one persistent EOS batch
-// launch (milliseconds of MD per zone) followed by one hydro launch (~10 us).
+// The hydro state is a few thousand zones: a thread-block cluster runs a whole step on
+// slabs of it in shared memory (meshes above about 35,000 zones: one CTA on global
+// memory), and the analytic closures run many steps per launch.  With the MD closure a
+// step is one persistent EOS batch launch (milliseconds of MD per zone) followed by one
+// hydro launch (~6 us).
 //
 // Arithmetic is FP64 in one fixed evaluation order per expression; this file is
 // compiled with -fmad=false so no multiply-add is contracted, making every
