@@ -471,10 +471,10 @@ struct ListReader {
 // selects of the branch-free form only add to it (energy + virial, 4000 atoms: 164k SM cycles
 // in groups, 146k one by one); a pass with the minimum image and the virial of every pair
 // is bound by issue slots, and a branch per entry costs more than the selects (500 atoms,
-// eight boxes per CTA: 149k one by one, 136k in groups), but not with several threads per
-// atom: their sub-lists are two or three words, a third of them padding, which a branch
-// skips (1216 boxes of 256 atoms, 420 steps: rho 1.0 37.4 ms in groups, 36.2 one by one; 0.5
-// 28.8 and 29.7; 152 boxes, rho 0.75: 6.4 and 6.1).
+// eight boxes per CTA: 149k one by one, 136k in groups).  There a group of padding alone is
+// skipped: with several threads per atom a sub-list is two or three words, a third of them
+// padding (1216 boxes of 300 atoms, 420 steps: rho 0.5 42.4 ms one by one, 40.1-40.8 in groups with
+// the skip; rho 1.0 61.5 and 59.9-60.5).
 template <bool EN, bool VIR, bool MI>
 constexpr bool kPairInGroups = MDEOS_LIST_AHEAD > 1 || (VIR && MI);
 
@@ -586,7 +586,8 @@ __device__ __noinline__ FSums force_pass(uint32_t xs_a, float4* fs, const uint16
         const uint4* lp = reinterpret_cast<const uint4*>(nl) + u;
         const size_t wst = (size_t)npad * tpa;  // words between word kb and kb + 1
         const int meta = __float_as_int(cw);
-        const int nw = CODED ? meta & 0xfff : (sub_entries(meta, tpa, p) + 7) >> 3;
+        const int cnt = CODED ? 0 : sub_entries(meta, tpa, p);
+        const int nw = CODED ? meta & 0xfff : (cnt + 7) >> 3;
         ListReader rd(lp, wst, nw);
         if (CODED) {
           // home shift along an axis: +L for atoms in the lower half of the grid
@@ -654,13 +655,15 @@ __device__ __noinline__ FSums force_pass(uint32_t xs_a, float4* fs, const uint16
 #pragma unroll 1
           for (int kb = 0; kb < nw; ++kb) {
             const uint4 cur = rd.next();
-            if (kPairInGroups<EN, VIR, true> && (MDEOS_LIST_AHEAD > 1 || tpa == 1)) {
+            if constexpr (kPairInGroups<EN, VIR, true>) {
 #pragma unroll
-              for (int g = 0; g < 8; g += kPairGroup)
+              for (int g = 0; g < 8; g += kPairGroup) {
+                if (MDEOS_LIST_AHEAD == 1 && kb * 8 + g >= cnt) break;  // padding only
                 pair_group<kPairGroup, EN, VIR, true>(
                     [&](int q) { return ld_shared4(xs_a + 16u * (uint32_t)word_entry(cur, g + q)); },
                     [&](int q) { return word_entry(cur, g + q) != i; }, xi.x, xi.y, xi.z, L, invL,
                     c, fx, fy, fz, e, w, np);
+              }
             } else {
 #pragma unroll
               for (int g = 0; g < 8; ++g) {
@@ -717,7 +720,9 @@ __device__ __noinline__ FSums force_pass(uint32_t xs_a, float4* fs, const uint16
       if (p == 0) fs[i] = make_float4(fx, fy, fz, cw);
       if (EN) {
         bad |= !(fabsf(e) < 1e9f);
-        bool small = fabsf(e) < kFixFast;  // one range test for all the atom's values
+        // one range test for all the atom's values; with several threads per atom in a full
+        // CTA a pass is so short of issue slots that the conversion instruction is the cheaper
+        bool small = fabsf(e) < kFixFast && (MDEOS_LIST_AHEAD > 1 || tpa == 1);
         if (VIR) {
           const float wn = fabsf(w[0]) + fabsf(w[1]) + fabsf(w[2]);
           bad |= !(wn < 1e9f);
