@@ -95,12 +95,6 @@ __device__ __forceinline__ float rcp_approx(float x) {
   return y;
 }
 
-__device__ __forceinline__ float warp_sum(float v) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-  return v;
-}
-
 // 64-bit fixed point of the box sums: v * 2^32 rounded to the nearest integer
 // (exact for |v| >= 2^-9, where the scaled float is already an integer).  Values
 // are kept below 2^30 in magnitude by the callers' finiteness checks.
@@ -490,15 +484,6 @@ __device__ __forceinline__ void st_shared_u16(uint32_t a, int v) {
 
 __device__ __forceinline__ void st_shared_s32(uint32_t a, int v) {
   asm volatile("st.shared.s32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
-}
-
-__device__ __forceinline__ uint4 ld_shared_u4(uint32_t a) {
-  uint4 v;
-  asm volatile("ld.shared.v4.u32 {%0, %1, %2, %3}, [%4];"
-               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-               : "r"(a)
-               : "memory");
-  return v;
 }
 
 __device__ __forceinline__ int ld_shared_u16(uint32_t a) {
@@ -891,12 +876,6 @@ __device__ __forceinline__ int ld_shared_s32(uint32_t a) {
   int v;
   asm volatile("ld.shared.s32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
   return v;
-}
-
-__device__ __forceinline__ void st_shared_v4(uint32_t a, float4 v) {
-  asm volatile("st.shared.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(a), "f"(v.x), "f"(v.y), "f"(v.z),
-               "f"(v.w)
-               : "memory");
 }
 
 // List layout shared by the searches and the force pass.  Entries are uint16 slots,
