@@ -349,7 +349,7 @@ static __device__ __noinline__ bool big_search(const float4* x, uint32_t sx_a, c
         if (d == 4 && part == 1) e1 = si;
         if (part == 2) e0 = si + 1;
         const float sx = part == 0 ? -L : (part == 3 ? L : 0.f);
-        if (__any_sync(__activemask(), sx != 0.f || sy != 0.f || sz != 0.f))
+        if (sx != 0.f || sy != 0.f || sz != 0.f)
           big_scan<WIN, true>(x, sx_a, l2, r, e0, e1, xi, sx, sy, sz, rs2);
         else
           big_scan<WIN, false>(x, sx_a, l2, r, e0, e1, xi, 0.f, 0.f, 0.f, rs2);
@@ -561,8 +561,10 @@ __device__ __noinline__ FSums big_force_pass(const float4* x, uint32_t sx_a, int
     float fx = 0.f, fy = 0.f, fz = 0.f;
     const uint4* p = nl + s;
     uint4 q = nw > 0 ? __ldcg(p) : make_uint4(0u, 0u, 0u, 0u);
-    const bool face = __any_sync(__activemask(), (__float_as_int(cw) & kBigFace) != 0);
-    if (face) {
+    // the warp's lanes of this turn (those up to s1) meet and decide together
+    const int left = s1 - (s - (int)(threadIdx.x & 31));
+    const unsigned turn = left >= 32 ? 0xffffffffu : (1u << left) - 1u;
+    if (__any_sync(turn, (__float_as_int(cw) & kBigFace) != 0)) {
 #pragma unroll 1
       for (int kb = 0; kb < nw; ++kb) {
         const uint4 cur = q;
