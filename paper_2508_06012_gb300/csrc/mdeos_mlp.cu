@@ -185,7 +185,8 @@ __device__ __forceinline__ void column_grads(const ColArgs& a, int e, int block,
       cp_async<8>(s.p[q], part == 0 ? a.dY + (r0 + b0 + q) * 2 : a.X + (long long)(b0 + q) * 2);
   };
   if (e == 0 && block == 0 && part == 0 && warp == 7 && lane == 0) {
-    // in order (reproducible), the rounding errors of the sum added at its end
+    // in order (reproducible), the rounding errors of the sum added at its end (a sum that
+    // has overflowed has none: its difference of infinities would make it a NaN)
     float l = 0.f, c = 0.f;
 #pragma unroll 8
     for (int k = 0; k < a.npart; ++k) {
@@ -193,7 +194,7 @@ __device__ __forceinline__ void column_grads(const ColArgs& a, int e, int block,
       c += (l - (n - d)) + (t - d);
       l = n;
     }
-    *a.loss = l + c;
+    *a.loss = isfinite(l) ? l + c : l;
   }
   const int nk = (B + kColRows - 1) / kColRows;
   for (int k = 0; k < kColStages - 1; ++k) {

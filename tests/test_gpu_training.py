@@ -1,0 +1,48 @@
+"""Training of the surrogate (mdeos_surrogate_train, mdeos_surrogate_grads): what its fused
+kernels and staged segments must keep, beside the comparisons with the oracle."""
+import numpy as np
+import pytest
+
+from oracle import surrogate as S
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def m():
+    import torch
+    if not torch.cuda.is_available():
+        pytest.skip("no GPU")
+    import paper_2508_06012_gb300 as m
+    m.build()
+    return m
+
+
+@pytest.fixture(scope="module")
+def h(m):
+    h = m.mdeos_create()
+    yield h
+    m.mdeos_destroy(h)
+
+
+IDENTITY = np.array([0.0, 0.0, 1.0, 1.0, 0.0, 0.0, 1.0, 1.0])
+
+
+def _inputs(n, seed):
+    rng = np.random.default_rng(seed)
+    return np.stack([rng.uniform(-1.0, 1.0, n), rng.uniform(-1.0, 1.0, n)], axis=1)
+
+
+@pytest.mark.parametrize("n", [100, 700])
+def test_an_overflowing_loss_is_infinite(m, h, n):
+    """Errors whose square exceeds FP32 make the sum of squares +inf (not NaN), wherever
+    their samples lie and however many other tiles follow."""
+    x = _inputs(n, n)
+    for at in (0, n // 2, n - 1):
+        y = np.zeros((n, 2))
+        y[at, 1] = 1e30
+        with m.Surrogate(h, 2, n, seed=3) as sg:
+            sg.set_params(S.init_params(2, 2).astype(np.float32), IDENTITY)
+            g, loss = sg.grads(x, y)
+            assert np.isfinite(g).all() and loss == np.inf
+            assert sg.train(x, y, epochs=1, batch=n, lr=1e-6, seed=1, set_norm=False)[0] == np.inf
