@@ -608,18 +608,36 @@ static void pinned_put(mdeos_handle* h, PinnedBlock& b) {
   b.size = 0;
 }
 
+// give the handle's list scratch back
+static mdeos_status drop_scratch(mdeos_handle* h) {
+  if (!h->d_nl) return MDEOS_OK;
+  CK(cudaStreamSynchronize(h->stream));
+  CK(cudaFree(h->d_nl));
+  h->used_bytes -= h->nl_bytes;
+  h->d_nl = nullptr;
+  h->nl_bytes = 0;
+  return MDEOS_OK;
+}
+
+// Room under the HBM budget for `bytes` more, beside `scratch` bytes of list scratch that this
+// call needs.  The handle may hold more scratch than that (an earlier cluster plan's: several
+// per box); where only that stands in the way it is given back, so that a call never fails
+// for the room an earlier one spent on speed.
+static mdeos_status make_room(mdeos_handle* h, size_t bytes, size_t scratch, const char* what) {
+  const size_t budget = h->cfg.hbm_budget_bytes;
+  if (budget == 0 || h->used_bytes + bytes <= budget) return MDEOS_OK;
+  if (h->nl_bytes <= scratch || h->used_bytes - h->nl_bytes + scratch + bytes > budget)
+    return fail(MDEOS_ENOMEM, what);
+  return drop_scratch(h);
+}
+
 static mdeos_status ensure_scratch(mdeos_handle* h, size_t bytes) {
   if (bytes <= h->nl_bytes) return MDEOS_OK;
   const size_t extra = bytes - h->nl_bytes;
   if (h->cfg.hbm_budget_bytes && h->used_bytes + extra > h->cfg.hbm_budget_bytes)
     return fail(MDEOS_ENOMEM, "neighbour-list scratch exceeds the HBM budget");
-  if (h->d_nl) {
-    CK(cudaStreamSynchronize(h->stream));
-    CK(cudaFree(h->d_nl));
-    h->used_bytes -= h->nl_bytes;
-    h->d_nl = nullptr;
-    h->nl_bytes = 0;
-  }
+  mdeos_status st = drop_scratch(h);
+  if (st != MDEOS_OK) return st;
   CK(cudaMalloc(&h->d_nl, bytes));
   h->nl_bytes = bytes;
   h->used_bytes += bytes;
@@ -804,8 +822,8 @@ extern "C" mdeos_status mdeos_submit(mdeos_handle* h, const mdeos_request* reqs,
   const size_t off_res = (in_bytes + 255) & ~size_t(255);
   const size_t off_cnt = off_res + (((size_t)n * sizeof(mdeos_result) + 255) & ~size_t(255));
   const size_t dev_bytes = off_cnt + 256;
-  if (h->cfg.hbm_budget_bytes && h->used_bytes + dev_bytes > h->cfg.hbm_budget_bytes)
-    return fail(MDEOS_ENOMEM, "batch exceeds the HBM budget");
+  const size_t scratch = nb > 0 ? (size_t)plan.grid * plan.nl_per_cta * sizeof(uint16_t) : 0;
+  if ((st = make_room(h, dev_bytes, scratch, "batch exceeds the HBM budget")) != MDEOS_OK) return st;
   if ((st = pinned_get(h, in_bytes, t.h_in)) != MDEOS_OK) return st;
   if ((st = pinned_get(h, (size_t)n * sizeof(mdeos_result), t.h_out)) != MDEOS_OK) {
     pinned_put(h, t.h_in);
@@ -817,7 +835,6 @@ extern "C" mdeos_status mdeos_submit(mdeos_handle* h, const mdeos_request* reqs,
   h->last_h2d = 0;
   h->last_d2h = 0;
   if (t.any_device) {
-    const size_t scratch = (size_t)plan.grid * plan.nl_per_cta * sizeof(uint16_t);
     if ((st = ensure_scratch(h, scratch)) != MDEOS_OK) {
       pinned_put(h, t.h_in);
       pinned_put(h, t.h_out);
@@ -861,9 +878,9 @@ static mdeos_status run_plan_sync(mdeos_handle* h, const Plan& plan, int n, mdeo
   const size_t off_res = (off_items + ni * sizeof(WorkItem) + 255) & ~size_t(255);
   const size_t off_cnt = off_res + (((size_t)n * sizeof(mdeos_result) + 255) & ~size_t(255));
   const size_t dev_bytes = off_cnt + 256;
-  if (h->cfg.hbm_budget_bytes && h->used_bytes + dev_bytes > h->cfg.hbm_budget_bytes)
-    return fail(MDEOS_ENOMEM, "re-run exceeds the HBM budget");
-  mdeos_status st = ensure_scratch(h, (size_t)plan.grid * plan.nl_per_cta * sizeof(uint16_t));
+  const size_t scratch = (size_t)plan.grid * plan.nl_per_cta * sizeof(uint16_t);
+  mdeos_status st = make_room(h, dev_bytes, scratch, "re-run exceeds the HBM budget");
+  if (st == MDEOS_OK) st = ensure_scratch(h, scratch);
   if (st != MDEOS_OK) return st;
   std::vector<char> in(off_items + ni * sizeof(WorkItem));
   std::memcpy(in.data(), plan.boxes.data(), nb * sizeof(BoxDesc));
@@ -1005,9 +1022,9 @@ extern "C" mdeos_status mdeos_batch_create(mdeos_handle* h, const mdeos_request*
   const size_t off_nl = off_cnt + 256;
   const size_t nl_bytes = (size_t)p.grid * p.nl_per_cta * sizeof(uint16_t);
   const size_t total = off_nl + nl_bytes;
-  if (h->cfg.hbm_budget_bytes && h->used_bytes + total > h->cfg.hbm_budget_bytes) {
+  if ((st = make_room(h, total, 0, "batch exceeds the HBM budget")) != MDEOS_OK) {
     delete b;
-    return fail(MDEOS_ENOMEM, "batch exceeds the HBM budget");
+    return st;
   }
   cudaError_t e = cudaMalloc(&b->d_mem, total);
   if (e != cudaSuccess) {
@@ -1333,12 +1350,14 @@ mdeos_status eval_into_device(mdeos_handle* h, const mdeos_request* reqs, int n,
   const size_t in_bytes = off_items + ni * sizeof(WorkItem);
   const size_t off_cnt = (in_bytes + 255) & ~size_t(255);
   const size_t dev_bytes = off_cnt + 256;
+  const size_t scratch = nb > 0 ? (size_t)plan.grid * plan.nl_per_cta * sizeof(uint16_t) : 0;
   bool rejected = false;
   for (int i = 0; i < n; ++i) rejected = rejected || plan.status[i] != MDEOS_OK;
   const size_t host_bytes = std::max(in_bytes, rejected ? (size_t)n * sizeof(mdeos_result) : 0);
   if (dev_bytes > h->eval_bytes) {
-    if (h->cfg.hbm_budget_bytes && h->used_bytes + dev_bytes - h->eval_bytes > h->cfg.hbm_budget_bytes)
-      return fail(MDEOS_ENOMEM, "batch exceeds the HBM budget");
+    if ((st = make_room(h, dev_bytes - h->eval_bytes, scratch, "batch exceeds the HBM budget")) !=
+        MDEOS_OK)
+      return st;
     if (h->d_eval) CK(cudaFree(h->d_eval));
     h->used_bytes -= h->eval_bytes;
     h->d_eval = nullptr;
@@ -1365,7 +1384,6 @@ mdeos_status eval_into_device(mdeos_handle* h, const mdeos_request* reqs, int n,
   if (nb == 0) return MDEOS_OK;
   std::memcpy(h->eval_pinned.p, plan.boxes.data(), nb * sizeof(BoxDesc));
   std::memcpy((char*)h->eval_pinned.p + off_items, plan.items.data(), ni * sizeof(WorkItem));
-  const size_t scratch = (size_t)plan.grid * plan.nl_per_cta * sizeof(uint16_t);
   if ((st = ensure_scratch(h, scratch)) != MDEOS_OK) return st;
   CK(cudaMemcpyAsync(d, h->eval_pinned.p, in_bytes, cudaMemcpyHostToDevice, h->stream));
   CK(cudaMemsetAsync(d + off_cnt, 0, sizeof(int), h->stream));

@@ -210,3 +210,29 @@ def test_cluster_scratch_stays_within_the_budget(m):
         assert m.mdeos_batch_info(batch)["ctas"] == 1
         m.mdeos_batch_destroy(batch)
     assert ra["status"][0] == 0 and ra.tobytes() == rb.tobytes()
+
+
+def test_cluster_scratch_gives_way_to_later_calls(m):
+    """After a box has run on a cluster of 8 whose list scratch fills the budget, a batch of
+    many boxes (large tables) and a device-resident batch still get their room, and the box
+    runs again with the same answer."""
+    q = [dict(rho=0.8, e=m.e_from_temperature(1.5, 4000), natoms=4000, steps_equil=20, steps_avg=20,
+              seed=5)]
+    many = [dict(rho=0.3, e=m.e_from_temperature(1.5, 32), natoms=32, steps_equil=2, steps_avg=2,
+                 seed=k) for k in range(4000)]
+    with m.Engine() as a:
+        base = m.mdeos_stats(a.h)["device_bytes"]
+        ref = a.evaluate(q)
+        per = (m.mdeos_stats(a.h)["device_bytes"] - base) // 8
+        rmany = a.evaluate(many)
+    with m.Engine(hbm_budget_bytes=base + 8 * per + per // 2) as a:
+        assert a.evaluate(q).tobytes() == ref.tobytes()
+        assert m.mdeos_stats(a.h)["device_bytes"] >= base + 8 * per
+        assert a.evaluate(many).tobytes() == rmany.tobytes()
+        assert a.evaluate(q).tobytes() == ref.tobytes()
+        b = m.mdeos_batch_create(a.h, q + q)
+        m.mdeos_batch_launch(b)
+        assert m.mdeos_batch_results(b, 2)[:1].tobytes() == ref.tobytes()
+        assert m.mdeos_stats(a.h)["device_bytes"] <= base + 8 * per + per // 2
+        m.mdeos_batch_destroy(b)
+        assert a.evaluate(q).tobytes() == ref.tobytes()
