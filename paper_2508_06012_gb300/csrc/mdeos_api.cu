@@ -646,17 +646,20 @@ static mdeos_status ensure_scratch(mdeos_handle* h, size_t bytes) {
 
 // Plan a batch of handle h for a launch that takes `extra` more device bytes (own_scratch:
 // and its list scratch from them rather than from the handle).  A cluster plan keeps a list
-// scratch per CTA, several per box: where the HBM budget has no room for that, one CTA per
-// box.
+// scratch per CTA, several per box: where the HBM budget has no room for that, clusters of
+// half as many CTAs, down to one CTA per box.
 static mdeos_status plan_for_handle(mdeos_handle* h, const mdeos_request* reqs, int n, Plan& plan,
                                     size_t extra, bool own_scratch, const int* cap_min = nullptr) {
-  mdeos_status st = make_plan(reqs, n, h->cfg, h->nsm, h->smem_max, plan, true, &h->tuned_skin,
-                              cap_min, true, h->fit);
-  if (st != MDEOS_OK || plan.cluster == 1 || h->cfg.hbm_budget_bytes == 0) return st;
-  const size_t need = (size_t)plan.grid * plan.nl_per_cta * sizeof(uint16_t);
-  const size_t held = own_scratch ? 0 : h->nl_bytes;
-  if (h->used_bytes + extra + (need > held ? need - held : 0) <= h->cfg.hbm_budget_bytes) return st;
-  return make_plan(reqs, n, h->cfg, h->nsm, h->smem_max, plan, true, &h->tuned_skin, cap_min);
+  mdeos_config c = h->cfg;
+  for (;;) {
+    mdeos_status st = make_plan(reqs, n, c, h->nsm, h->smem_max, plan, true, &h->tuned_skin,
+                                cap_min, true, h->fit);
+    if (st != MDEOS_OK || plan.cluster == 1 || c.hbm_budget_bytes == 0) return st;
+    const size_t need = (size_t)plan.grid * plan.nl_per_cta * sizeof(uint16_t);
+    const size_t held = own_scratch ? 0 : h->nl_bytes;
+    if (h->used_bytes + extra + (need > held ? need - held : 0) <= c.hbm_budget_bytes) return st;
+    c.max_cluster = plan.cluster / 2;
+  }
 }
 
 // upper bound of a batch's boxes, items, results and counter

@@ -212,6 +212,28 @@ def test_cluster_scratch_stays_within_the_budget(m):
     assert ra["status"][0] == 0 and ra.tobytes() == rb.tobytes()
 
 
+@pytest.mark.parametrize("n", [4000, 16000])
+def test_budget_halves_the_cluster_until_its_scratch_fits(m, n):
+    """A budget with room for 4 (2, 1) list scratches of a box whose default is a cluster of
+    8 plans 4 (2, 1) CTAs, not one."""
+    q = [dict(rho=0.8, e=m.e_from_temperature(1.5, n), natoms=n, steps_equil=20, steps_avg=20,
+              seed=5)]
+    with m.Engine() as a:
+        base = m.mdeos_stats(a.h)["device_bytes"]
+        b = m.mdeos_batch_create(a.h, q)
+        info = m.mdeos_batch_info(b)
+        m.mdeos_batch_destroy(b)
+    assert info["ctas"] == 8
+    per = info["scratch_bytes"] // 8
+    for ctas in (8, 4, 2, 1):
+        # the tables of one request take far less than half a scratch
+        with m.Engine(hbm_budget_bytes=base + ctas * per + per // 2) as a:
+            b = m.mdeos_batch_create(a.h, q)
+            got = m.mdeos_batch_info(b)["ctas"]
+            m.mdeos_batch_destroy(b)
+        assert got == ctas
+
+
 def test_cluster_scratch_gives_way_to_later_calls(m):
     """After a box has run on a cluster of 8 whose list scratch fills the budget, a batch of
     many boxes (large tables) and a device-resident batch still get their room, and the box
