@@ -1232,25 +1232,19 @@ struct TrainBuffers {
   }
 };
 
-// Staging of predict's host arrays, kept with the surrogate: up to kIoRows queries at a
-// time (inputs 16 B; outputs a head with the error word, mean and sd 16 B each, 8 B per
-// model), grown to the largest chunk asked for.
+// Staging of predict's host arrays, allocated and given back with the surrogate: kIoRows
+// queries at a time, or max_batch if that is fewer (inputs 16 B; outputs a head with the error
+// word, mean and sd 16 B each, 8 B per model).  A predict allocates nothing: a cudaFree in it
+// could wait for whatever else runs on the device.
 constexpr int kIoRows = 1 << 18;
 constexpr size_t kIoHead = 256;
 struct PredictBuffers {
-  int rows = 0;
   char *h_in = nullptr, *h_out = nullptr, *d_out = nullptr;
-  cudaError_t reserve(int n, int E) {
-    if (n <= rows) return cudaSuccess;
-    release();
-    const size_t out = kIoHead + (size_t)n * (32 + 8 * (size_t)E);
-    cudaError_t e = cudaMallocHost((void**)&h_in, (size_t)n * 16);
+  cudaError_t allocate(int rows, int E) {
+    const size_t out = kIoHead + (size_t)rows * (32 + 8 * (size_t)E);
+    cudaError_t e = cudaMallocHost((void**)&h_in, (size_t)rows * 16);
     if (e == cudaSuccess) e = cudaMallocHost((void**)&h_out, out);
     if (e == cudaSuccess) e = cudaMalloc((void**)&d_out, out);
-    if (e == cudaSuccess)
-      rows = n;
-    else
-      release();
     return e;
   }
   void release() {
@@ -1258,7 +1252,6 @@ struct PredictBuffers {
     if (h_out) cudaFreeHost(h_out);
     if (d_out) cudaFree(d_out);
     h_in = h_out = d_out = nullptr;
-    rows = 0;
   }
 };
 
@@ -1462,6 +1455,7 @@ extern "C" mdeos_status mdeos_surrogate_create(mdeos_handle* h, int32_t n_models
   dalloc((void**)&s->err, 256);
   s->ws_elems = 2LL * kMaxSplitK * E * kH * kH;  // two products' partial tiles
   dalloc((void**)&s->ws, (size_t)s->ws_elems * 4);
+  if (e == cudaSuccess) e = s->io.allocate(std::min(max_batch, kIoRows), E);
   if (e != cudaSuccess) {
     mdeos_surrogate_destroy(s);
     return set_error(MDEOS_ECUDA, std::string("surrogate_create: ") + cudaGetErrorString(e));
@@ -1738,7 +1732,6 @@ extern "C" mdeos_status mdeos_surrogate_predict(mdeos_surrogate* s, const double
   // memory are staged and waited for one by one: eight of them took half of a 2000-query
   // call, 123 us; it takes 67 now.)
   const int chunk = std::min(s->maxB, kIoRows);
-  SCK(s->io.reserve(std::min(chunk, n), s->E));
   int err = 0;
   for (int off = 0; off < n; off += chunk) {
     const int B = std::min(chunk, n - off);

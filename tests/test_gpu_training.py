@@ -46,3 +46,33 @@ def test_an_overflowing_loss_is_infinite(m, h, n):
             g, loss = sg.grads(x, y)
             assert np.isfinite(g).all() and loss == np.inf
             assert sg.train(x, y, epochs=1, batch=n, lr=1e-6, seed=1, set_norm=False)[0] == np.inf
+
+
+def test_predict_allocates_no_device_memory(m, h):
+    """The first predict of a surrogate, and one larger than any before it, take no memory:
+    its staging comes with the surrogate (here 4 MB, so an allocation would show)."""
+    import torch
+    n = 1 << 16
+    x = _inputs(n, 1)
+    with m.Surrogate(h, 4, n, seed=1) as warm:   # the kernels' own first-use memory
+        warm.predict(x)
+    with m.Surrogate(h, 4, n, seed=1) as sg:
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        small = sg.predict(x[:100])
+        assert torch.cuda.mem_get_info()[0] == free
+        full = sg.predict(x)
+        assert torch.cuda.mem_get_info()[0] == free
+    assert np.array_equal(small[0], full[0][:100]) and np.array_equal(small[1], full[1][:100])
+
+
+def test_predict_in_pieces_of_its_staging(m, h):
+    """More queries than the staging holds, a ragged last piece: the answers of the same
+    queries asked in another order of pieces."""
+    n = 2 * 5000 + 777
+    x = _inputs(n, 2)
+    with m.Surrogate(h, 3, 5000, seed=1) as sg:
+        mean, sd, pm = sg.predict(x, per_model=True)
+        m2, s2, p2 = sg.predict(x[::-1], per_model=True)
+    assert np.array_equal(mean, m2[::-1]) and np.array_equal(sd, s2[::-1])
+    assert np.array_equal(pm, p2[:, ::-1])
