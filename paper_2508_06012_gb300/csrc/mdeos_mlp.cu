@@ -1188,33 +1188,29 @@ __global__ void debug_tanh_kernel(const float* x, float* y, int n) {
 
 using namespace mdeos;
 
-// batches of a training segment (see mdeos_surrogate_train), and its size where they are large
+// batches of a training segment (see mdeos_surrogate_train), and its samples where the batches
+// are large: whole batches, at least one
 constexpr int kSegBatches = 16;
-constexpr size_t kSegBytes = 16 << 20;
+constexpr int kSegRows = 1 << 16;
+static int train_seg(int batch) { return std::max(1, std::min(kSegBatches, kSegRows / batch)); }
 
-// Buffers of the training calls, kept with the surrogate (allocating pinned memory takes
-// longer than a short call's training) and given back with it: two segments of samples
-// (16 B each) and their batches' losses, grown to the largest segment asked for.
+// Buffers of the training calls, allocated and given back with the surrogate: two segments of
+// samples (16 B each) and their batches' losses.  A training call allocates nothing: a
+// cudaFree in it could wait for whatever else runs on the device.
 struct TrainBuffers {
-  size_t floats = 0;  // of one segment
   float *h[2] = {nullptr, nullptr}, *d[2] = {nullptr, nullptr};
   float *h_loss = nullptr, *d_loss = nullptr;  // [2][kSegBatches]
   cudaEvent_t done[2] = {nullptr, nullptr};
-  // no work of an earlier call uses them: training calls end with the stream idle
-  cudaError_t reserve(size_t n) {
-    if (n <= floats) return cudaSuccess;
-    release();
+  cudaError_t allocate(int max_batch) {
+    // the longest segment of any batch size
+    const size_t bytes = 16 * (size_t)std::max(max_batch, std::min(kSegRows, kSegBatches * max_batch));
     cudaError_t e = cudaMallocHost((void**)&h_loss, 2 * kSegBatches * 4);
     if (e == cudaSuccess) e = cudaMalloc((void**)&d_loss, 2 * kSegBatches * 4);
     for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
-      e = cudaMallocHost((void**)&h[k], n * 4);
-      if (e == cudaSuccess) e = cudaMalloc((void**)&d[k], n * 4);
+      e = cudaMallocHost((void**)&h[k], bytes);
+      if (e == cudaSuccess) e = cudaMalloc((void**)&d[k], bytes);
       if (e == cudaSuccess) e = cudaEventCreateWithFlags(&done[k], cudaEventDisableTiming);
     }
-    if (e == cudaSuccess)
-      floats = n;
-    else
-      release();
     return e;
   }
   void release() {
@@ -1228,7 +1224,6 @@ struct TrainBuffers {
     if (h_loss) cudaFreeHost(h_loss);
     if (d_loss) cudaFree(d_loss);
     h_loss = d_loss = nullptr;
-    floats = 0;
   }
 };
 
@@ -1456,6 +1451,7 @@ extern "C" mdeos_status mdeos_surrogate_create(mdeos_handle* h, int32_t n_models
   s->ws_elems = 2LL * kMaxSplitK * E * kH * kH;  // two products' partial tiles
   dalloc((void**)&s->ws, (size_t)s->ws_elems * 4);
   if (e == cudaSuccess) e = s->io.allocate(std::min(max_batch, kIoRows), E);
+  if (e == cudaSuccess) e = s->tb.allocate(max_batch);
   if (e != cudaSuccess) {
     mdeos_surrogate_destroy(s);
     return set_error(MDEOS_ECUDA, std::string("surrogate_create: ") + cudaGetErrorString(e));
@@ -1591,10 +1587,8 @@ extern "C" mdeos_status mdeos_surrogate_train(mdeos_surrogate* s, const double* 
   // turn, so a segment is gathered and normalised while the one before trains), and their
   // losses come back with them.
   const int nbat = n / batch;  // full batches only
-  const int seg = std::max(1, (int)std::min<size_t>(std::min(nbat, kSegBatches),
-                                                    kSegBytes / ((size_t)batch * 16)));
+  const int seg = train_seg(batch);
   TrainBuffers& tb = s->tb;
-  SCK(tb.reserve((size_t)seg * batch * 4));
   const float b1 = 0.9f, b2 = 0.999f;
   for (int ep = 0; ep < epochs; ++ep) {
     std::shuffle(perm.begin(), perm.end(), rng);

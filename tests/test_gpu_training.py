@@ -76,3 +76,21 @@ def test_predict_in_pieces_of_its_staging(m, h):
         m2, s2, p2 = sg.predict(x[::-1], per_model=True)
     assert np.array_equal(mean, m2[::-1]) and np.array_equal(sd, s2[::-1])
     assert np.array_equal(pm, p2[:, ::-1])
+
+
+def test_training_allocates_no_device_memory(m, h):
+    """The first training call of a surrogate takes no memory: its segments (2 MB each here, so
+    an allocation would show) come with the surrogate."""
+    import torch
+    batch = 1 << 17
+    x = _inputs(2 * batch, 1)
+    y = np.stack([x[:, 0] * x[:, 1], x[:, 1]], axis=1)
+    with m.Surrogate(h, 1, batch, seed=1) as warm:   # the kernels' own first-use memory
+        warm.train(x, y, epochs=1, batch=batch, set_norm=False)
+    with m.Surrogate(h, 1, batch, seed=1) as sg:
+        torch.cuda.synchronize()
+        free = torch.cuda.mem_get_info()[0]
+        sg.train(x[:200], y[:200], epochs=1, batch=100, set_norm=False)
+        assert torch.cuda.mem_get_info()[0] == free
+        sg.train(x, y, epochs=1, batch=batch, set_norm=False)
+        assert torch.cuda.mem_get_info()[0] == free
