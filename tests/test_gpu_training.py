@@ -1,5 +1,8 @@
 """Training of the surrogate (mdeos_surrogate_train, mdeos_surrogate_grads): what its fused
 kernels and staged segments must keep, beside the comparisons with the oracle."""
+import ctypes
+import subprocess
+
 import numpy as np
 import pytest
 
@@ -94,3 +97,72 @@ def test_training_allocates_no_device_memory(m, h):
         assert torch.cuda.mem_get_info()[0] == free
         sg.train(x, y, epochs=1, batch=batch, set_norm=False)
         assert torch.cuda.mem_get_info()[0] == free
+
+
+ORDER_SOURCE = """
+#include <algorithm>
+#include <cstdint>
+#include <random>
+#include <vector>
+// the sample order of each epoch of a training call: one generator, one permutation
+extern "C" void order(uint64_t seed, int n, int epochs, int* out) {
+  std::mt19937_64 rng(seed);
+  std::vector<int> perm(n);
+  for (int i = 0; i < n; ++i) perm[i] = i;
+  for (int e = 0; e < epochs; ++e) {
+    std::shuffle(perm.begin(), perm.end(), rng);
+    std::copy(perm.begin(), perm.end(), out + (size_t)e * n);
+  }
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def order(tmp_path_factory):
+    d = tmp_path_factory.mktemp("order")
+    (d / "order.cpp").write_text(ORDER_SOURCE)
+    subprocess.run(["g++", "-O1", "-std=c++17", "-shared", "-fPIC", "-o", str(d / "order.so"),
+                    str(d / "order.cpp")], check=True)
+    f = ctypes.CDLL(str(d / "order.so")).order
+    f.argtypes = [ctypes.c_uint64, ctypes.c_int, ctypes.c_int, ctypes.c_void_p]
+    f.restype = None
+
+    def get(seed, n, epochs=1):
+        out = np.zeros((epochs, n), dtype=np.int32)
+        f(seed, n, epochs, out.ctypes.data_as(ctypes.c_void_p))
+        return out
+    return get
+
+
+# one batch, a full segment, one more, two segments and one, a ragged third; whole segments
+# of one large batch; a remainder of samples that no batch holds
+@pytest.mark.parametrize("batch,nb,extra,epochs", [(64, 1, 0, 1), (64, 16, 0, 1), (64, 17, 5, 1),
+                                                   (64, 33, 0, 2), (64, 37, 63, 2), (129, 20, 1, 1),
+                                                   (40000, 3, 7, 1)])
+def test_an_epoch_equals_its_batches_one_call_at_a_time(m, h, order, batch, nb, extra, epochs):
+    """Parameters and losses of a training call, bit for bit, against the same batches in the
+    same order, each a call of its own on the same Adam state."""
+    n = batch * nb + extra
+    x = _inputs(n, n)
+    y = np.stack([x[:, 0] * x[:, 1], np.sin(3.0 * x[:, 1])], axis=1)
+    norm = np.array([0.1, -0.2, 0.7, 0.6, 0.05, 0.1, 0.4, 0.8])
+    inside = order(77, batch)[0]   # the order in which a call of one batch takes its rows
+    with m.Surrogate(h, 2, batch, seed=4) as a, m.Surrogate(h, 2, batch, seed=4) as b:
+        a.set_params(None, norm)
+        b.set_params(None, norm)
+        la = a.train(x, y, epochs=epochs, batch=batch, lr=1e-3, seed=8, set_norm=False)
+        lb = []
+        for perm in order(8, n, epochs):
+            lsum = 0.0
+            for k in range(nb):
+                rows = np.empty(batch, dtype=np.int64)
+                rows[inside] = perm[k * batch:(k + 1) * batch]
+                lsum += b.train(x[rows], y[rows], epochs=1, batch=batch, lr=1e-3, seed=77,
+                                set_norm=False)[0]
+            lb.append(lsum / nb)
+        pa, pb = a.get_params()[0], b.get_params()[0]
+        assert pa.tobytes() == pb.tobytes() and list(la) == lb
+        # and the comparison sees a batch that is not the same
+        b.train(x[rows][::-1], y[rows], epochs=1, batch=batch, lr=1e-3, seed=77, set_norm=False)
+        a.train(x[rows], y[rows], epochs=1, batch=batch, lr=1e-3, seed=77, set_norm=False)
+        assert a.get_params()[0].tobytes() != b.get_params()[0].tobytes()
