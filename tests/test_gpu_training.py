@@ -166,3 +166,39 @@ def test_an_epoch_equals_its_batches_one_call_at_a_time(m, h, order, batch, nb, 
         b.train(x[rows][::-1], y[rows], epochs=1, batch=batch, lr=1e-3, seed=77, set_norm=False)
         a.train(x[rows], y[rows], epochs=1, batch=batch, lr=1e-3, seed=77, set_norm=False)
         assert a.get_params()[0].tobytes() != b.get_params()[0].tobytes()
+
+
+@pytest.mark.parametrize("n", [1, 2, 63, 65, 127, 128, 129, 192, 193, 257, 640, 1025, 4203])
+def test_every_sample_of_a_ragged_batch_reaches_every_gradient(m, h, n):
+    """All targets but one are the network's own outputs, so the gradient is one sample's
+    alone: per parameter block it is the oracle's, wherever the sample lies.  A sample lost
+    from a block leaves it zero, one counted twice doubles it.
+
+    Bound: the oracle takes the same bfloat16 roundings, and a value that rounds the other
+    way moves by 2^-8 of itself; 2e-2 allows five such steps in every element of a block.
+    The other samples' errors, at most 2^-20 each against 5, add n 2^-20 / 5 < 1e-3."""
+    x = _inputs(n, n)
+    p = S.init_params(9, 1)
+    d = S.unpack(p[0])
+    rng = np.random.default_rng(n)
+    for name in ("b1", "b2", "b3", "b4"):
+        d[name] = 0.1 * rng.standard_normal(d[name].shape)
+    p = S.pack(d)[None].astype(np.float32).astype(np.float64)
+    edges = [0, 1, 62, 63, 64, 65, 127, 128, 191, 192, 255, 256, n // 2, n - 66, n - 65, n - 2, n - 1]
+    with m.Surrogate(h, 1, n, seed=1) as sg:
+        sg.set_params(p.astype(np.float32), IDENTITY)
+        y = sg.predict(x, per_model=True)[2][0].astype(np.float64)
+        g0, _ = sg.grads(x, y)
+        assert np.abs(g0).max() <= 1e-5   # nothing but those rounding errors
+        for at in sorted({k for k in edges if 0 <= k < n}):
+            t = y.copy()
+            t[at] += [5.0, -3.0]
+            g, loss = sg.grads(x, t)
+            # the oracle on that sample alone, with the batch's error signal d / n
+            out = S.forward(p[0], x[at:at + 1])[0]
+            _, ref = S.loss_and_grad(p[0], x[at:at + 1], out + np.array([5.0, -3.0]) / n)
+            got, want = S.unpack(g[0]), S.unpack(ref)
+            for name, _ in S.SHAPES:
+                err = np.linalg.norm(got[name] - want[name])
+                assert err <= 2.1e-2 * np.linalg.norm(want[name]), (at, name)
+            assert loss == pytest.approx((25.0 + 9.0) / (2 * n), rel=1e-5)
