@@ -1392,10 +1392,12 @@ static cudaError_t gradients(mdeos_surrogate* s, const float* X, const float* T,
   const ColArgs c{s->dY, s->dZf, X, s->H3, s->dZb, dZ2, s->G, B, s->Y, (int)(grid.x * grid.y), loss};
   const int ncol = 2 * (kH / 32) * E;
   mlp_batch_sums<<<ncol + g.Z * g.S, kGThreads, kSumSmem, st>>>(c, g, ncol, s->err);
+  count_launch(s->h, 2);
   if (splits) {
     *splits = g.S;
     return cudaGetLastError();
   }
+  if (g.S > 1) count_launch(s->h, 1);
   return gemm_reduce(g, st);
 }
 
@@ -1548,7 +1550,6 @@ extern "C" mdeos_status mdeos_surrogate_grads(mdeos_surrogate* s, const double* 
   mdeos_status ms = load_batch(s, x, y, n, st);
   if (ms != MDEOS_OK) return ms;
   SCK(gradients(s, s->X, s->T, n, s->loss, nullptr, st));
-  count_launch(s->h, 3);
   if (grads)
     SCK(cudaMemcpyAsync(grads, s->G, (size_t)s->E * kNParam * 4, cudaMemcpyDeviceToHost, st));
   float l = 0.f;
@@ -1632,7 +1633,7 @@ extern "C" mdeos_status mdeos_surrogate_train(mdeos_surrogate* s, const double* 
                    (float)(1.0 - std::pow(0.999, (double)s->step))};
         mlp_adam<<<dim3(nblk(kNParam), s->E), 256, 0, st>>>(a);
         SCK(cudaGetLastError());
-        count_launch(s->h, 3);
+        count_launch(s->h, 1);
       }
       SCK(cudaMemcpyAsync(tb.h_loss + turn * kSegBatches, dl, (size_t)nb * 4,
                           cudaMemcpyDeviceToHost, st));
@@ -1655,7 +1656,7 @@ static cudaError_t infer(mdeos_surrogate* s, const double* dx, int B, double* dm
   cudaError_t e;
   if (path == MDEOS_SURROGATE_INFER_MMA) {
     e = forward(s, B, dY, st);
-    count_launch(s->h, 9);
+    count_launch(s->h, 8);  // six of the layers (K = 128 is not split)
   } else {
     if (!s->tc_ready) {
       e = cudaFuncSetAttribute(mlp_infer_tc_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,

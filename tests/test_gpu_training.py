@@ -202,3 +202,22 @@ def test_every_sample_of_a_ragged_batch_reaches_every_gradient(m, h, n):
                 err = np.linalg.norm(got[name] - want[name])
                 assert err <= 2.1e-2 * np.linalg.norm(want[name]), (at, name)
             assert loss == pytest.approx((25.0 + 9.0) / (2 * n), rel=1e-5)
+
+
+def test_launch_counts(m, h):
+    """Kernels counted by mdeos_stats: a gradient is two, and a third where the batch's K is
+    split (from four chunks of 64 samples on); a training step three; inference three on the
+    fused path, eight on the layered one."""
+    def count(f):
+        before = m.mdeos_stats(h)["launches"]
+        f()
+        return m.mdeos_stats(h)["launches"] - before
+
+    x = _inputs(640, 1)
+    with m.Surrogate(h, 2, 640, seed=1) as sg:
+        for n, k in ((1, 2), (192, 2), (193, 3), (640, 3)):
+            assert count(lambda: sg.grads(x[:n], x[:n])) == k, n
+        assert count(lambda: sg.train(x, x, epochs=2, batch=64, set_norm=False)) == 3 * 20
+        assert count(lambda: sg.predict(x)) == 3
+        sg.set_infer_path(1)
+        assert count(lambda: sg.predict(x)) == 8
