@@ -607,7 +607,8 @@ mdeos_status mdeos_debug_gemm_bf16(const uint16_t* A, const uint16_t* B, float* 
                                    int64_t sb_n, int64_t sc_m, int64_t sc_n, void* stream);
 
 /* The surrogate's hidden-layer tanh on its own: y[i] = tanh(x[i]) for n device floats
- * (relative error below 2e-6: an exp2 form, and an odd series below |x| = 1/4).
+ * (relative error below 2e-6: an exp2 form, and an odd series below |x| = 1/4), by the
+ * function of the fused kernels, which takes two values at a time (2 i and 2 i + 1).
  * Synchronous on `stream` (cudaStream_t).  Errors: MDEOS_EINVAL (NULL, n < 1),
  * MDEOS_ECUDA. */
 mdeos_status mdeos_debug_tanh(const float* x, float* y, int32_t n, void* stream);

@@ -55,6 +55,32 @@ struct GemmArgs {
 // ---------------------------------------------------------------------------
 // elementwise parts; index layout [model][sample][unit]
 
+// two FP32 values in one register pair; the packed instructions round each half as the
+// scalar ones do
+__device__ __forceinline__ uint64_t f2_pack(float a, float b) {
+  uint64_t r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+  return r;
+}
+__device__ __forceinline__ void f2_unpack(uint64_t v, float& a, float& b) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
+}
+__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
+  uint64_t r;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+  return r;
+}
+__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
+  uint64_t r;
+  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+  return r;
+}
+
 // tanh for the hidden layers, whose outputs are rounded to bf16 next (half an ulp:
 // 2^-9 relative).  |x| >= 1/4: tanh|x| = 1 - 2 / (1 + e^{2|x|}) with e^{2|x|} =
 // 2^{2|x| log2 e} from ex2.approx and the reciprocal from rcp.approx; |x| < 1/4, where
@@ -63,16 +89,34 @@ struct GemmArgs {
 // (3.8e-7 with exact exp2 and division; the approximate instructions add at most ~5e-7,
 // largest near |x| = 1/4), so a bf16 rounding differs from that of the exact tanh only
 // within 2e-6 of a rounding boundary.  Saturates to +-1 for large |x|; NaN stays NaN.
+// Two values at a time: the multiply-adds in packed form fill half the issue slots (the
+// special-function results bound the rest).  |x| c = |x c| and x poly = copysign(|x| poly, x)
+// exactly, so the absolute value is taken by the exponential and the small branch keeps its
+// sign by itself.
+__device__ __forceinline__ void tanh_act2(uint64_t x, float& t0, float& t1) {
+  const uint64_t one = f2_pack(1.0f, 1.0f);
+  float x0, x1, a0, a1, e0, e1, r0, r1, b0, b1, s0, s1;
+  f2_unpack(x, x0, x1);
+  f2_unpack(f2_mul(x, f2_pack(2.885390081777927f, 2.885390081777927f)), a0, a1);  // 2 log2(e)
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(fabsf(a0)));
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(fabsf(a1)));
+  f2_unpack(f2_add(one, f2_pack(e0, e1)), e0, e1);
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(e0));
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r1) : "f"(e1));
+  f2_unpack(f2_fma(f2_pack(-2.0f, -2.0f), f2_pack(r0, r1), one), b0, b1);
+  const uint64_t x2 = f2_mul(x, x);
+  uint64_t p = f2_fma(x2, f2_pack(-17.0f / 315.0f, -17.0f / 315.0f), f2_pack(2.0f / 15.0f, 2.0f / 15.0f));
+  p = f2_fma(x2, p, f2_pack(-1.0f / 3.0f, -1.0f / 3.0f));
+  p = f2_fma(x2, p, one);
+  f2_unpack(f2_mul(x, p), s0, s1);
+  t0 = fabsf(x0) < 0.25f ? s0 : copysignf(b0, x0);
+  t1 = fabsf(x1) < 0.25f ? s1 : copysignf(b1, x1);
+}
+
 __device__ __forceinline__ float tanh_act(float x) {
-  const float ax = fabsf(x);
-  float e, r;
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e) : "f"(ax * 2.885390081777927f));  // 2 log2(e)
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(1.0f + e));
-  const float big = fmaf(-2.0f, r, 1.0f);
-  const float x2 = x * x;
-  const float small =
-      ax * fmaf(x2, fmaf(x2, fmaf(x2, -17.0f / 315.0f, 2.0f / 15.0f), -1.0f / 3.0f), 1.0f);
-  return copysignf(ax < 0.25f ? small : big, x);
+  float t0, t1;
+  tanh_act2(f2_pack(x, x), t0, t1);
+  return t0;
 }
 
 // refresh the bf16 weight copies from the FP32 master parameters
@@ -418,56 +462,6 @@ __device__ __forceinline__ void tc_ld32(uint32_t taddr, float (&v)[32]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
 #pragma unroll
   for (int j = 0; j < 32; ++j) v[j] = __uint_as_float(r[j]);
-}
-
-// two FP32 values in one register pair; the packed instructions round each half as the
-// scalar ones do
-__device__ __forceinline__ uint64_t f2_pack(float a, float b) {
-  uint64_t r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
-  return r;
-}
-__device__ __forceinline__ void f2_unpack(uint64_t v, float& a, float& b) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(a), "=f"(b) : "l"(v));
-}
-__device__ __forceinline__ uint64_t f2_add(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
-  uint64_t r;
-  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
-  return r;
-}
-__device__ __forceinline__ uint64_t f2_fma(uint64_t a, uint64_t b, uint64_t c) {
-  uint64_t r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-
-// tanh_act of two values: the same operations, the multiply-adds in packed form (they fill
-// half the issue slots; the special-function results bound the rest).  |x| c = |x c| and
-// x poly = copysign(|x| poly, x) exactly, so the absolute value is taken by the exponential
-// and the small branch keeps its sign by itself.
-__device__ __forceinline__ void tanh_act2(uint64_t x, float& t0, float& t1) {
-  const uint64_t one = f2_pack(1.0f, 1.0f);
-  float x0, x1, a0, a1, e0, e1, r0, r1, b0, b1, s0, s1;
-  f2_unpack(x, x0, x1);
-  f2_unpack(f2_mul(x, f2_pack(2.885390081777927f, 2.885390081777927f)), a0, a1);  // 2 log2(e)
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e0) : "f"(fabsf(a0)));
-  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(e1) : "f"(fabsf(a1)));
-  f2_unpack(f2_add(one, f2_pack(e0, e1)), e0, e1);
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r0) : "f"(e0));
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r1) : "f"(e1));
-  f2_unpack(f2_fma(f2_pack(-2.0f, -2.0f), f2_pack(r0, r1), one), b0, b1);
-  const uint64_t x2 = f2_mul(x, x);
-  uint64_t p = f2_fma(x2, f2_pack(-17.0f / 315.0f, -17.0f / 315.0f), f2_pack(2.0f / 15.0f, 2.0f / 15.0f));
-  p = f2_fma(x2, p, f2_pack(-1.0f / 3.0f, -1.0f / 3.0f));
-  p = f2_fma(x2, p, one);
-  f2_unpack(f2_mul(x, p), s0, s1);
-  t0 = fabsf(x0) < 0.25f ? s0 : copysignf(b0, x0);
-  t1 = fabsf(x1) < 0.25f ? s1 : copysignf(b1, x1);
 }
 
 // bf16(tanh(z + bias)) of 8 consecutive units, packed as one 16-byte core-matrix row
@@ -1179,9 +1173,14 @@ __global__ void gemm_splitk_reduce(const float* ws, float* C, float* C2, int z2,
   }
 }
 
+// tanh_act2 of elements 2 i and 2 i + 1, one in each half
 __global__ void debug_tanh_kernel(const float* x, float* y, int n) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) y[i] = tanh_act(x[i]);
+  const long long i = 2 * (blockIdx.x * (long long)blockDim.x + threadIdx.x);
+  if (i >= n) return;
+  float t0, t1;
+  tanh_act2(f2_pack(x[i], x[i + 1 < n ? i + 1 : i]), t0, t1);
+  y[i] = t0;
+  if (i + 1 < n) y[i + 1] = t1;
 }
 
 }  // namespace mdeos
@@ -1919,7 +1918,7 @@ extern "C" mdeos_status mdeos_debug_gemm_bf16(const uint16_t* A, const uint16_t*
 extern "C" mdeos_status mdeos_debug_tanh(const float* x, float* y, int32_t n, void* stream) {
   if (!x || !y || n < 1) return set_error(MDEOS_EINVAL, "bad tanh arguments");
   cudaStream_t st = (cudaStream_t)stream;
-  debug_tanh_kernel<<<(n + 255) / 256, 256, 0, st>>>(x, y, n);
+  debug_tanh_kernel<<<(n - 1) / 512 + 1, 256, 0, st>>>(x, y, n);
   SCK(cudaGetLastError());
   SCK(cudaStreamSynchronize(st));
   return MDEOS_OK;

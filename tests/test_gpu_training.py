@@ -221,3 +221,33 @@ def test_launch_counts(m, h):
         assert count(lambda: sg.predict(x)) == 3
         sg.set_infer_path(1)
         assert count(lambda: sg.predict(x)) == 8
+
+
+def test_both_halves_of_the_packed_tanh(m):
+    """The tanh of the fused kernels takes two values at a time: each value in either half
+    gives the same bits, beside whatever value, within 2e-6 of tanh."""
+    import torch
+    g = np.linspace(-12.0, 12.0, 100001)
+    tiny = 10.0 ** np.linspace(-37, -1, 1001)
+    edge = np.array([0.25, np.nextafter(np.float32(0.25), np.float32(0)), 43.9, 44.0, 88.0, 3e38,
+                     np.inf, 0.0])
+    x = np.concatenate([g, tiny, -tiny, edge, -edge]).astype(np.float32)
+    rng = np.random.default_rng(1)
+
+    def tanh(v):
+        return m.mdeos_debug_tanh(torch.from_numpy(np.ascontiguousarray(v)).cuda()).cpu().numpy()
+
+    y = tanh(x)
+    ref = np.tanh(x.astype(np.float64))
+    nz = np.abs(ref) > 1e-36
+    assert (np.abs(y[nz] - ref[nz]) < 2e-6 * np.abs(ref[nz])).all()
+    assert (np.signbit(y) == np.signbit(x)).all()
+    assert tanh(x[1:]).tobytes() == y[1:].tobytes()      # every value in the other half
+    p = rng.permutation(len(x))
+    assert tanh(x[p]).tobytes() == y[p].tobytes()
+    with_nan = np.repeat(x, 2)
+    with_nan[0::4] = np.nan                               # a NaN beside either half
+    with_nan[3::4] = np.nan
+    yn = tanh(with_nan)
+    keep = ~np.isnan(with_nan)
+    assert np.isnan(yn[~keep]).all() and yn[keep].tobytes() == np.repeat(y, 2)[keep].tobytes()
