@@ -463,12 +463,13 @@ static void serve_loop(mdeos_server* s) {
       }
     }
     // idle CTAs stay while traffic is active (work outstanding or waiting, or an
-    // arrival in the last 100 ms)
+    // arrival less than idle_ms ago)
     {
       bool active;
       {
         std::lock_guard<std::mutex> lk(s->mu);
-        active = !s->waiting.empty() || (s->last_arrival >= 0 && s->now() - s->last_arrival < 0.1);
+        active = !s->waiting.empty() ||
+                 (s->last_arrival >= 0 && s->now() - s->last_arrival < 1e-3 * s->cfg.idle_ms);
       }
       active = active || s->outstanding_items > 0 || !held.empty();
       reinterpret_cast<std::atomic<int>*>(s->h_linger)->store(active && !s->stop.load() ? 1 : 0,

@@ -139,6 +139,26 @@ def test_idle_exit_and_relaunch(m, h):
     assert st["launches"] >= 2
 
 
+def test_idle_grid_leaves_after_idle_ms(m, h):
+    """The grid leaves the GPU idle_ms after its last work, so a caller that waits for the
+    device right after a short burst waits for that and not for a longer hold (200 ms of the
+    box's own work would show as well: it is a few ms)."""
+    import torch
+    r = dict(rho=0.8, e=1.5, natoms=256, steps_equil=40, steps_avg=40, seed=9)
+    with m.Server(h, idle_ms=5) as srv:
+        srv.enqueue([r])
+        srv.wait_all(1, timeout_s=60)        # first use: loading, warm clocks
+        torch.cuda.synchronize()
+        waits = []
+        for k in range(3):
+            srv.enqueue([dict(r, seed=10 + k)])
+            assert srv.wait_all(1, timeout_s=60)["result"]["status"][0] == 0
+            t = time.perf_counter()
+            torch.cuda.synchronize()
+            waits.append(time.perf_counter() - t)
+    assert min(waits) < 0.05, waits
+
+
 def _element_requests(m, sizes, seed, round_k):
     """One request per element (element_id k + 1) for a hydro-like step; each round
     moves every element's density a little, as a Lagrangian mesh does."""
