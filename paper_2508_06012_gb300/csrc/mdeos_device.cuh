@@ -705,9 +705,12 @@ __device__ __noinline__ FSums force_pass(uint32_t xs_a, float4* fs, const uint16
       if (p == 0) fs[i] = make_float4(fx, fy, fz, cw);
       if (EN) {
         bad |= !(fabsf(e) < 1e9f);
-        // one range test for all the atom's values; with several threads per atom in a full
-        // CTA a pass is so short of issue slots that the conversion instruction is the cheaper
-        bool small = fabsf(e) < kFixFast && (MDEOS_LIST_AHEAD > 1 || tpa == 1);
+        // Few warps (clusters): one range test for all the atom's values, then FP32 forms of
+        // the conversion.  In a full CTA the conversion instruction every time, as that test is
+        // a branch on the data: with it, 1216 boxes of 256, 300 (rho 0.5), 380 and 500 atoms
+        // (0.75), 420 steps, took 29.1, 40.9, 49.6 and 58.8 ms; without it 27.4, 37.6, 47.2
+        // and 53.8.
+        bool small = MDEOS_LIST_AHEAD > 1 && fabsf(e) < kFixFast;
         if (VIR) {
           const float wn = fabsf(w[0]) + fabsf(w[1]) + fabsf(w[2]);
           bad |= !(wn < 1e9f);
