@@ -542,7 +542,10 @@ __device__ __noinline__ FSums force_pass(uint32_t xs_a, float4* fs, const uint16
   unsigned long long es = 0, ws[6] = {0, 0, 0, 0, 0, 0};
   int np = 0, bad = 0;
   // units u0 .. u1 - 1 (u0 a multiple of tpa); unit u = i tpa + p: sub-list p of atom
-  // i (tpa = 1 but for lists without cells)
+  // i (tpa = 1 but for lists without cells; in a full CTA, as a constant, that leaves registers
+  // to the sums, which otherwise wait in local memory: 4000 atoms, rho 0.8, 100 sampling steps
+  // of 304 boxes 33.2 ms, 31.6 so; with three list words ahead it is no gain)
+  if (CODED && MDEOS_LIST_AHEAD == 1) tpa = 1;
   const int sh = tpa == 4 ? 2 : (tpa == 2 ? 1 : 0);
   // entries in flight at once: a whole word, or half of one where the energy and virial
   // sums need the registers
