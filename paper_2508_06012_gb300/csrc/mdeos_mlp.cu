@@ -1226,26 +1226,35 @@ struct TrainBuffers {
   }
 };
 
-// Staging of predict's host arrays, allocated and given back with the surrogate: kIoRows
-// queries at a time, or max_batch if that is fewer (inputs 16 B; outputs a head with the error
+// Staging of predict's host arrays, allocated and given back with the surrogate: two slots of
+// kIoRows queries, or max_batch if that is fewer (inputs 16 B; outputs a head with the error
 // word, mean and sd 16 B each, 8 B per model).  A predict allocates nothing: a cudaFree in it
 // could wait for whatever else runs on the device.
-constexpr int kIoRows = 1 << 18;
+constexpr int kIoRows = 1 << 15;
 constexpr size_t kIoHead = 256;
 struct PredictBuffers {
-  char *h_in = nullptr, *h_out = nullptr, *d_out = nullptr;
+  char *h_in[2] = {nullptr, nullptr}, *h_out[2] = {nullptr, nullptr}, *d_out = nullptr;
+  cudaEvent_t done[2] = {nullptr, nullptr};
   cudaError_t allocate(int rows, int E) {
     const size_t out = kIoHead + (size_t)rows * (32 + 8 * (size_t)E);
-    cudaError_t e = cudaMallocHost((void**)&h_in, (size_t)rows * 16);
-    if (e == cudaSuccess) e = cudaMallocHost((void**)&h_out, out);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&d_out, out);
+    cudaError_t e = cudaMalloc((void**)&d_out, out);
+    for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
+      e = cudaMallocHost((void**)&h_in[k], (size_t)rows * 16);
+      if (e == cudaSuccess) e = cudaMallocHost((void**)&h_out[k], out);
+      if (e == cudaSuccess) e = cudaEventCreateWithFlags(&done[k], cudaEventDisableTiming);
+    }
     return e;
   }
   void release() {
-    if (h_in) cudaFreeHost(h_in);
-    if (h_out) cudaFreeHost(h_out);
+    for (int k = 0; k < 2; ++k) {
+      if (h_in[k]) cudaFreeHost(h_in[k]);
+      if (h_out[k]) cudaFreeHost(h_out[k]);
+      if (done[k]) cudaEventDestroy(done[k]);
+      h_in[k] = h_out[k] = nullptr;
+      done[k] = nullptr;
+    }
     if (d_out) cudaFree(d_out);
-    h_in = h_out = d_out = nullptr;
+    d_out = nullptr;
   }
 };
 
@@ -1721,24 +1730,23 @@ extern "C" mdeos_status mdeos_surrogate_predict(mdeos_surrogate* s, const double
   if (!s || !x || n < 0) return set_error(MDEOS_EINVAL, "bad predict arguments");
   SCK(cudaSetDevice(handle_device(s->h)));
   cudaStream_t st = handle_stream(s->h);
-  // One copy in and one out per chunk, through pinned memory: the chunk's mean, sd and
-  // per-model outputs and the error word share a device block.  (Copies to and from pageable
-  // memory are staged and waited for one by one: eight of them took half of a 2000-query
-  // call, 123 us; it takes 67 now.)
+  // One copy in and one out per piece, through pinned memory: the piece's mean, sd and per-model
+  // outputs and the error word share a device block.  (Copies to and from pageable memory are
+  // waited for one by one: eight of them took half of a 2000-query call, 123 us; it takes 67
+  // now.  Into arrays that the device has not written before they are far slower: 2^18 queries,
+  // one model, 7.2 ms.)  Two slots in turn: the host copies one piece's arrays while the device
+  // works on the other's.
   const int chunk = std::min(s->maxB, kIoRows);
   int err = 0;
-  for (int off = 0; off < n; off += chunk) {
-    const int B = std::min(chunk, n - off);
-    const size_t ob = (size_t)B * 16, yb = per_model ? (size_t)s->E * B * 8 : 0;
-    char* d = s->io.d_out;
-    std::memcpy(s->io.h_in, x + 2 * (size_t)off, ob);
-    SCK(cudaMemcpyAsync(s->Xp, s->io.h_in, ob, cudaMemcpyHostToDevice, st));
-    SCK(infer(s, s->Xp, B, (double*)(d + kIoHead), (double*)(d + kIoHead + ob),
-              (float*)(d + kIoHead + 2 * ob), s->infer_path, st));
-    SCK(cudaMemcpyAsync(d, s->err, 4, cudaMemcpyDeviceToDevice, st));
-    SCK(cudaMemcpyAsync(s->io.h_out, d, kIoHead + 2 * ob + yb, cudaMemcpyDeviceToHost, st));
-    SCK(cudaStreamSynchronize(st));
-    const char* h = s->io.h_out;
+  int held[2] = {0, 0}, first[2] = {0, 0};  // queries of the piece in flight in each slot
+  auto collect = [&](int t) -> cudaError_t {
+    const int B = held[t], off = first[t];
+    if (B == 0) return cudaSuccess;
+    held[t] = 0;
+    const cudaError_t e = cudaEventSynchronize(s->io.done[t]);
+    if (e != cudaSuccess) return e;
+    const size_t ob = (size_t)B * 16;
+    const char* h = s->io.h_out[t];
     if (mean) std::memcpy(mean + 2 * (size_t)off, h + kIoHead, ob);
     if (sd) std::memcpy(sd + 2 * (size_t)off, h + kIoHead + ob, ob);
     if (per_model)
@@ -1746,7 +1754,33 @@ extern "C" mdeos_status mdeos_surrogate_predict(mdeos_surrogate* s, const double
         std::memcpy(per_model + ((size_t)m * n + off) * 2, h + kIoHead + 2 * ob + (size_t)m * B * 8,
                     (size_t)B * 8);
     err |= *reinterpret_cast<const int*>(h);
-  }
+    return cudaSuccess;
+  };
+  const auto run = [&]() -> cudaError_t {
+    cudaError_t e = cudaSuccess;
+    for (int off = 0, t = 0; off < n && e == cudaSuccess; off += chunk, t ^= 1) {
+      if ((e = collect(t)) != cudaSuccess) break;
+      const int B = std::min(chunk, n - off);
+      const size_t ob = (size_t)B * 16, yb = per_model ? (size_t)s->E * B * 8 : 0;
+      char* d = s->io.d_out;
+      std::memcpy(s->io.h_in[t], x + 2 * (size_t)off, ob);
+      e = cudaMemcpyAsync(s->Xp, s->io.h_in[t], ob, cudaMemcpyHostToDevice, st);
+      if (e == cudaSuccess)
+        e = infer(s, s->Xp, B, (double*)(d + kIoHead), (double*)(d + kIoHead + ob),
+                  (float*)(d + kIoHead + 2 * ob), s->infer_path, st);
+      if (e == cudaSuccess) e = cudaMemcpyAsync(d, s->err, 4, cudaMemcpyDeviceToDevice, st);
+      if (e == cudaSuccess)
+        e = cudaMemcpyAsync(s->io.h_out[t], d, kIoHead + 2 * ob + yb, cudaMemcpyDeviceToHost, st);
+      if (e == cudaSuccess) e = cudaEventRecord(s->io.done[t], st);
+      if (e != cudaSuccess) break;
+      held[t] = B;
+      first[t] = off;
+    }
+    for (int t = 0; t < 2 && e == cudaSuccess; ++t) e = collect(t);
+    if (e != cudaSuccess) cudaStreamSynchronize(st);  // nothing still uses the slots
+    return e;
+  };
+  SCK(run());
   if (err) {
     SCK(cudaMemsetAsync(s->err, 0, 4, st));
     SCK(cudaStreamSynchronize(st));

@@ -69,16 +69,21 @@ def test_predict_allocates_no_device_memory(m, h):
     assert np.array_equal(small[0], full[0][:100]) and np.array_equal(small[1], full[1][:100])
 
 
-def test_predict_in_pieces_of_its_staging(m, h):
-    """More queries than the staging holds, a ragged last piece: the answers of the same
-    queries asked in another order of pieces."""
-    n = 2 * 5000 + 777
+# pieces of max_batch, of the staging's 32768, one query more, an odd number of pieces
+@pytest.mark.parametrize("n,max_batch", [(2 * 5000 + 777, 5000), (32768, 1 << 18),
+                                         (32769, 1 << 18), (5 * 32768 - 1, 1 << 18),
+                                         (3 * 20000 + 1, 20000)])
+def test_predict_in_pieces(m, h, n, max_batch):
+    """The answers do not depend on the pieces and the way a call's arrays take: the same
+    queries in reverse, and a few of them alone."""
     x = _inputs(n, 2)
-    with m.Surrogate(h, 3, 5000, seed=1) as sg:
+    with m.Surrogate(h, 3, max_batch, seed=1) as sg:
         mean, sd, pm = sg.predict(x, per_model=True)
         m2, s2, p2 = sg.predict(x[::-1], per_model=True)
+        m3, s3 = sg.predict(x[-50:])
     assert np.array_equal(mean, m2[::-1]) and np.array_equal(sd, s2[::-1])
     assert np.array_equal(pm, p2[:, ::-1])
+    assert np.array_equal(mean[-50:], m3) and np.array_equal(sd[-50:], s3)
 
 
 def test_training_allocates_no_device_memory(m, h):
