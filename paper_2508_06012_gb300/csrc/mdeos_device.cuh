@@ -694,7 +694,7 @@ __device__ __noinline__ FSums force_pass(uint32_t xs_a, float4* fs, const uint16
       // (1216 boxes of 300 atoms, rho 0.5, 420 steps: 61.7 ms without, 41.8 with).
       const int left = u1 - (u - (tid & 31));
       const unsigned m = left >= 32 ? 0xffffffffu : (1u << left) - 1u;
-      __syncwarp(m);
+      if (PATH == PATH_NLIST) __syncwarp(m);
       if (tpa > 1) {  // the partial forces of the atom's units, in a fixed order
         fx += __shfl_xor_sync(m, fx, 1);
         fy += __shfl_xor_sync(m, fy, 1);
@@ -1713,11 +1713,18 @@ __device__ void run_box(const Group& g, const BoxDesc& __restrict__ bd, const Ru
   const double invV = 1.0 / V, inv3V = 1.0 / (3.0 * V), inv_ndof = 1.0 / ndof;
   const int lead = (g.bar - 1) & 3 & (g.nwarps - 1);  // spreads group leaders over SMSPs
   const double lane_unit = g.lane() < 8 ? kFixInv : 1.0;  // the leader's lane's quantity
-  // block of the averaging step, floor(s_avg nb / steps_avg), and the steps to the next
-  // rescaling, carried along instead of divided for
+  // On a cluster (kDefer) an averaging step's sums wait in the leader's local memory until the
+  // rescaling step (every tenth by default), a full buffer, or the end of a block or of the
+  // run, and are then added in step order, as a step's FP64 instructions (one per 19 SM cycles)
+  // would run while the other warps wait at the next step's barrier; the block, floor(s_avg nb /
+  // steps_avg), and the steps to the next rescaling are carried along instead of divided for
+  // (16 x 256 atoms, 800 steps: 7.39 ms adding and dividing every step, 7.22 so).  In a full CTA
+  // the other boxes fill that time, and what is carried along costs registers in every thread
+  // (4000 boxes of 108 atoms, rho 0.9, 120 steps: 40.5 ms so, 38.7 adding every step).
+  constexpr bool kDefer = MDEOS_LIST_AHEAD > 1;
   int blk = 0;
   long long blk_num = 0;
-  constexpr int kPend = 10;
+  constexpr int kPend = kDefer ? 10 : 1;
   long long pend[kPend];  // the leader's: averaging steps whose sums are not added up yet
   int npend = 0;
   const auto flush = [&] {  // every lane of the leader's warp
@@ -1743,6 +1750,7 @@ __device__ void run_box(const Group& g, const BoxDesc& __restrict__ bd, const Ru
   if (g.tid == 0) boxc[3] = Tk;
   for (int step = 0; step < total && status == MDEOS_OK; ++step) {
     const bool avg = step >= bd.steps_equil;
+    const int s_avg = step - bd.steps_equil;
     const bool seg_end = !avg && (seg_pos == seg_len - 1);
     const bool esamp = !avg && !temp_mode && (seg_pos >= seg_len - nsamp);
     const bool need = kick_drift<APT>(g, b, rp, lam);
@@ -1845,7 +1853,11 @@ __device__ void run_box(const Group& g, const BoxDesc& __restrict__ bd, const Ru
     }
     // thermostat steps and segment ends rescale the velocities
     bool resc = seg_end;
-    if (!avg) {
+    if (!kDefer) {
+      resc = resc ||
+             (!avg && rp.rescale_every_equil > 0 && (seg_pos + 1) % rp.rescale_every_equil == 0) ||
+             (avg && rp.rescale_every_avg > 0 && (s_avg + 1) % rp.rescale_every_avg == 0);
+    } else if (!avg) {
       if (rp.rescale_every_equil > 0 && ++since_eq == rp.rescale_every_equil) {
         resc = true;
         since_eq = 0;
@@ -1867,13 +1879,12 @@ __device__ void run_box(const Group& g, const BoxDesc& __restrict__ bd, const Ru
       double Ts = 0.0;
       if (resc) Ts = 2.0 * ((double)__shfl_sync(0xffffffffu, qi, 7) * kFixInv) * inv_ndof;
       if (avg) {
-        // The step's sums wait in the leader's local memory until the rescaling step (every
-        // tenth by default), a full buffer, or the end of a block or of the run, and are then
-        // added in step order: a step's FP64 instructions (one per 19 SM cycles) would run
-        // while the other warps wait at the next step's barrier (2000 boxes of 500 atoms,
-        // 500 steps: 128.9 ms adding them every step, 126.8 ms so).
+        if (!kDefer) {
+          blk = (int)(((long long)s_avg * nb) / bd.steps_avg);
+          npend = 0;
+        }
         pend[npend++] = qi;
-        if (resc || npend == kPend || blk_num + nb >= bd.steps_avg) flush();
+        if (!kDefer || resc || npend == kPend || blk_num + nb >= bd.steps_avg) flush();
       } else if (esamp && lane == 6) {
         acc[ACC_RUN + 12] += (double)qi * kFixInv;
       }
@@ -1892,7 +1903,7 @@ __device__ void run_box(const Group& g, const BoxDesc& __restrict__ bd, const Ru
           g.bc()[5] = (Tn > 0.0 && Ts > 0.0 && isfinite(Tn) && isfinite(Ts)) ? sqrt(Tn / Ts) : -1.0;
       }
     }
-    if (avg) {
+    if (kDefer && avg) {
       blk_num += nb;
       while (blk_num >= bd.steps_avg) {
         blk_num -= bd.steps_avg;
@@ -1923,7 +1934,7 @@ __device__ void run_box(const Group& g, const BoxDesc& __restrict__ bd, const Ru
       ++seg_pos;
     }
   }
-  if (g.warp() == lead && npend > 0) flush();
+  if (kDefer && g.warp() == lead && npend > 0) flush();
   gbar(g.bar, g.nt);
   if (status == MDEOS_OK && g.ctrl()[CTRL_STATUS] != 0) status = g.ctrl()[CTRL_STATUS];
   if (bd.warm_state != nullptr) {
