@@ -964,8 +964,8 @@ def bigbox(args):
     --big-natoms atoms (default one per SM; state, cells and Verlet lists in global
     memory, positions staged in shared-memory windows), one batch timed end to end.
     Few boxes (fewer than half the SMs) run each on a thread-block cluster of up to
-    --max-cluster CTAs (default 4; 1: one CTA per box), which sets the latency of one
-    large box.  Algorithmic HBM bytes per atom and step: the kick-drift reads x, v, f
+    --max-cluster CTAs (default: 8 from 16000 atoms on, else 4; 1: one CTA per box), which
+    sets the latency of one large box.  Algorithmic HBM bytes per atom and step: the kick-drift reads x, v, f
     and writes x, v (80 B); the force pass reads the positions (16 B, once per window)
     and the list entries (2 B each) and writes f (16 B).  The dram counters of the same
     launch come from ncu."""
@@ -1039,7 +1039,7 @@ def main():
     ap.add_argument("--big-natoms", type=int, default=32000, help="bigbox: atoms per box")
     ap.add_argument("--big-boxes", type=int, default=0, help="bigbox: boxes (0: one per SM)")
     ap.add_argument("--max-cluster", type=int, default=0,
-                    help="CTAs per box for batches of few small boxes (0: up to 4, 1: none)")
+                    help="CTAs per box for batches of few boxes (0: the library's default, 1: none)")
     ap.add_argument("--workload", choices=["uneven", "queries16x256", "coupled", "serving",
                                            "surrogate", "surrogate-infer", "forcepass",
                                            "bigbox"],

@@ -152,6 +152,11 @@ mdeos_status mdeos_create(const mdeos_config* cfg, mdeos_handle** out);
  * computes the forces of its share of the atoms); one with fewer boxes than half the SMs,
  * all above 4096 atoms, does the same with one state per box in global memory (each CTA
  * owns a slab of the cell-ordered atoms).  Results do not depend on the launch shape.
+ * A cluster starts when as many SMs of one GPC are free at once.  Beside work that holds
+ * SMs and lets them go one by one (a serving grid, another handle's batch) such a batch can
+ * start later than boxes on one CTA each, which max_cluster = 1 asks for.  Under
+ * hbm_budget_bytes clusters are halved until their list scratch (one per CTA) fits, and
+ * scratch that an earlier batch left with the handle is given back where a call needs the room.
  * Errors: MDEOS_EINVAL (n < 1, NULL, or a request field out of range),
  * MDEOS_ENOMEM, MDEOS_ECUDA. */
 mdeos_status mdeos_submit(mdeos_handle* h, const mdeos_request* reqs, int32_t n,
@@ -340,7 +345,9 @@ mdeos_status mdeos_hydro_create(mdeos_handle* h, const mdeos_hydro_config* cfg, 
                                 mdeos_hydro** out);
 
 /* Advance nsteps steps (synchronous).  Analytic closures run all steps in one
- * launch; the MD closure runs one EOS batch and one hydro launch per step.
+ * launch; the MD closure runs one EOS batch and one hydro launch per step.  A launch
+ * for up to about 35,000 zones is one thread-block cluster of up to 16 CTAs, which needs that
+ * many SMs of one GPC at once (see mdeos_submit).
  * Errors: MDEOS_EUNPHYS (tangled mesh, non-finite state, or an EOS box that
  * failed; the state is left at the last good step), MDEOS_ECUDA. */
 mdeos_status mdeos_hydro_step(mdeos_hydro* hy, int32_t nsteps);
@@ -384,7 +391,8 @@ typedef struct {
   int32_t max_batch;        /* requests planned together per admission step, default 2048 */
   double max_wait_s;        /* waiting longer than this: shed (MDEOS_ECANCELLED); 0 = never */
   int32_t max_queue;        /* waiting requests beyond this are shed on arrival; 0 = no cap */
-  int32_t idle_ms;          /* an idle kernel exits after this long, default 20 */
+  int32_t idle_ms;          /* an idle kernel exits this long after its last work and the last
+                               arrival, default 20 */
   size_t hbm_budget_bytes;  /* device memory the server may hold: the per-SM scratch for the
                                largest box (32768 atoms) plus the element store; creation
                                fails if the scratch alone exceeds it; 0 = no cap */

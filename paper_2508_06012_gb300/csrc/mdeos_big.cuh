@@ -368,8 +368,8 @@ static __device__ __noinline__ bool big_search(const float4* x, uint32_t sx_a, c
 
 // Verlet list from wrapped positions: counting sort into cell order (inside a
 // cell by previous slot: deterministic), permutation of x and v into the second
-// buffers (then swapped), 27-cell search with one image shift per cell.  In a
-// cluster: cells are dealt to the cluster's threads, slots to their owners, the
+// buffers (then swapped), then the search of the 27 cells (big_search: nine rows of three
+// adjacent cells, shifted to their image only across a face).  In a cluster: cells are dealt to the cluster's threads, slots to their owners, the
 // prefix sum over the cells is rank 0's, and each phase ends at a cluster barrier.
 // Returns whether a list overflowed anywhere in the cluster.
 static __device__ bool big_build(BigMem& m, BigShared* sh, BigClu& cl, int n, int nc, float L,
@@ -525,8 +525,9 @@ static __device__ bool big_build(BigMem& m, BigShared* sh, BigClu& cl, int n, in
   return ovf;
 }
 
-// Forces on every atom (strided over the CTA) from the Verlet list, minimum image
-// on every entry; partial sums over the thread's atoms.  Out of line and fed
+// Forces on every atom (strided over the CTA) from the Verlet list; partial sums over the
+// thread's atoms.  The minimum image is taken on every entry only where a lane of the warp has
+// an atom near a face (below).  Out of line and fed
 // scalars, like force_pass.  Positions come from the shared-memory copy at sx_a
 // (SM) or from global memory with ordinary (L1-cached) loads: they were written by
 // this CTA before the last barrier.

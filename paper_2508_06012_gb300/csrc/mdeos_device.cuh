@@ -462,13 +462,12 @@ struct ListReader {
 // Whether a pass takes its entries in groups (pair_group) or one by one (list_pair).  With
 // few warps resident the group's independent chains fill the pipes.  In a full CTA the
 // other warps do: there a coded list's pass is bound by its shared-memory gathers, and the
-// selects of the branch-free form only add to it (energy + virial, 4000 atoms: 164k SM cycles
-// in groups, 146k one by one); a pass with the minimum image and the virial of every pair
-// is bound by issue slots, and a branch per entry costs more than the selects (500 atoms,
-// eight boxes per CTA: 149k one by one, 136k in groups).  There a group of padding alone is
-// skipped: with several threads per atom a sub-list is two or three words, a third of them
-// padding (1216 boxes of 300 atoms, 420 steps: rho 0.5 42.4 ms one by one, 40.1-40.8 in groups with
-// the skip; rho 1.0 61.5 and 59.9-60.5).
+// selects of the branch-free form only add to it (energy + virial, 4000 atoms: 128k SM cycles
+// in groups, 122k one by one); a pass with the minimum image and the virial of every pair
+// is bound by issue slots, and a branch per entry costs more than the selects.  There a group
+// of padding alone is skipped: with several threads per atom a sub-list is two or three words,
+// a third of them padding (1216 boxes, 420 steps: 300 atoms, rho 0.5, 39.3 ms one by one, 39.3
+// in groups, 37.6 with the skip; rho 1.0 59.7, 58.4 and 56.4; 500 atoms 56.6, 54.6 and 53.8).
 template <bool EN, bool VIR, bool MI>
 constexpr bool kPairInGroups = MDEOS_LIST_AHEAD > 1 || (VIR && MI);
 
@@ -690,8 +689,9 @@ __device__ __noinline__ FSums force_pass(uint32_t xs_a, float4* fs, const uint16
       }
       // The warp's lanes of this turn (those up to u1) meet again here.  Their lists differ in
       // length, and a shuffle among the four lanes of an atom does not bring the others
-      // back: without this the parts of a warp ran the remaining turns one after another
-      // (1216 boxes of 300 atoms, rho 0.5, 420 steps: 61.7 ms without, 41.8 with).
+      // back: without this the parts of a warp may run the remaining turns one after another
+      // (1216 boxes of 300 atoms, rho 0.5, 420 steps: 38.4 ms without, 37.6 with, and 61.7
+      // without where the sums below also branched on the data).
       const int left = u1 - (u - (tid & 31));
       const unsigned m = left >= 32 ? 0xffffffffu : (1u << left) - 1u;
       if (PATH == PATH_NLIST) __syncwarp(m);

@@ -483,12 +483,13 @@ __device__ __forceinline__ uint4 tanh_pack8(const float* z, const float* bias) {
 // of a group serves row m = t % 128 (TMEM lane m) and column half t / 128: warps w and w + 4
 // read the same 32 lanes, columns 0-63 and 64-127.
 //
-// What bounds it is the 384 tanh per row, two special-function results each (16 per clock
-// and SM: 12.3k cycles for two tiles), then the issue slots of the rest.  A tile alternates
-// between its product and its tanh, so other tiles have to fill the gaps: with two CTAs of
-// 256 threads per SM, each with its own copy of the weights (101 KB), two tiles took 21.5k
-// cycles; four groups around one copy (197 KB, all 512 TMEM columns)
-// fill them (2^20 queries, normalising and averaging included: 1348 us before, 1112 now).
+// What bounds it is the 384 tanh per row: their issue slots (74 % of all, measured), and their
+// special-function results (an exp2 at 32 and a reciprocal at 16 per clock and SM, measured:
+// 9.2k cycles for two tiles).  A tile alternates between its product and its tanh, so other
+// tiles have to fill the gaps: with two CTAs of 256 threads per SM, each with its own copy of
+// the weights (101 KB), two tiles took 21.5k cycles; four groups around one copy (197 KB, all
+// 512 TMEM columns) fill them (2^20 queries, normalising and averaging included: 1348 us
+// before, 1104 now).
 constexpr int kTcGroups = 4;
 constexpr int infer_tc_smem(int groups) {
   return (2 + groups) * kTcTile + 1024 + 128 + kTcSmall * 4;
