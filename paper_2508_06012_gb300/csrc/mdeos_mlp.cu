@@ -1200,68 +1200,54 @@ constexpr int kSegBatches = 16;
 constexpr int kSegRows = 1 << 16;
 static int train_seg(int batch) { return std::max(1, std::min(kSegBatches, kSegRows / batch)); }
 
-// Buffers of the training calls, allocated and given back with the surrogate: two segments of
-// samples (16 B each) and their batches' losses.  A training call allocates nothing: a
-// cudaFree in it could wait for whatever else runs on the device.
-struct TrainBuffers {
-  float *h[2] = {nullptr, nullptr}, *d[2] = {nullptr, nullptr};
-  float *h_loss = nullptr, *d_loss = nullptr;  // [2][kSegBatches]
-  cudaEvent_t done[2] = {nullptr, nullptr};
-  cudaError_t allocate(int max_batch) {
-    // the longest segment of any batch size
-    const size_t bytes = 16 * (size_t)std::max(max_batch, std::min(kSegRows, kSegBatches * max_batch));
-    cudaError_t e = cudaMallocHost((void**)&h_loss, 2 * kSegBatches * 4);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&d_loss, 2 * kSegBatches * 4);
-    for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
-      e = cudaMallocHost((void**)&h[k], bytes);
-      if (e == cudaSuccess) e = cudaMalloc((void**)&d[k], bytes);
-      if (e == cudaSuccess) e = cudaEventCreateWithFlags(&done[k], cudaEventDisableTiming);
-    }
-    return e;
-  }
-  void release() {
-    for (int k = 0; k < 2; ++k) {
-      if (h[k]) cudaFreeHost(h[k]);
-      if (d[k]) cudaFree(d[k]);
-      if (done[k]) cudaEventDestroy(done[k]);
-      h[k] = d[k] = nullptr;
-      done[k] = nullptr;
-    }
-    if (h_loss) cudaFreeHost(h_loss);
-    if (d_loss) cudaFree(d_loss);
-    h_loss = d_loss = nullptr;
-  }
-};
-
-// Staging of predict's host arrays, allocated and given back with the surrogate: two slots of
-// kIoRows queries, or max_batch if that is fewer (inputs 16 B; outputs a head with the error
-// word, mean and sd 16 B each, 8 B per model).  A predict allocates nothing: a cudaFree in it
-// could wait for whatever else runs on the device.
+// Staging of the calls on host arrays, one pinned and one device block that come and go with the
+// surrogate, so that a call allocates nothing (a cudaFree in it could wait for whatever else
+// runs on the device; in blocks of their own they took mdeos_surrogate_create to 0.99 ms, 0.91 so).
+// predict: two slots of kIoRows queries, or max_batch if that is fewer (inputs 16 B; outputs a
+// head with the error word, mean and sd 16 B each, 8 B per model) and one device block of
+// outputs.  Training: two segments of samples (16 B each) and their batches' losses.
 constexpr int kIoRows = 1 << 15;
 constexpr size_t kIoHead = 256;
-struct PredictBuffers {
-  char *h_in[2] = {nullptr, nullptr}, *h_out[2] = {nullptr, nullptr}, *d_out = nullptr;
-  cudaEvent_t done[2] = {nullptr, nullptr};
-  cudaError_t allocate(int rows, int E) {
-    const size_t out = kIoHead + (size_t)rows * (32 + 8 * (size_t)E);
-    cudaError_t e = cudaMalloc((void**)&d_out, out);
-    for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
-      e = cudaMallocHost((void**)&h_in[k], (size_t)rows * 16);
-      if (e == cudaSuccess) e = cudaMallocHost((void**)&h_out[k], out);
-      if (e == cudaSuccess) e = cudaEventCreateWithFlags(&done[k], cudaEventDisableTiming);
+struct Staging {
+  char *host = nullptr, *dev = nullptr;
+  char *h_in[2], *h_out[2], *d_out;
+  float *h_seg[2], *d_seg[2], *h_loss, *d_loss;  // losses [2][kSegBatches]
+  cudaEvent_t io_done[2] = {nullptr, nullptr}, seg_done[2] = {nullptr, nullptr};
+  cudaError_t allocate(int max_batch, int E) {
+    const auto up = [](size_t b) { return (b + 255) & ~(size_t)255; };
+    const size_t rows = (size_t)std::min(max_batch, kIoRows);
+    const size_t in = up(rows * 16), out = up(kIoHead + rows * (32 + 8 * (size_t)E));
+    // the longest segment of any batch size
+    const size_t seg = up(16 * (size_t)std::max(max_batch, std::min(kSegRows, kSegBatches * max_batch)));
+    const size_t loss = up(2 * kSegBatches * 4);
+    cudaError_t e = cudaMallocHost((void**)&host, 2 * (in + out + seg) + loss);
+    if (e == cudaSuccess) e = cudaMalloc((void**)&dev, out + 2 * seg + loss);
+    if (e != cudaSuccess) return e;
+    char *h = host, *d = dev;
+    d_out = d;
+    d += out;
+    for (int k = 0; k < 2; ++k) {
+      h_in[k] = h;
+      h_out[k] = h + in;
+      h_seg[k] = (float*)(h + in + out);
+      h += in + out + seg;
+      d_seg[k] = (float*)d;
+      d += seg;
+      e = cudaEventCreateWithFlags(&io_done[k], cudaEventDisableTiming);
+      if (e == cudaSuccess) e = cudaEventCreateWithFlags(&seg_done[k], cudaEventDisableTiming);
+      if (e != cudaSuccess) return e;
     }
+    h_loss = (float*)h;
+    d_loss = (float*)d;
     return e;
   }
   void release() {
     for (int k = 0; k < 2; ++k) {
-      if (h_in[k]) cudaFreeHost(h_in[k]);
-      if (h_out[k]) cudaFreeHost(h_out[k]);
-      if (done[k]) cudaEventDestroy(done[k]);
-      h_in[k] = h_out[k] = nullptr;
-      done[k] = nullptr;
+      if (io_done[k]) cudaEventDestroy(io_done[k]);
+      if (seg_done[k]) cudaEventDestroy(seg_done[k]);
     }
-    if (d_out) cudaFree(d_out);
-    d_out = nullptr;
+    if (host) cudaFreeHost(host);
+    if (dev) cudaFree(dev);
   }
 };
 
@@ -1282,8 +1268,7 @@ struct mdeos_surrogate {
   float* ws = nullptr;  // partial tiles of the products whose K is split
   long long ws_elems = 0;
   int infer_path = MDEOS_SURROGATE_INFER_TC;
-  TrainBuffers tb;
-  PredictBuffers io;
+  Staging io;
   bool tc_ready = false, train_ready = false;
   int nsm = 1;
   std::vector<void*> allocs;
@@ -1467,8 +1452,7 @@ extern "C" mdeos_status mdeos_surrogate_create(mdeos_handle* h, int32_t n_models
   dalloc((void**)&s->err, 256);
   s->ws_elems = 2LL * kMaxSplitK * E * kH * kH;  // two products' partial tiles
   dalloc((void**)&s->ws, (size_t)s->ws_elems * 4);
-  if (e == cudaSuccess) e = s->io.allocate(std::min(max_batch, kIoRows), E);
-  if (e == cudaSuccess) e = s->tb.allocate(max_batch);
+  if (e == cudaSuccess) e = s->io.allocate(max_batch, E);
   if (e != cudaSuccess) {
     mdeos_surrogate_destroy(s);
     return set_error(MDEOS_ECUDA, std::string("surrogate_create: ") + cudaGetErrorString(e));
@@ -1604,7 +1588,7 @@ extern "C" mdeos_status mdeos_surrogate_train(mdeos_surrogate* s, const double* 
   // losses come back with them.
   const int nbat = n / batch;  // full batches only
   const int seg = train_seg(batch);
-  TrainBuffers& tb = s->tb;
+  Staging& io = s->io;
   const float b1 = 0.9f, b2 = 0.999f;
   for (int ep = 0; ep < epochs; ++ep) {
     std::shuffle(perm.begin(), perm.end(), rng);
@@ -1613,9 +1597,9 @@ extern "C" mdeos_status mdeos_surrogate_train(mdeos_surrogate* s, const double* 
     // the losses of buffer t's segment, once it is done
     auto collect = [&](int t) -> cudaError_t {
       if (held[t] == 0) return cudaSuccess;
-      const cudaError_t e = cudaEventSynchronize(tb.done[t]);
+      const cudaError_t e = cudaEventSynchronize(io.seg_done[t]);
       for (int k = 0; k < held[t]; ++k)
-        lsum += (double)tb.h_loss[t * kSegBatches + k] / (2.0 * batch * s->E);
+        lsum += (double)io.h_loss[t * kSegBatches + k] / (2.0 * batch * s->E);
       held[t] = 0;
       return e;
     };
@@ -1624,7 +1608,7 @@ extern "C" mdeos_status mdeos_surrogate_train(mdeos_surrogate* s, const double* 
       const int nb = std::min(seg, nbat - b0);
       const size_t rows = (size_t)nb * batch;
       SCK(collect(turn));
-      float* hx = tb.h[turn];
+      float* hx = io.h_seg[turn];
       float* ht = hx + 2 * rows;
       for (size_t k = 0; k < rows; ++k) {
         const size_t i = (size_t)perm[(size_t)b0 * batch + k];
@@ -1634,8 +1618,8 @@ extern "C" mdeos_status mdeos_surrogate_train(mdeos_surrogate* s, const double* 
           ht[2 * k + c] = (float)((t - s->norm[4 + c]) / s->norm[6 + c]);
         }
       }
-      float* dx = tb.d[turn];
-      float* dl = tb.d_loss + turn * kSegBatches;
+      float* dx = io.d_seg[turn];
+      float* dl = io.d_loss + turn * kSegBatches;
       SCK(cudaMemcpyAsync(dx, hx, rows * 16, cudaMemcpyHostToDevice, st));
       for (int k = 0; k < nb; ++k) {
         const float* bx = dx + 2 * (size_t)k * batch;
@@ -1650,9 +1634,9 @@ extern "C" mdeos_status mdeos_surrogate_train(mdeos_surrogate* s, const double* 
         SCK(cudaGetLastError());
         count_launch(s->h, 1);
       }
-      SCK(cudaMemcpyAsync(tb.h_loss + turn * kSegBatches, dl, (size_t)nb * 4,
+      SCK(cudaMemcpyAsync(io.h_loss + turn * kSegBatches, dl, (size_t)nb * 4,
                           cudaMemcpyDeviceToHost, st));
-      SCK(cudaEventRecord(tb.done[turn], st));
+      SCK(cudaEventRecord(io.seg_done[turn], st));
       held[turn] = nb;
     }
     SCK(collect(turn));  // the older segment first: the losses add up in batch order
@@ -1759,7 +1743,7 @@ extern "C" mdeos_status mdeos_surrogate_predict(mdeos_surrogate* s, const double
     const int B = held[t], off = first[t];
     if (B == 0) return cudaSuccess;
     held[t] = 0;
-    const cudaError_t e = cudaEventSynchronize(s->io.done[t]);
+    const cudaError_t e = cudaEventSynchronize(s->io.io_done[t]);
     if (e != cudaSuccess) return e;
     const size_t ob = (size_t)B * 16;
     const char* h = s->io.h_out[t];
@@ -1787,7 +1771,7 @@ extern "C" mdeos_status mdeos_surrogate_predict(mdeos_surrogate* s, const double
       if (e == cudaSuccess) e = cudaMemcpyAsync(d, s->err, 4, cudaMemcpyDeviceToDevice, st);
       if (e == cudaSuccess)
         e = cudaMemcpyAsync(s->io.h_out[t], d, kIoHead + 2 * ob + yb, cudaMemcpyDeviceToHost, st);
-      if (e == cudaSuccess) e = cudaEventRecord(s->io.done[t], st);
+      if (e == cudaSuccess) e = cudaEventRecord(s->io.io_done[t], st);
       if (e != cudaSuccess) break;
       held[t] = B;
       first[t] = off;
@@ -1932,7 +1916,6 @@ extern "C" mdeos_status mdeos_surrogate_destroy(mdeos_surrogate* s) {
     cudaSetDevice(handle_device(s->h));
     cudaStreamSynchronize(handle_stream(s->h));
   }
-  s->tb.release();
   s->io.release();
   for (void* p : s->allocs) cudaFree(p);
   delete s;
